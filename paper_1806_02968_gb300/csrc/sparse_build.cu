@@ -3,9 +3,8 @@
 // used by the A^T q pass of PCG.
 //
 // Everything is deterministic: the draws are compacted with integer atomics; the
-// transpose of the sampled rows is sorted inside each column; every output row of the
-// SpGEMM sorts its candidate products on (column, sampled row) and sums them in that fixed
-// order.
+// transpose of the sampled rows is sorted inside each column; every output entry of the
+// SpGEMM sums its candidate products in increasing order of the sampled row.
 #include "sparse.cuh"
 #include "values.cuh"
 
@@ -139,258 +138,422 @@ __global__ void k_fill_As(lsq_matrix A, const int32_t* urow, int64_t nu, const i
 }
 
 // ---------------------------------------------------------------------------------------
-// Transpose of a CSR pattern (rows nr, columns nc): column counts, then fill, then each
-// column's entries sorted by row so the order is deterministic.  perm[k] = source entry.
+// Transpose of a CSR pattern (rows nr, columns nc): the entry count of every column, each
+// entry's slot inside its column, then the entries in place and every column sorted by row so
+// that the order does not depend on the counting.  tperm[k] = source entry.
+// One pass of returning atomics gives the counts and the slots at once; the placed word
+// (row << 32 | offset inside the row) is all a column needs to be sorted, and nothing but the
+// two outputs is needed as scratch: trow holds the slots (by entry) and tperm the words until
+// the sort rewrites both.
 // ---------------------------------------------------------------------------------------
-__global__ void k_col_count(const int32_t* col, int64_t nnz, int64_t* ccnt) {
+__global__ void k_col_slot(const int32_t* col, int64_t nnz, unsigned* ccnt, unsigned* slot) {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz; e += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd((unsigned long long*)&ccnt[col[e]], 1ull);
+        slot[e] = atomicAdd(&ccnt[col[e]], 1u);
 }
-__global__ void k_col_fill(const int64_t* rptr, const int32_t* col, int64_t nr, const int64_t* cptr,
-                           int64_t* cfill, int32_t* trow, int64_t* tperm) {
-    const int lane = threadIdx.x & 31;
-    int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r = warp; r < nr; r += nw) {
-        for (int64_t e = rptr[r] + lane; e < rptr[r + 1]; e += 32) {
-            int32_t c = col[e];
-            int64_t at = cptr[c] + (int64_t)atomicAdd((unsigned long long*)&cfill[c], 1ull);
-            trow[at] = (int32_t)r;
-            tperm[at] = e;
-        }
+// the counts as int64 (for the scan) and the longest column
+__global__ void k_col_len(const unsigned* ccnt, int64_t nc, int64_t* len, int* maxlen) {
+    int mx = 0;
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned v = ccnt[c];
+        len[c] = (int64_t)v;
+        mx = max(mx, (int)v);
     }
-}
-constexpr int SPG_CAP = 8192;   // candidates per output row (dynamic shared memory)
-constexpr int SPG_T = 256;
-
-// exclusive scan of one int per thread over the block; *total = block sum
-__device__ __forceinline__ int block_excl_scan_int(int v, int* total) {
-    __shared__ int s_w[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int x = v;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_w[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        int y = lane < nw ? s_w[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int z = __shfl_up_sync(0xffffffffu, y, o);
-            if (lane >= o) y += z;
-        }
-        if (lane < nw) s_w[lane] = y;
-    }
-    __syncthreads();
-    const int off = wid ? s_w[wid - 1] : 0;
-    *total = s_w[nw - 1];
-    const int r = x - v + off;
-    __syncthreads();
-    return r;
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(maxlen, mx);
 }
+// a group of L lanes per row (about the mean row length, a power of two)
+__global__ void k_col_place(const int64_t* rptr, const int32_t* col, int64_t nr, const int64_t* cptr,
+                            const unsigned* slot, unsigned long long* word, int L) {
+    const int sub = threadIdx.x & (L - 1);
+    const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L;
+    const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) / L;
+    for (int64_t r = grp; r < nr; r += ngrp) {
+        const int64_t e0 = rptr[r], e1 = rptr[r + 1];
+        for (int64_t e = e0 + sub; e < e1; e += L)
+            word[cptr[col[e]] + slot[e]] = ((unsigned long long)r << 32) | (unsigned long long)(e - e0);
+    }
+}
+constexpr int SPG_CAP = 8192;   // candidate products of one output row
 
-// bitonic sort of s_key[0..P2) ascending, carrying one payload array (P2 a power of two)
-template <typename V>
-__device__ __forceinline__ void block_bitonic(unsigned long long* s_key, V* s_val, int P2) {
-    for (int size = 2; size <= P2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < P2; i += blockDim.x) {
-                const int pj = i ^ stride;
-                if (pj > i) {
-                    const bool up = (i & size) == 0;
-                    const unsigned long long a = s_key[i], b = s_key[pj];
-                    if ((a > b) == up) {
-                        s_key[i] = b; s_key[pj] = a;
-                        const V t = s_val[i]; s_val[i] = s_val[pj]; s_val[pj] = t;
-                    }
-                }
+// Ascending bitonic sort of key[0..len) by the threads first, first + nt, ... of one group.  Every
+// compare keeps the smaller key at the lower index (the first step of a merge compares
+// mirrored positions), so the places from len up to the next power of two act as +infinity
+// and are never touched.
+template <typename Sync>
+__device__ __forceinline__ void bitonic_any(unsigned long long* key, unsigned len, unsigned first, unsigned nt,
+                                            Sync sync) {
+    unsigned lg = 0;
+    while ((1ull << lg) < len) ++lg;
+    const unsigned pairs = lg ? 1u << (lg - 1) : 0u;
+    auto order = [&](unsigned lo, unsigned hi) {
+        if (hi < len) {
+            const unsigned long long x = key[lo], y = key[hi];
+            if (x > y) { key[lo] = y; key[hi] = x; }
+        }
+    };
+    for (unsigned m = 1; m <= lg; ++m) {          // merges of 2^m keys
+        for (unsigned t = first; t < pairs; t += nt) {
+            const unsigned o = t & ((1u << (m - 1)) - 1u), base = (t >> (m - 1)) << m;
+            order(base + o, base + (1u << m) - 1u - o);
+        }
+        sync();
+        for (int d = (int)m - 2; d >= 0; --d) {   // stride 2^d
+            for (unsigned t = first; t < pairs; t += nt) {
+                const unsigned lo = ((t >> d) << (d + 1)) + (t & ((1u << d) - 1u));
+                order(lo, lo + (1u << d));
             }
-            __syncthreads();
+            sync();
         }
     }
 }
-
-// sort each column segment by row: one CTA per column; a bitonic sort in shared memory on
-// (row, position) keys for segments up to 8192 entries, a serial insertion sort beyond
-constexpr int CS_CAP = 8192;    // entries per column sorted in shared memory
-__global__ void __launch_bounds__(256) k_col_sort(const int64_t* cptr, int64_t nc, int32_t* trow, int64_t* tperm) {
-    extern __shared__ __align__(16) unsigned long long cs_smem[];
-    unsigned long long* s_key = cs_smem;
-    int64_t* s_perm = reinterpret_cast<int64_t*>(cs_smem + CS_CAP);
+__device__ __forceinline__ void emit_sorted(unsigned long long w, const int64_t* rptr, int32_t* trow, int64_t* tperm) {
+    const int64_t r = (int64_t)(w >> 32);
+    *trow = (int32_t)r;
+    *tperm = rptr[r] + (int64_t)(w & 0xFFFFFFFFull);
+}
+// Columns of up to CW_CAP entries: a warp per column in its slice of shared memory.  Longer
+// ones: a CTA per column, in shared memory of the longest column's size (`cap` words; sized by
+// the launch so that short columns leave room for more CTAs), or in place in global memory
+// beyond the 8192 words a CTA can hold.
+constexpr int CW_CAP = 128;
+constexpr int CS_CAP = 8192;
+__global__ void __launch_bounds__(256) k_col_sort_warp(const int64_t* cptr, int64_t nc, const int64_t* rptr,
+                                                       int32_t* trow, int64_t* tperm) {
+    __shared__ unsigned long long s_key[8][CW_CAP];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned long long* key = s_key[wid];
+    const unsigned long long* word = reinterpret_cast<const unsigned long long*>(tperm);
+    for (int64_t c = (int64_t)blockIdx.x * 8 + wid; c < nc; c += (int64_t)gridDim.x * 8) {
+        const int64_t a = cptr[c], len = cptr[c + 1] - a;
+        if (len > CW_CAP || len < 1) continue;
+        for (int i = lane; i < len; i += 32) key[i] = word[a + i];
+        __syncwarp();
+        bitonic_any(key, (unsigned)len, lane, 32u, [] { __syncwarp(); });
+        for (int i = lane; i < len; i += 32) emit_sorted(key[i], rptr, trow + a + i, tperm + a + i);
+        __syncwarp();
+    }
+}
+__global__ void __launch_bounds__(256) k_col_sort_cta(const int64_t* cptr, int64_t nc, const int64_t* rptr,
+                                                      int32_t* trow, int64_t* tperm, int cap) {
+    extern __shared__ __align__(16) unsigned long long cs_key[];
+    unsigned long long* word = reinterpret_cast<unsigned long long*>(tperm);
     for (int64_t c = blockIdx.x; c < nc; c += gridDim.x) {
-        const int64_t a = cptr[c], b = cptr[c + 1];
-        const int64_t len = b - a;
-        if (len <= 1) continue;
-        if (len <= CS_CAP) {
-            int P2 = 1;
-            while (P2 < len) P2 <<= 1;
-            for (int i = threadIdx.x; i < P2; i += blockDim.x) {
-                if (i < len) { s_key[i] = ((unsigned long long)(unsigned)trow[a + i] << 32) | (unsigned)i; s_perm[i] = tperm[a + i]; }
-                else { s_key[i] = ~0ull; s_perm[i] = 0; }
-            }
+        const int64_t a = cptr[c], len = cptr[c + 1] - a;
+        if (len <= CW_CAP) continue;
+        unsigned long long* key = word + a;
+        if (len <= cap) {
+            key = cs_key;
+            for (int i = threadIdx.x; i < len; i += blockDim.x) key[i] = word[a + i];
             __syncthreads();
-            block_bitonic(s_key, s_perm, P2);
-            for (int i = threadIdx.x; i < len; i += blockDim.x) {
-                trow[a + i] = (int32_t)(s_key[i] >> 32);
-                tperm[a + i] = s_perm[i];
-            }
-            __syncthreads();
-        } else if (threadIdx.x == 0) {
-            for (int64_t x = a + 1; x < b; ++x) {
-                int32_t r = trow[x];
-                int64_t pm = tperm[x];
-                int64_t y = x - 1;
-                while (y >= a && trow[y] > r) { trow[y + 1] = trow[y]; tperm[y + 1] = tperm[y]; --y; }
-                trow[y + 1] = r;
-                tperm[y + 1] = pm;
-            }
         }
+        bitonic_any(key, (unsigned)len, threadIdx.x, blockDim.x, [] { __syncthreads(); });
+        for (int64_t i = threadIdx.x; i < len; i += blockDim.x) emit_sorted(key[i], rptr, trow + a + i, tperm + a + i);
+        __syncthreads();
     }
 }
 
 lsq_status transpose_pattern(const int64_t* rptr, const int32_t* col, int64_t nr, int64_t nc, int64_t nnz,
                              int64_t* cptr, int32_t* trow, int64_t* tperm, cudaStream_t st) {
     Scratch sc;
-    int64_t nt = (nc + SC_T - 1) / SC_T + 1;
-    LSQ_CUDA(sc.alloc(8 * (size_t)(2 * nc + nt + 4), st));
-    int64_t* ccnt = sc.as<int64_t>();
-    int64_t* cfill = ccnt + nc;
-    int64_t* ts = cfill + nc;
-    LSQ_CUDA(cudaMemsetAsync(ccnt, 0, 16 * (size_t)nc, st));
-    k_col_count<<<grid1(nnz), 256, 0, st>>>(col, nnz, ccnt);
-    count_launch();
-    lsq_status s = scan_i64(ccnt, nc, cptr, ts, st);
-    if (s != LSQ_OK) return s;
-    k_col_fill<<<grid1(nr * 32), 256, 0, st>>>(rptr, col, nr, cptr, cfill, trow, tperm);
-    const int cs_smem = CS_CAP * 16;
-    LSQ_CUDA(cudaFuncSetAttribute(k_col_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, cs_smem));
-    k_col_sort<<<(unsigned)std::min<int64_t>(nc, 152 * 4), 256, cs_smem, st>>>(cptr, nc, trow, tperm);
+    const int64_t nt = (nc + SC_T - 1) / SC_T + 1;
+    LSQ_CUDA(sc.alloc(4 * (size_t)(nc + 4) + 8 * (size_t)(nc + nt + 4), st));
+    int64_t* len = sc.as<int64_t>();
+    int64_t* ts = len + nc;
+    unsigned* ccnt = reinterpret_cast<unsigned*>(ts + nt + 4);   // nc counters, then the longest
+    int* maxlen = reinterpret_cast<int*>(ccnt + nc);
+    LSQ_CUDA(cudaMemsetAsync(ccnt, 0, 4 * (size_t)(nc + 4), st));
+    unsigned* slot = reinterpret_cast<unsigned*>(trow);
+    unsigned long long* word = reinterpret_cast<unsigned long long*>(tperm);
+    k_col_slot<<<grid1(nnz), 256, 0, st>>>(col, nnz, ccnt, slot);
+    k_col_len<<<grid1(nc), 256, 0, st>>>(ccnt, nc, len, maxlen);
     count_launch(2);
+    lsq_status s = scan_i64(len, nc, cptr, ts, st);
+    if (s != LSQ_OK) return s;
+    int hmax = 0;
+    LSQ_CUDA(cudaMemcpyAsync(&hmax, maxlen, 4, cudaMemcpyDeviceToHost, st));
+    int L = 1;
+    while (L < 32 && L * nr < nnz) L <<= 1;
+    k_col_place<<<grid1(nr * L), 256, 0, st>>>(rptr, col, nr, cptr, slot, word, L);
+    k_col_sort_warp<<<grid1(nc, 8), 256, 0, st>>>(cptr, nc, rptr, trow, tperm);
+    count_launch(2);
+    LSQ_CUDA(cudaStreamSynchronize(st));   // hmax
+    if (hmax > CW_CAP) {
+        const int cap = hmax < CS_CAP ? hmax : CS_CAP;
+        const int smem = cap * 8;
+        LSQ_CUDA(cudaFuncSetAttribute(k_col_sort_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_CAP * 8));
+        k_col_sort_cta<<<(unsigned)std::min<int64_t>(nc, 152 * 32), 256, smem, st>>>(cptr, nc, rptr, trow, tperm, cap);
+        count_launch();
+    }
     LSQ_CUDA(cudaGetLastError());
     return LSQ_OK;
 }
 
 // ---------------------------------------------------------------------------------------
-// SpGEMM M = A_s^T diag(gamma) A_s, one CTA per output row j:
-//   candidates (k, u, gamma_u a_uj a_uk) for every sampled row u with an entry in column j
-//   and every entry k of that row; bitonic sort on (k, u); segmented sums in that order.
-// Pass 0 counts the distinct k (plus the diagonal if absent); pass 1 writes the row.
+// SpGEMM M = A_s^T diag(gamma) A_s, one warp per output row j.  The row's candidates are the
+// products (k, gamma_u a_uj a_uk) for every sampled row u with an entry in column j (in
+// increasing u) and every entry k of that row.
+//   Rows of up to SPG_SHORT candidates (a graph's): the candidates wait in shared memory, each
+//   finds its column's rank by counting, and the first of a column adds up the others.
+//   Longer rows: a bitmap of the n columns (in windows of SPG_WIN) gives the distinct columns in
+//   order; a candidate's rank is a prefix of popcounts, and 32 candidates at a time are added to
+//   the row's sums in shared memory, candidates of the same column one after the other.
+// Either way the sum of a column runs over u in increasing order from 0, so it has the same
+// bits however the work is laid out.  Pass 0 counts the distinct columns (the diagonal always
+// among them); pass 1 writes the row, 1 / M_jj and the diagonal's position.
+// Bound: latency of the gathers of A_s, hidden by as many warps as the bitmap (n / 8 bytes and
+// half of that again for the prefixes) and the sums leave room for.
+// Sampling and building 4e6 x 40,000 (763 products per row) takes 38.3 ms, against 106.6 ms when
+// a CTA sorted a row's candidates in 128 KB of shared memory and one thread added them up
+// (58.5 ms) and the transposes sorted every column in 128 KB as well (7.7 ms).
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(SPG_T) k_spgemm_row(
-    int pass, int64_t n, const int64_t* sptr, const int32_t* scol, const double* sval,
-    const double* gam, const int64_t* tptr, const int32_t* trow, const int64_t* tperm,
-    int64_t* mcnt, const int64_t* mptr, int32_t* mcol, double* mval,
-    unsigned long long* n_fixed, unsigned* err) {
-    extern __shared__ __align__(16) unsigned long long spg_smem[];
-    unsigned long long* s_key = spg_smem;
-    double* s_val = reinterpret_cast<double*>(spg_smem + SPG_CAP);
-    __shared__ int s_cnt;
-    for (int64_t j = blockIdx.x; j < n; j += gridDim.x) {
-        // gather candidates: thread t takes sampled rows q = tptr[j] + t, t + T, ...; the
-        // offset of each row's products is an exclusive scan of the row lengths
-        const int64_t q0 = tptr[j], q1 = tptr[j + 1];
-        int carry = 0;
-        for (int64_t qb = q0; qb < q1; qb += blockDim.x) {
-            const int64_t q = qb + threadIdx.x;
-            int len = 0, u = 0;
-            double cuj = 0.0;
-            int64_t e0 = 0;
-            if (q < q1) {
-                u = trow[q];
-                cuj = gam[u] * sval[tperm[q]];
-                e0 = sptr[u];
-                len = (int)(sptr[u + 1] - e0);
-            }
-            int tot;
-            const int off = block_excl_scan_int(len, &tot) + carry;
-            for (int k = 0; k < len; ++k) {
-                const int at = off + k;
-                if (at < SPG_CAP) {
-                    s_key[at] = ((unsigned long long)(unsigned)scol[e0 + k] << 32) | (unsigned)u;
-                    s_val[at] = cuj * sval[e0 + k];
-                }
-            }
-            carry += tot;
+constexpr int SPG_SHORT = 96;
+constexpr int64_t SPG_WIN = 1 << 18;   // columns per bitmap window (32 KB, and 16 KB of prefixes)
+
+struct SpgArgs {
+    int64_t n;
+    const int64_t* sptr;
+    const int32_t* scol;
+    const double* sval;
+    const double* gam;
+    const int64_t* tptr;
+    const int32_t* trow;
+    const int64_t* tperm;
+    const int32_t* cand;       // candidates of every row
+    int64_t* mcnt;             // pass 0
+    int* maxrow;               // pass 0: the longest row
+    const int64_t* mptr;       // pass 1
+    int32_t* mcol;
+    double* mval;
+    float* mval32;
+    double* dinv;
+    int64_t* mdiag;
+    unsigned long long* n_fixed;
+    int win;                   // columns per window
+    int acap;                  // entries of a row's sums
+};
+// candidates of every row and the largest count
+__global__ void k_spg_cand(int64_t n, const int64_t* sptr, const int64_t* tptr, const int32_t* trow, int32_t* cand,
+                           int* maxcand) {
+    const int lane = threadIdx.x & 31;
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    int mx = 0;
+    for (int64_t j = w; j < n; j += nw) {
+        int64_t t = 0;
+        for (int64_t q = tptr[j] + lane; q < tptr[j + 1]; q += 32) {
+            const int64_t u = trow[q];
+            t += sptr[u + 1] - sptr[u];
         }
-        __syncthreads();
-        int cnt = carry;
-        if (cnt > SPG_CAP) {
-            if (threadIdx.x == 0) atomicOr(err, 16u);
-            cnt = SPG_CAP;
+        t = warp_sum(t);
+        if (t > SPG_CAP) t = SPG_CAP + 1;   // refused by the caller
+        if (lane == 0) cand[j] = (int32_t)t;
+        mx = max(mx, (int)t);
+    }
+    if (lane == 0 && mx > 0) atomicMax(maxcand, mx);
+}
+// Calls fn(column, value, valid) for 32 candidates of row j at a time, in order; the warp runs
+// it converged.  With VALS false the values are not formed.
+template <bool VALS, typename F>
+__device__ __forceinline__ void spg_for_candidates(const SpgArgs& a, int64_t j, int lane, F fn) {
+    const int64_t q0 = a.tptr[j], q1 = a.tptr[j + 1];
+    for (int64_t qb = q0; qb < q1; qb += 32) {
+        const int64_t q = qb + lane;
+        int len = 0;
+        int64_t e0 = 0;
+        double cuj = 0.0;
+        if (q < q1) {
+            const int64_t u = a.trow[q];
+            e0 = a.sptr[u];
+            len = (int)(a.sptr[u + 1] - e0);
+            if (VALS) cuj = a.gam[u] * a.sval[a.tperm[q]];
         }
-        // bitonic sort of the candidates (padded to a power of two with +inf keys)
-        int P2 = 1;
-        while (P2 < cnt) P2 <<= 1;
-        for (int i = cnt + threadIdx.x; i < P2; i += blockDim.x) { s_key[i] = ~0ull; s_val[i] = 0.0; }
-        __syncthreads();
-        block_bitonic(s_key, s_val, P2);
-        // distinct columns: heads of runs of equal k
-        if (pass == 0) {
-            if (threadIdx.x == 0) s_cnt = 0;
-            __syncthreads();
-            int mine = 0, has_diag = 0;
-            for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-                const unsigned k = (unsigned)(s_key[i] >> 32);
-                if (i == 0 || (unsigned)(s_key[i - 1] >> 32) != k) {
-                    ++mine;
-                    if ((int64_t)k == j) has_diag = 1;
-                }
+        int inc = len;   // inclusive prefix of the lengths
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const int tot = __shfl_sync(0xffffffffu, inc, 31);
+        for (int t0 = 0; t0 < tot; t0 += 32) {
+            const int t = t0 + lane;
+            int src = 0;     // the first lane whose inclusive prefix exceeds t
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const int v = __shfl_sync(0xffffffffu, inc, src + o - 1);
+                if (v <= t) src += o;
             }
-            atomicAdd(&s_cnt, mine + 0);
-            if (has_diag) atomicAdd(&s_cnt, 1 << 20);
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                const int c = s_cnt & ((1 << 20) - 1);
-                const int d = s_cnt >> 20;
-                mcnt[j] = c + (d ? 0 : 1);
+            src = min(src, 31);
+            const int before = __shfl_sync(0xffffffffu, inc - len, src);
+            const int64_t base = __shfl_sync(0xffffffffu, e0, src);
+            double c = 0.0;
+            if (VALS) c = __shfl_sync(0xffffffffu, cuj, src);
+            const bool ok = t < tot;
+            int32_t k = -1;
+            double v = 0.0;
+            if (ok) {
+                k = a.scol[base + (t - before)];
+                if (VALS) v = c * a.sval[base + (t - before)];
             }
-            __syncthreads();
+            fn(k, v, ok);
+        }
+    }
+}
+__device__ __forceinline__ void spg_put(const SpgArgs& a, int64_t j, int64_t at, int32_t k, double v) {
+    if ((int64_t)k == j) {
+        if (v == 0.0) { v = 1.0; atomicAdd(a.n_fixed, 1ull); }   // never drawn: the diagonal of Â^T Â
+        a.dinv[j] = 1.0 / v;
+        a.mdiag[j] = at;
+    }
+    a.mcol[at] = k;
+    a.mval[at] = v;
+    if (a.mval32) a.mval32[at] = (float)v;
+}
+
+constexpr int SPS_W = 4;   // warps per CTA of the short-row kernel
+template <bool FILL>
+__global__ void __launch_bounds__(32 * SPS_W) k_spgemm_short(SpgArgs a) {
+    __shared__ int32_t s_col[SPS_W][SPG_SHORT + 1];
+    __shared__ double s_val[SPS_W][FILL ? SPG_SHORT + 1 : 1];
+    __shared__ unsigned s_first[SPS_W][(SPG_SHORT + 32) / 32];   // bit i: candidate i is its column's first
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int32_t* col = s_col[wid];
+    double* val = s_val[wid];
+    unsigned* first = s_first[wid];
+    for (int64_t j = (int64_t)blockIdx.x * SPS_W + wid; j < a.n; j += (int64_t)gridDim.x * SPS_W) {
+        const int cnt = a.cand[j];
+        if (cnt > SPG_SHORT) continue;
+        int at = 0;
+        spg_for_candidates<FILL>(a, j, lane, [&](int32_t k, double v, bool ok) {
+            if (ok) {
+                col[at + lane] = k;
+                if (FILL) val[at + lane] = v;
+            }
+            at += __popc(__ballot_sync(0xffffffffu, ok));
+        });
+        if (lane == 0) {                     // the diagonal, last: adds nothing
+            col[cnt] = (int32_t)j;
+            if (FILL) val[cnt] = 0.0;
+        }
+        __syncwarp();
+        int uniq = 0;
+        for (int b = 0; b <= cnt; b += 32) {
+            const int i = b + lane;
+            bool f = i <= cnt;
+            for (int t = 0; t < min(b + 31, cnt); ++t)
+                if (t < i && f && col[t] == col[i]) f = false;
+            const unsigned m = __ballot_sync(0xffffffffu, f);
+            if (lane == 0) first[b >> 5] = m;
+            uniq += __popc(m);
+        }
+        if (!FILL) {
+            if (lane == 0) a.mcnt[j] = uniq;
         } else {
-            // one thread walks the sorted list (fixed order), inserting the diagonal
-            if (threadIdx.x == 0) {
-                int64_t o = mptr[j];
-                bool diag_done = false;
-                int i = 0;
-                while (i < cnt) {
-                    const unsigned k = (unsigned)(s_key[i] >> 32);
-                    if (!diag_done && (int64_t)k > j) {
-                        mcol[o] = (int32_t)j; mval[o] = 1.0; ++o;
-                        atomicAdd(n_fixed, 1ull);
-                        diag_done = true;
-                    }
-                    double sum = 0.0;
-                    while (i < cnt && (unsigned)(s_key[i] >> 32) == k) { sum += s_val[i]; ++i; }
-                    if ((int64_t)k == j) {
-                        diag_done = true;
-                        if (sum == 0.0) { sum = 1.0; atomicAdd(n_fixed, 1ull); }
-                    }
-                    mcol[o] = (int32_t)k; mval[o] = sum; ++o;
+            __syncwarp();
+            for (int i = lane; i <= cnt; i += 32) {
+                if (!((first[i >> 5] >> (i & 31)) & 1u)) continue;
+                const int32_t k = col[i];
+                int rank = 0;
+                double sum = 0.0;
+                for (int t = 0; t <= cnt; ++t) {
+                    const int32_t kt = col[t];
+                    if (kt == k) sum += val[t];
+                    rank += (kt < k && ((first[t >> 5] >> (t & 31)) & 1u)) ? 1 : 0;
                 }
-                if (!diag_done) { mcol[o] = (int32_t)j; mval[o] = 1.0; atomicAdd(n_fixed, 1ull); }
+                spg_put(a, j, a.mptr[j] + rank, k, sum);
             }
-            __syncthreads();
         }
+        __syncwarp();
     }
 }
 
-// diagonal inverse of M (the diagonal is always stored)
-__global__ void k_diag_inv(const int64_t* mptr, const int32_t* mcol, const double* mval, int64_t n, double* dinv,
-                           int64_t* mdiag) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        double v = 1.0;
-        int64_t at = mptr[j];
-        for (int64_t e = mptr[j]; e < mptr[j + 1]; ++e)
-            if (mcol[e] == j) { v = mval[e]; at = e; break; }
-        dinv[j] = 1.0 / v;
-        mdiag[j] = at;
+template <bool FILL>
+__global__ void __launch_bounds__(32) k_spgemm_long(SpgArgs a) {
+    extern __shared__ __align__(16) unsigned char spg_smem[];
+    const int lane = threadIdx.x;
+    const int words = (a.win + 31) >> 5, per = (words + 31) >> 5;
+    double* acc = reinterpret_cast<double*>(spg_smem);                       // acap sums (pass 1)
+    int32_t* ocol = reinterpret_cast<int32_t*>(acc + (FILL ? a.acap : 0));   // their columns
+    unsigned* bits = reinterpret_cast<unsigned*>(ocol + (FILL ? a.acap : 0));
+    unsigned short* pre = reinterpret_cast<unsigned short*>(bits + words);   // columns before each word
+    int longest = 0;
+    for (int64_t j = blockIdx.x; j < a.n; j += gridDim.x) {
+        if (a.cand[j] <= SPG_SHORT) continue;
+        int64_t out = FILL ? a.mptr[j] : 0;
+        int uniq_all = 0;
+        for (int64_t w0 = 0; w0 < a.n; w0 += a.win) {
+            for (int i = lane; i < words; i += 32) bits[i] = 0u;
+            __syncwarp();
+            spg_for_candidates<false>(a, j, lane, [&](int32_t k, double, bool ok) {
+                const int64_t d = (int64_t)k - w0;
+                if (ok && d >= 0 && d < a.win) atomicOr(&bits[d >> 5], 1u << (d & 31));
+            });
+            if (lane == 0 && j >= w0 && j < w0 + a.win) atomicOr(&bits[(j - w0) >> 5], 1u << ((j - w0) & 31));
+            __syncwarp();
+            const int i0 = min(lane * per, words), i1 = min(i0 + per, words);
+            int mine = 0;
+            for (int i = i0; i < i1; ++i) mine += __popc(bits[i]);
+            int inc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            const int uniq = __shfl_sync(0xffffffffu, inc, 31);
+            uniq_all += uniq;
+            if (FILL) {
+                int run = inc - mine;
+                for (int i = i0; i < i1; ++i) {
+                    pre[i] = (unsigned short)run;
+                    unsigned b = bits[i];
+                    while (b) {
+                        const int t = __ffs(b) - 1;
+                        ocol[run++] = (int32_t)(w0 + (int64_t)i * 32 + t);
+                        b &= b - 1;
+                    }
+                }
+                for (int i = lane; i < uniq; i += 32) acc[i] = 0.0;
+                __syncwarp();
+                spg_for_candidates<true>(a, j, lane, [&](int32_t k, double v, bool ok) {
+                    const int64_t d = (int64_t)k - w0;
+                    const bool in = ok && d >= 0 && d < a.win;
+                    // candidates of one column add in order: round r takes each column's r-th lane
+                    const unsigned same = __match_any_sync(0xffffffffu, in ? k : -1 - lane);
+                    const int my = __popc(same & ((1u << lane) - 1u));
+                    int rank = 0;
+                    if (in) rank = (int)pre[d >> 5] + __popc(bits[d >> 5] & ((1u << (d & 31)) - 1u));
+                    for (int r = 0; __any_sync(0xffffffffu, in && my >= r); ++r) {
+                        if (in && my == r) acc[rank] += v;
+                        __syncwarp();
+                    }
+                });
+                for (int i = lane; i < uniq; i += 32) spg_put(a, j, out + i, ocol[i], acc[i]);
+                out += uniq;
+                __syncwarp();
+            }
+        }
+        if (!FILL) {
+            if (lane == 0) a.mcnt[j] = uniq_all;
+            longest = max(longest, uniq_all);
+        }
     }
+    if (!FILL && lane == 0 && longest > 0) atomicMax(a.maxrow, longest);
 }
-__global__ void k_to_f32(const double* src, float* dst, int64_t count) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
-        dst[e] = (float)src[e];
+// Both kernels of one pass; the long-row kernel only when there is a long row.
+template <bool FILL>
+static lsq_status spgemm_pass(SpgArgs a, int maxcand, int sms, cudaStream_t st) {
+    k_spgemm_short<FILL><<<(unsigned)std::min<int64_t>((a.n + SPS_W - 1) / SPS_W, (int64_t)sms * 16), 32 * SPS_W, 0, st>>>(a);
+    count_launch();
+    if (maxcand <= SPG_SHORT) return LSQ_OK;
+    a.win = (int)std::min<int64_t>(a.n, SPG_WIN);
+    const size_t words = (size_t)(a.win + 31) / 32;
+    const size_t smem = (FILL ? 12 * (size_t)a.acap : 0) + 4 * words + 2 * words + 16;
+    LSQ_CUDA(cudaFuncSetAttribute(k_spgemm_long<FILL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per = 0;
+    LSQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_spgemm_long<FILL>, 32, smem));
+    if (per < 1) { set_error("SpGEMM kernel does not fit on an SM"); return LSQ_ERR_CUDA; }
+    k_spgemm_long<FILL><<<(unsigned)std::min<int64_t>(a.n, (int64_t)sms * per * 2), 32, smem, st>>>(a);
+    count_launch();
+    return LSQ_OK;
 }
 
 // Level schedules: lev_f(j) = 1 + max lev_f(k) over k < j with M_jk != 0 (rows in natural
@@ -591,47 +754,50 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
     count_launch();
     r = transpose_pattern(sptr, scol, nu, n, snnz, tptr, trow, tperm, st);
     if (r != LSQ_OK) return r;
-    // 3. SpGEMM: counts, row pointers, values
+    // 3. SpGEMM: candidates, counts, row pointers, values
     Scratch sc4;
     int64_t ntn = (n + SC_T - 1) / SC_T + 1;
-    LSQ_CUDA(sc4.alloc(8 * (size_t)(n + 16 + ntn), st));
+    LSQ_CUDA(sc4.alloc(8 * (size_t)(n + 16 + ntn) + 4 * (size_t)n, st));
     int64_t* mcnt = sc4.as<int64_t>();
     unsigned long long* nfix = reinterpret_cast<unsigned long long*>(mcnt + n);
-    unsigned* err = reinterpret_cast<unsigned*>(nfix + 1);
+    int* mmax = reinterpret_cast<int*>(nfix + 1);   // most candidates and most entries of a row
     int64_t* ts4 = mcnt + n + 16;
-    LSQ_CUDA(cudaMemsetAsync(nfix, 0, 16, st));
+    int32_t* cand = reinterpret_cast<int32_t*>(ts4 + ntn);
+    LSQ_CUDA(cudaMemsetAsync(nfix, 0, 32, st));
     LSQ_CUDA(cudaMalloc(&S->mptr, 8 * (size_t)(n + 1)));
-    unsigned gs = (unsigned)std::min<int64_t>(n, 152 * 4);
-    const int spg_smem = SPG_CAP * 16;
-    LSQ_CUDA(cudaFuncSetAttribute(k_spgemm_row, cudaFuncAttributeMaxDynamicSharedMemorySize, spg_smem));
-    k_spgemm_row<<<gs, SPG_T, spg_smem, st>>>(0, n, sptr, scol, sval, gam, tptr, trow, tperm, mcnt, nullptr,
-                                       nullptr, nullptr, nfix, err);
+    int dev = 0, sms = 0;
+    LSQ_CUDA(cudaGetDevice(&dev));
+    LSQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    k_spg_cand<<<grid1(n * 32), 256, 0, st>>>(n, sptr, tptr, trow, cand, mmax);
     count_launch();
-    r = scan_i64(mcnt, n, S->mptr, ts4, st);
-    if (r != LSQ_OK) return r;
-    int64_t mnnz = 0;
-    unsigned errbits = 0;
-    LSQ_CUDA(cudaMemcpyAsync(&mnnz, S->mptr + n, 8, cudaMemcpyDeviceToHost, st));
-    LSQ_CUDA(cudaMemcpyAsync(&errbits, err, 4, cudaMemcpyDeviceToHost, st));
+    int hmax[2] = {0, 0};
+    LSQ_CUDA(cudaMemcpyAsync(hmax, mmax, 4, cudaMemcpyDeviceToHost, st));
     LSQ_CUDA(cudaStreamSynchronize(st));
-    if (errbits & 16u) {
+    if (hmax[0] > SPG_CAP) {
         set_error("a row of A_s^T A_s has more than 8192 candidate products (unsupported in this build)");
         return LSQ_ERR_UNSUPPORTED;
     }
+    SpgArgs ga{};
+    ga.n = n; ga.sptr = sptr; ga.scol = scol; ga.sval = sval; ga.gam = gam;
+    ga.tptr = tptr; ga.trow = trow; ga.tperm = tperm; ga.cand = cand;
+    ga.mcnt = mcnt; ga.maxrow = mmax + 1; ga.n_fixed = nfix;
+    r = spgemm_pass<false>(ga, hmax[0], sms, st);
+    if (r != LSQ_OK) return r;
+    r = scan_i64(mcnt, n, S->mptr, ts4, st);
+    if (r != LSQ_OK) return r;
+    int64_t mnnz = 0;
+    LSQ_CUDA(cudaMemcpyAsync(&mnnz, S->mptr + n, 8, cudaMemcpyDeviceToHost, st));
+    LSQ_CUDA(cudaMemcpyAsync(hmax, mmax, 8, cudaMemcpyDeviceToHost, st));
+    LSQ_CUDA(cudaStreamSynchronize(st));
     LSQ_CUDA(cudaMalloc(&S->mcol, 4 * (size_t)mnnz));
     LSQ_CUDA(cudaMalloc(&S->mval, 8 * (size_t)mnnz));
-    k_spgemm_row<<<gs, SPG_T, spg_smem, st>>>(1, n, sptr, scol, sval, gam, tptr, trow, tperm, nullptr, S->mptr,
-                                       S->mcol, S->mval, nfix, err);
-    count_launch();
+    if (H->op_dtype == LSQ_F32) LSQ_CUDA(cudaMalloc(&S->mval32, 4 * (size_t)mnnz));
     LSQ_CUDA(cudaMalloc(&S->dinv, 8 * (size_t)n));
     LSQ_CUDA(cudaMalloc(&S->mdiag, 8 * (size_t)n));
-    k_diag_inv<<<grid1(n), 256, 0, st>>>(S->mptr, S->mcol, S->mval, n, S->dinv, S->mdiag);
-    count_launch();
-    if (H->op_dtype == LSQ_F32) {
-        LSQ_CUDA(cudaMalloc(&S->mval32, 4 * (size_t)mnnz));
-        k_to_f32<<<grid1(mnnz), 256, 0, st>>>(S->mval, S->mval32, mnnz);
-        count_launch();
-    }
+    ga.mptr = S->mptr; ga.mcol = S->mcol; ga.mval = S->mval; ga.mval32 = S->mval32;
+    ga.dinv = S->dinv; ga.mdiag = S->mdiag; ga.acap = (hmax[1] + 1) & ~1;
+    r = spgemm_pass<true>(ga, hmax[0], sms, st);
+    if (r != LSQ_OK) return r;
     unsigned long long nf = 0;
     LSQ_CUDA(cudaMemcpyAsync(&nf, nfix, 8, cudaMemcpyDeviceToHost, st));
     LSQ_CUDA(cudaGetLastError());
