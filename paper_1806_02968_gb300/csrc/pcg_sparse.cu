@@ -13,7 +13,7 @@
 // waits (bounded) for the values of its own dependencies, in one CTA the levels meet at
 // block barriers.  A device flag ends the remaining kernels of a batch once PCG has
 // converged.
-#include "sparse.cuh"
+#include "sweep_blocked.cuh"
 #include "values.cuh"
 #include "dfloat.cuh"
 
@@ -22,12 +22,6 @@
 #include <algorithm>
 
 namespace lsq {
-
-struct SpState {
-    double rho, hn, gstart, rec;
-    int32_t iters, done, status, napply;   // napply: preconditioner applications so far
-    unsigned err, pad, r0, r1;
-};
 
 struct SpArgs {
     int64_t m, n;
@@ -55,6 +49,8 @@ struct SpArgs {
     int64_t one_f, one_b;       // level count when that direction runs in one CTA, else 0
     int64_t cl_f, cl_b;         // level count when that direction runs in one cluster, else 0
     int64_t nlev_f, nlev_b;     // level counts of the two schedules
+    const void* inv;            // inverted diagonal blocks when the sweeps run by blocks, else NULL
+    const double* mval64;
     int cl_lg;                  // log2 of that cluster's size
     int lpr, lpc;               // lanes per row of A, lanes per column of A (powers of two <= 32)
     int sweeps;
@@ -855,6 +851,17 @@ template <typename MT, bool FWD>
 static lsq_status launch_sweep(const SpArgs& a, const double* r, const double* eold, double* enew,
                                double* out64, int identity, int check, int nparts, int idx, cudaStream_t st) {
     static std::atomic<int> grid_cache{0};   // one per kernel instance; callers may be threads
+    if (a.inv) {   // deep level structure: by blocks of rows
+        k_fill_empty<<<(unsigned)std::min<int64_t>((a.n + SP_T - 1) / SP_T, 152 * 8), SP_T, 0, st>>>(enew, a.n);
+        count_launch();
+        SbArgs b{};
+        b.n = a.n; b.K = 1; b.mptr = a.mptr; b.mcol = a.mcol; b.mval = a.mval; b.mdiag = a.mdiag;
+        b.mval64 = a.mval64; b.inv = a.inv; b.done = &a.S->done; b.err = &a.S->err; b.max_polls = a.max_polls;
+        b.r = r; b.e_old = eold; b.e_new = enew; b.out64 = out64; b.identity = identity;
+        b.S = check ? a.S : nullptr; b.part = a.part + a.rblk; b.nparts = nparts;
+        b.tol = a.tol; b.inner_tol = a.inner_tol; b.maxit = a.maxit;
+        return sb_launch(b, FWD, sizeof(MT) == 4, sizeof(MT) == 4, st);
+    }
     auto kern = k_sp_sweep_vf<MT, FWD>;
     int grid = grid_cache.load(std::memory_order_relaxed);
     if (grid == 0) {
@@ -890,7 +897,8 @@ static lsq_status launch_sweep(const SpArgs& a, const double* r, const double* e
     return LSQ_OK;
 }
 
-// The sweep form of each direction.  By shape (form 0): one CTA when a level holds fewer than
+// The sweep form of each direction.  By shape (form 0): by blocks of rows where the handle
+// holds the inverted blocks (sb_build_inverse); otherwise one CTA when a level holds fewer than
 // 2048 dependency entries on average: block barriers between levels are then cheaper than a
 // grid of warps polling for the values they depend on, and one SM's loads still keep up with
 // a level's gathers (at ~10,000 entries per level one SM is twice slower than the grid);
@@ -902,6 +910,8 @@ static void choose_sweep_form(SpArgs& a, const SparseHandle* SH, int64_t n) {
     const double dep = 0.5 * (double)(SH->nnz_M - n);   // dependency entries per direction
     const int form = g_sweep_form.load(std::memory_order_relaxed);
     const bool fits = 8 * ((n + (1 << SC_LG) - 1) >> SC_LG) <= SC_SMEM;
+    a.inv = form == 0 && sb_use(SH) ? SH->inv : nullptr;
+    a.mval64 = SH->mval;
     a.cl_lg = SC_LG;
     auto pick = [&](int64_t nlev, int64_t& one, int64_t& clv) {
         one = clv = 0;

@@ -22,6 +22,7 @@
 // so results do not depend on timing.
 #include "bk_device.cuh"
 #include "sparse_persist.cuh"
+#include "sweep_blocked.cuh"
 
 #include <cooperative_groups.h>
 
@@ -465,6 +466,10 @@ static lsq_status bk_solve_impl(const lsq_matrix* A, const lsq_precond* P, const
     // last sweep also writing z in FP64 (a dependent FP64 step costs ~64 cycles on GB300);
     // the cluster and persistent forms keep FP64 sums
     const bool pairs = m32 && smode == 2 && !cl_f && !cl_b;
+    // by shape, deep level schedules run by blocks of rows (the same arithmetic: pairs where
+    // the CTA-per-row form uses them, FP64 sums otherwise).  Short rows (graphs) stay with the
+    // lane-per-column form, whose bits the persistent kernel shares.
+    const bool blocked = form == 0 && smode > 0 && sb_use(SH);
     const void* kf = pairs ? bk_sweep_kernel<float, true, true>(smode, K)
                            : (m32 ? bk_sweep_kernel<float, true>(smode, K) : bk_sweep_kernel<double, true>(smode, K));
     const void* kb = pairs ? bk_sweep_kernel<float, false, true>(smode, K)
@@ -473,7 +478,15 @@ static lsq_status bk_solve_impl(const lsq_matrix* A, const lsq_precond* P, const
     auto sweep = [&](bool fwd, const double* r, const double* eold, double* enew, double* out64, int identity,
                      int idx) {
         lsq_status q;
-        if (fwd && cl_f) q = bk_launch_sweep_cl(cf, a, r, eold, enew, identity, SH->loff_f, SH->nlev_f, st);
+        if (blocked) {
+            k_bk_fill_empty<<<(unsigned)std::min<int64_t>((nK + BK_T - 1) / BK_T, 152 * 8), BK_T, 0, st>>>(enew, nK);
+            count_launch();
+            SbArgs b{};
+            b.n = n; b.K = K; b.mptr = a.mptr; b.mcol = a.mcol; b.mval = a.mval; b.mdiag = a.mdiag;
+            b.mval64 = SH->mval; b.inv = SH->inv; b.done = &S->done; b.err = &S->err; b.max_polls = a.max_polls;
+            b.r = r; b.e_old = eold; b.e_new = enew; b.out64 = out64; b.identity = identity;
+            q = sb_launch(b, fwd, m32, pairs, st);
+        } else if (fwd && cl_f) q = bk_launch_sweep_cl(cf, a, r, eold, enew, identity, SH->loff_f, SH->nlev_f, st);
         else if (!fwd && cl_b) q = bk_launch_sweep_cl(cb, a, r, eold, enew, identity, SH->loff_b, SH->nlev_b, st);
         else q = bk_launch_sweep(fwd ? kf : kb, a, r, eold, enew, out64, identity, idx,
                                  fwd ? SH->nlev_f : SH->nlev_b, smode == 2 ? 1 : BK_T / 32, st);

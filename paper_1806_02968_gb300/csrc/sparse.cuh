@@ -19,6 +19,9 @@ struct SparseHandle {
     int64_t nlev_f = 0, nlev_b = 0;
     int64_t* loff_f = nullptr;    // first schedule slot of every level (nlev + 1 entries)
     int64_t* loff_b = nullptr;
+    // inverses of the 128-row lower diagonal blocks (sweep_blocked.cu), where the schedule is
+    // deep; NULL otherwise
+    void* inv = nullptr;
     // transposed pattern of A: column pointers, row indices, source entry of each
     int64_t* atptr = nullptr;
     int32_t* atrow = nullptr;

@@ -1,0 +1,564 @@
+// Gauss-Seidel sweeps of Alg. 3 by blocks of B consecutive rows, for deep level schedules.
+//
+// A forward sweep solves (D + L) x = s for s = r - U e_old in the natural row order.  With the
+// rows in blocks, block k needs x of the blocks before it; inside the block the triangular
+// system is solved by one product with the block's inverse, computed once per handle:
+//     x_k = (D + L)_kk^{-1} (s_k - sum_{i < k} L_ki x_i).
+// The chain of a sweep is then n / B blocks instead of the level schedule's depth.  A CTA owns
+// blocks k, k + G, ...; it follows the blocks before its own one after the other: it waits for
+// their B values (the values are their own completion flags, as in the row forms: a slot holds
+// SB_EMPTY until it is written), puts them in shared memory, and every thread adds up the
+// entries of its row that fall in them (rows are sorted, so a thread's cursor only moves on).
+// Behind the last of them only the reduction of ES partial sums and the B x B product stand
+// between two blocks.  A block that starts late finds the first blocks finished and takes four
+// at a time until it has caught up.
+//
+// Bound: the chain's latency: the values' way to another SM, the last entries, the reduction of
+// ES sums and the product.  The inverse sits in registers (each thread holds the part of its row
+// it multiplies), loaded while the CTA waits.
+// Measured per sweep: 40,000 rows of 380 dependencies in 1583 levels, one column, double-float:
+// 0.75 ms (2.4 us per block of 128 rows), against 1.75 ms forward and 3.5 ms backward by rows;
+// 10,000 rows of 350 dependencies in 1227 levels, 16 columns: 0.48 ms (3.1 us per block of 64),
+// against 5.3 and 6.1 ms.
+// Columns are independent chains, so a block of right-hand sides is split over CTAs by KC
+// columns.
+//
+// Waits are bounded as everywhere: one that gives up sets the error word, which ends the others.
+// Every CTA is resident (cooperative launch) and takes its blocks in increasing order, so every
+// wait ends.
+#include "sweep_blocked.cuh"
+#include "dfloat.cuh"
+
+#include <algorithm>
+#include <mutex>
+#include <unordered_map>
+
+namespace lsq {
+
+constexpr unsigned long long SB_EMPTY = 0xFFF7DEADBEEFCAFEull;   // the row forms' empty marker
+constexpr int SB_T = 512;
+constexpr int SB_SPAN = 4;          // blocks taken at once while catching up
+constexpr int SB_AHEAD = 4;         // entries of its row a thread holds ahead
+
+__device__ __forceinline__ unsigned long long sb_ldv(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sb_stv(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Arithmetic of a sweep: double-float pairs for FP32 M, or FP64 sums for either type of M.
+struct SbPair {
+    typedef f2 V;
+    static __device__ __forceinline__ V zero() { return f2{0.f, 0.f}; }
+    static __device__ __forceinline__ V from_bits(unsigned long long u) {
+        return f2{__uint_as_float((unsigned)u), __uint_as_float((unsigned)(u >> 32))};
+    }
+    static __device__ __forceinline__ unsigned long long to_bits(V v) {
+        return (unsigned long long)__float_as_uint(v.hi) | ((unsigned long long)__float_as_uint(v.lo) << 32);
+    }
+    static __device__ __forceinline__ V from_double(double x) { return df_from_double(x); }
+    static __device__ __forceinline__ double to_double(V v) { return df_to_double(v); }
+    // acc += m x, cascaded (the errors gather in the low word)
+    static __device__ __forceinline__ void mad(V& acc, float m, V x) {
+        float p, pe, s, e;
+        two_prod(m, x.hi, p, pe);
+        pe = fmaf(m, x.lo, pe);
+        two_sum(acc.hi, p, s, e);
+        acc.hi = s;
+        acc.lo += e + pe;
+    }
+    static __device__ __forceinline__ void madv(V& acc, V m, V x) { df_fma_cascade(acc, m, x); }
+    static __device__ __forceinline__ void norm(V& v) { v = df_norm(v); }
+    static __device__ __forceinline__ void add(V& a, V b) { df_add(a, b); }
+    static __device__ __forceinline__ V xorv(V v, int o) { return df_shfl_xor(v, o); }
+    static __device__ __forceinline__ V neg(V v) { return f2{-v.hi, -v.lo}; }
+};
+struct SbDouble {
+    typedef double V;
+    static __device__ __forceinline__ V zero() { return 0.0; }
+    static __device__ __forceinline__ V from_bits(unsigned long long u) { return __longlong_as_double((long long)u); }
+    static __device__ __forceinline__ unsigned long long to_bits(V v) { return (unsigned long long)__double_as_longlong(v); }
+    static __device__ __forceinline__ V from_double(double x) { return x; }
+    static __device__ __forceinline__ double to_double(V v) { return v; }
+    static __device__ __forceinline__ void mad(V& acc, double m, V x) { acc = fma(m, x, acc); }
+    static __device__ __forceinline__ void madv(V& acc, V m, V x) { acc = fma(m, x, acc); }
+    static __device__ __forceinline__ void norm(V&) {}
+    static __device__ __forceinline__ void add(V& a, V b) { a += b; }
+    static __device__ __forceinline__ V xorv(V v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+    static __device__ __forceinline__ V neg(V v) { return -v; }
+};
+
+// MT: type of M's values; AR: arithmetic; INV: element of the inverse (f2 pairs for float M,
+// double otherwise); B rows per block, KC columns per CTA.  Thread (row, h, c) of the 512 owns
+// entries h, h + ES, ... of its row for column c.
+template <typename MT, typename AR, bool FWD, int B, int KC>
+__global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
+    typedef typename AR::V V;
+    constexpr int ES = SB_T / (B * KC);
+    constexpr int PER = B / ES;          // inverse entries per thread
+    static_assert(ES >= 1 && ES * KC <= 32 && SB_ROWS % B == 0, "thread layout");
+    __shared__ V s_x[2][SB_SPAN * B * KC];
+    __shared__ V s_s[B * KC];
+    __shared__ double s_red[SB_T / 32];
+    __shared__ int s_stop;
+    if (*a.done) return;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (a.S) {   // the convergence check of the one-column solve, the same decision in every CTA
+        double t = 0.0;
+        for (int i = tid; i < a.nparts; i += SB_T) t += a.part[i];
+        t = warp_sum(t);
+        if (lane == 0) s_red[tid >> 5] = t;
+        __syncthreads();
+        if (tid == 0) {
+            double gg = 0.0;
+            for (int w = 0; w < SB_T / 32; ++w) gg += s_red[w];
+            const double gn = sqrt(gg);
+            s_stop = (gn <= a.tol * a.S->hn || gn <= a.inner_tol * a.S->gstart || a.S->iters >= a.maxit) ? 1 : 0;
+            if (blockIdx.x == 0) a.S->rec = gn / a.S->hn;
+        }
+        __syncthreads();
+        if (s_stop) {
+            if (blockIdx.x == 0 && tid == 0) a.S->done = 1;
+            return;
+        }
+    }
+    const MT* __restrict__ mv = reinterpret_cast<const MT*>(a.mval);
+    const int32_t* __restrict__ mc = a.mcol;
+    unsigned long long* xnew = reinterpret_cast<unsigned long long*>(a.e_new);
+    const unsigned long long* xold = reinterpret_cast<const unsigned long long*>(a.e_old);
+    const int c = tid % KC, h = (tid / KC) % ES, row = tid / (KC * ES);
+    const int nblk = (int)((a.n + B - 1) / B);
+    const int ngrp = (a.K + KC - 1) / KC;
+    const int64_t ntask = (int64_t)nblk * ngrp;
+    for (int64_t task = blockIdx.x; task < ntask; task += gridDim.x) {
+        const int kk = (int)(task / ngrp), cg = (int)(task % ngrp);
+        const int kb = FWD ? kk : nblk - 1 - kk;          // this block
+        const int64_t j = (int64_t)kb * B + row;
+        const int col = cg * KC + c;
+        const bool live = j < a.n && col < a.K;
+        // the part of the inverse this thread multiplies: entries h, h + ES, ... of its row
+        // (backward: M is symmetric, so the upper block's inverse is the transpose)
+        V inv[PER];
+        {
+            const int sub = (kb * B) % SB_ROWS;           // place inside the stored block
+            const int64_t at = (int64_t)((int64_t)kb * B / SB_ROWS) * SB_ROWS * SB_ROWS;
+            const int ri = sub + row;
+#pragma unroll
+            for (int t = 0; t < PER; ++t) {
+                const int ci = sub + h + ES * t;
+                const int64_t e = at + (FWD ? (int64_t)ri * SB_ROWS + ci : (int64_t)ci * SB_ROWS + ri);
+                if constexpr (sizeof(MT) == 4) {
+                    const f2 p = reinterpret_cast<const f2*>(a.inv)[e];
+                    if constexpr (std::is_same<AR, SbPair>::value) inv[t] = p;
+                    else inv[t] = df_to_double(p);
+                } else {
+                    inv[t] = reinterpret_cast<const double*>(a.inv)[e];
+                }
+            }
+        }
+        // base term, the other side's terms (previous sweep: complete), and the cursor
+        V acc = AR::zero(), base = AR::zero();
+        int64_t e = 0, e_end = 0;
+        if (live) {
+            const int64_t p0 = a.mptr[j], pd = a.mdiag[j], p1 = a.mptr[j + 1];
+            if (a.identity) {      // r - L e_old = D e_old after one forward sweep from zero
+                if (h == 0) AR::madv(base, AR::from_double(a.mval64[pd]), AR::from_bits(xold[j * a.K + col]));
+            } else {
+                if (h == 0) base = AR::from_double(a.r[j * a.K + col]);
+                if (a.e_old) {
+                    const int64_t o0 = FWD ? pd + 1 : p0, o1 = FWD ? p1 : pd;
+                    for (int64_t q = o0 + h; q < o1; q += ES)
+                        AR::mad(acc, mv[q], AR::from_bits(xold[(int64_t)mc[q] * a.K + col]));
+                }
+            }
+            if (FWD) { e = p0 + h; e_end = pd; }
+            else { e = p1 - 1 - h; e_end = pd; }
+        }
+        // the cursor holds SB_AHEAD entries: M streams from L2 or HBM, and a load that is waited
+        // for inside the walk stands in the chain; a column past every block ends the walk
+        constexpr int PAST = FWD ? 0x7fffffff : -1;
+        int cq[SB_AHEAD];
+        MT vq[SB_AHEAD];
+        auto fetch = [&](int& cc, MT& vv) {
+            const bool in = FWD ? e < e_end : e > e_end;
+            cc = PAST;
+            vv = MT(0);
+            if (in) { cc = mc[e]; vv = mv[e]; e += FWD ? ES : -ES; }
+        };
+#pragma unroll
+        for (int q = 0; q < SB_AHEAD; ++q) { cq[q] = PAST; vq[q] = MT(0); }
+        if (live) {
+#pragma unroll
+            for (int q = 0; q < SB_AHEAD; ++q) fetch(cq[q], vq[q]);
+        }
+        // slot of this thread's value in block i of the chain (i-th block done)
+        const int lrow = tid / KC;
+        auto slot = [&](int i) -> const unsigned long long* {
+            const int64_t jj = (int64_t)(FWD ? i : nblk - 1 - i) * B + lrow;
+            return (tid < B * KC && jj < a.n && col < a.K) ? xnew + jj * a.K + cg * KC + tid % KC : nullptr;
+        };
+        int i = 0, buf = 0;
+        while (i < kk) {
+            // the first block must be there; three more are taken if they are
+            const int more = min(SB_SPAN, kk - i);
+            unsigned long long u[SB_SPAN];
+#pragma unroll
+            for (int q = 0; q < SB_SPAN; ++q) {
+                const unsigned long long* p = q < more ? slot(i + q) : nullptr;
+                u[q] = p ? sb_ldv(p) : 0ull;
+            }
+            if (tid < ((B * KC + 31) & ~31)) {
+                const unsigned long long* p = slot(i);
+                unsigned polls = 0;
+                while (__any_sync(0xffffffffu, u[0] == SB_EMPTY)) {
+                    ++polls;
+                    const bool give_up = polls > a.max_polls ||
+                                         ((polls & 255u) == 0 && *(volatile unsigned*)a.err != 0u);
+                    if (__any_sync(0xffffffffu, give_up)) {
+                        if (lane == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
+                        if (u[0] == SB_EMPTY) u[0] = 0ull;
+                        break;
+                    }
+                    if (polls > 64) __nanosleep(polls > 4096 ? 128 : 20);
+                    if (u[0] == SB_EMPTY) u[0] = sb_ldv(p);
+                }
+#pragma unroll
+                for (int q = 0; q < SB_SPAN; ++q)
+                    if (tid < B * KC) s_x[buf][q * B * KC + tid] = AR::from_bits(u[q]);
+            }
+            bool ready = more == SB_SPAN;
+#pragma unroll
+            for (int q = 1; q < SB_SPAN; ++q) ready = ready && u[q] != SB_EMPTY;
+            const int span = __syncthreads_and(ready) ? SB_SPAN : 1;
+            // this thread's entries inside the blocks just loaded
+            const int64_t first = (int64_t)(FWD ? i : nblk - i - span) * B;   // lowest row of the span
+            const int lim = FWD ? (int)min(first + (int64_t)span * B, (int64_t)0x7fffffff) : (int)first;
+            while (FWD ? cq[0] < lim : cq[0] >= lim) {
+                const int d = cq[0] - (int)first;
+                // forward: block q of the span starts at q B; backward: the span runs downwards
+                const int at = FWD ? d : (span - 1 - d / B) * B + (d & (B - 1));
+                AR::mad(acc, vq[0], s_x[buf][at * KC + c]);
+#pragma unroll
+                for (int q = 0; q + 1 < SB_AHEAD; ++q) { cq[q] = cq[q + 1]; vq[q] = vq[q + 1]; }
+                fetch(cq[SB_AHEAD - 1], vq[SB_AHEAD - 1]);
+            }
+            i += span;
+            buf ^= 1;
+        }
+        __syncwarp();
+        // s_row = base - sum over the row's ES threads
+        AR::norm(acc);
+        V s = AR::neg(acc);
+        if (h == 0) { AR::norm(base); AR::add(s, base); }
+#pragma unroll
+        for (int o = KC; o < KC * ES; o <<= 1) AR::add(s, AR::xorv(s, o));
+        if (h == 0) s_s[row * KC + c] = s;
+        __syncthreads();
+        // x_row = sum_k inv(row, k) s_k over the triangle; the warp skips what is zero for all
+        // of its rows
+        const int wrow0 = (tid & ~31) / (KC * ES), wrow1 = (tid | 31) / (KC * ES);
+        V x = AR::zero();
+#pragma unroll
+        for (int t = 0; t < PER; ++t) {
+            const bool need = FWD ? ES * t <= wrow1 : ES * t + ES - 1 >= wrow0;
+            if (need) AR::madv(x, inv[t], s_s[(h + ES * t) * KC + c]);
+        }
+        AR::norm(x);
+#pragma unroll
+        for (int o = KC; o < KC * ES; o <<= 1) AR::add(x, AR::xorv(x, o));
+        if (h == 0 && live) {
+            sb_stv(xnew + j * a.K + col, AR::to_bits(x));
+            if (a.out64) a.out64[j * a.K + col] = AR::to_double(x);
+        }
+        __syncthreads();   // s_s and s_x are reused by the next block
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// Inverses of the 128-row lower diagonal blocks D + L of M: the block in shared memory (M's
+// entries, the identity beyond n), inverted in place from the last column to the first
+// (column j of the inverse is -X_sub l_j / l_jj with X_sub the inverse of the rows below),
+// eight threads per row.  FP64 throughout; FP32 M (whose sweeps use the FP32-rounded
+// off-diagonal entries and the FP64 diagonal) gets them as float pairs.
+// Bound: FP64 FMA (350 k per block, two a clock per SM: ~85 us per block and SM).
+// ---------------------------------------------------------------------------------------
+constexpr int SI_LD = SB_ROWS + 1;
+constexpr size_t SI_SMEM = (size_t)SB_ROWS * SI_LD * 8;
+template <typename MT>
+__global__ void __launch_bounds__(1024, 1) k_block_inverse(int64_t n, const int64_t* mptr, const int32_t* mcol,
+                                                           const MT* mval, const double* mval64,
+                                                           const int64_t* mdiag, void* inv) {
+    extern __shared__ __align__(16) double s_a[];   // SB_ROWS x SI_LD, row-major
+    __shared__ double s_l[SB_ROWS];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int nblk = (int)((n + SB_ROWS - 1) / SB_ROWS);
+    for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
+        const int64_t j0 = (int64_t)b * SB_ROWS;
+        for (int t = tid; t < SB_ROWS * SI_LD; t += 1024) s_a[t] = 0.0;
+        __syncthreads();
+        for (int r = wid; r < SB_ROWS; r += 32) {
+            const int64_t j = j0 + r;
+            if (j >= n) {
+                if (lane == 0) s_a[r * SI_LD + r] = 1.0;
+                continue;
+            }
+            const int64_t ed = mdiag[j], e0 = mptr[j];
+            if (lane == 0) s_a[r * SI_LD + r] = mval64[ed];
+            for (int64_t e = ed - 1 - lane; e >= e0; e -= 32) {   // sorted: leave below the block
+                const int32_t k = mcol[e];
+                if (k < j0) break;
+                s_a[r * SI_LD + (int)(k - j0)] = (double)mval[e];
+            }
+        }
+        __syncthreads();
+        const int row = tid >> 3, h = tid & 7;
+        for (int j = SB_ROWS - 1; j >= 0; --j) {
+            if (tid < SB_ROWS) s_l[tid] = s_a[tid * SI_LD + j];
+            __syncthreads();
+            const double xjj = 1.0 / s_l[j];
+            double t0 = 0.0, t1 = 0.0;
+            if (row > j) {
+                int k = j + 1 + h;
+                for (; k + 8 <= row; k += 16) {
+                    t0 = fma(s_a[row * SI_LD + k], s_l[k], t0);
+                    t1 = fma(s_a[row * SI_LD + k + 8], s_l[k + 8], t1);
+                }
+                if (k <= row) t0 = fma(s_a[row * SI_LD + k], s_l[k], t0);
+            }
+            t0 += t1;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) t0 += __shfl_xor_sync(0xffffffffu, t0, o);
+            if (h == 0 && row > j) s_a[row * SI_LD + j] = -t0 * xjj;
+            if (tid == 0) s_a[j * SI_LD + j] = xjj;
+            __syncthreads();
+        }
+        for (int t = tid; t < SB_ROWS * SB_ROWS; t += 1024) {
+            const double v = s_a[(t / SB_ROWS) * SI_LD + t % SB_ROWS];
+            const int64_t at = (int64_t)b * SB_ROWS * SB_ROWS + t;
+            if (sizeof(MT) == 4) reinterpret_cast<f2*>(inv)[at] = df_from_double(v);
+            else reinterpret_cast<double*>(inv)[at] = v;
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// Level of every row by the same chain of blocks: lev1(j) = 1 + max lev1 over the row's
+// dependencies (1 without any); 0 = not yet known.  Dependencies in earlier blocks are
+// followed as in the sweep; inside the block the rows are relaxed until nothing changes
+// (as many rounds as the block's own depth).  Even CTAs take the forward direction, odd ones the
+// backward one.
+// ---------------------------------------------------------------------------------------
+constexpr int SL_T = 256;
+template <bool FWD>
+__device__ __forceinline__ void levels_blocked(int64_t n, const int64_t* mptr, const int32_t* mcol,
+                                               const int64_t* mdiag, int* lev1, int* maxlev, unsigned* err,
+                                               unsigned max_polls, int first_blk, int stride) {
+    constexpr int B = SB_ROWS, ES = SL_T / B;
+    __shared__ int s_x[2][B];
+    __shared__ int s_lev[B];
+    __shared__ unsigned s_bits[B][B / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int row = tid / ES, h = tid % ES;
+    const int nblk = (int)((n + B - 1) / B);
+    int mymax = 0;
+    for (int kk = first_blk; kk < nblk; kk += stride) {
+        const int kb = FWD ? kk : nblk - 1 - kk;
+        const int64_t j = (int64_t)kb * B + row;
+        const int64_t j0 = (int64_t)kb * B;
+        int64_t e = 0, e_end = 0;
+        if (j < n) {
+            e_end = mdiag[j];
+            e = FWD ? mptr[j] + h : mptr[j + 1] - 1 - h;
+        }
+        constexpr int PAST = FWD ? 0x7fffffff : -1;
+        auto fetch = [&]() -> int {
+            const bool in = j < n && (FWD ? e < e_end : e > e_end);
+            if (!in) return PAST;
+            const int cc = mcol[e];
+            e += FWD ? ES : -ES;
+            return cc;
+        };
+        for (int t = tid; t < B * (B / 32); t += SL_T) s_bits[t / (B / 32)][t % (B / 32)] = 0u;
+        int c0 = fetch(), c1 = fetch(), mx = 0;
+        int buf = 0;
+        for (int i = 0; i < kk; ++i) {
+            const int64_t f = (int64_t)(FWD ? i : nblk - 1 - i) * B;   // first row of that block
+            if (tid < B) {
+                int v = f + tid < n ? *(volatile int*)(lev1 + f + tid) : 1;
+                unsigned polls = 0;
+                while (__any_sync(0xffffffffu, v == 0)) {
+                    ++polls;
+                    const bool give_up = polls > max_polls || ((polls & 255u) == 0 && *(volatile unsigned*)err != 0u);
+                    if (__any_sync(0xffffffffu, give_up)) {
+                        if (lane == 0) atomicOr(err, DEV_ERR_TIMEOUT);
+                        v = max(v, 1);
+                        break;
+                    }
+                    if (polls > 64) __nanosleep(polls > 4096 ? 128 : 20);
+                    if (v == 0) v = *(volatile int*)(lev1 + f + tid);
+                }
+                s_x[buf][tid] = v;
+            }
+            __syncthreads();
+            const int64_t lim = FWD ? f + B : f;
+            while (FWD ? c0 < lim : (c0 >= lim && c0 >= 0)) {
+                mx = max(mx, s_x[buf][c0 - (int)f]);
+                c0 = c1;
+                c1 = fetch();
+            }
+            buf ^= 1;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = 1; o < ES; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        __syncthreads();   // s_bits cleared
+        while (c0 != PAST) {   // what is left of the row lies inside the block
+            const int d = c0 - (int)j0;
+            atomicOr(&s_bits[row][d >> 5], 1u << (d & 31));
+            c0 = c1;
+            c1 = fetch();
+        }
+        if (h == 0) s_lev[row] = mx + 1;
+        __syncthreads();
+        unsigned w[B / 32];
+        int lv = 0;
+        if (tid < B) {
+            lv = s_lev[tid];
+#pragma unroll
+            for (int q = 0; q < B / 32; ++q) w[q] = s_bits[tid][q];
+        }
+        for (int round = 0; round < B; ++round) {
+            int nv = lv;
+            if (tid < B) {
+#pragma unroll
+                for (int q = 0; q < B / 32; ++q) {
+                    unsigned m = w[q];
+                    while (m) {
+                        nv = max(nv, *(volatile int*)&s_lev[q * 32 + __ffs(m) - 1] + 1);
+                        m &= m - 1;
+                    }
+                }
+            }
+            const bool changed = nv != lv;
+            if (changed) { lv = nv; *(volatile int*)&s_lev[tid] = nv; }
+            if (!__syncthreads_or(changed)) break;
+        }
+        if (tid < B && j0 + tid < n) {
+            *(volatile int*)(lev1 + j0 + tid) = lv;
+            mymax = max(mymax, lv - 1);
+        }
+        __syncthreads();
+    }
+    if (mymax > 0) atomicMax(maxlev, mymax);
+}
+__global__ void __launch_bounds__(SL_T) k_levels_blocked(int64_t n, const int64_t* mptr, const int32_t* mcol,
+                                                         const int64_t* mdiag, int* lev1_f, int* lev1_b,
+                                                         int* max_f, int* max_b, unsigned* err,
+                                                         unsigned max_polls) {
+    const int half = gridDim.x >> 1, at = blockIdx.x >> 1;
+    if (blockIdx.x & 1) levels_blocked<false>(n, mptr, mcol, mdiag, lev1_b, max_b, err, max_polls, at, half);
+    else levels_blocked<true>(n, mptr, mcol, mdiag, lev1_f, max_f, err, max_polls, at, half);
+}
+
+// ---------------------------------------------------------------------------------------
+// Host side
+// ---------------------------------------------------------------------------------------
+// Resident CTAs of a kernel on the current device (looked up once per kernel and device).
+static lsq_status resident_ctas(const void* kern, int threads, size_t smem, int* out) {
+    static std::mutex mu;
+    static std::unordered_map<const void*, int> known[64];
+    int dev = 0;
+    LSQ_CUDA(cudaGetDevice(&dev));
+    if (dev < 64) {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = known[dev].find(kern);
+        if (it != known[dev].end()) { *out = it->second; return LSQ_OK; }
+    }
+    int sms = 0, per = 0;
+    LSQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    LSQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem));
+    if (per < 1) { set_error("blocked sweep kernel does not fit on an SM"); return LSQ_ERR_CUDA; }
+    *out = sms * per;
+    if (dev < 64) {
+        std::lock_guard<std::mutex> lk(mu);
+        known[dev][kern] = *out;
+    }
+    return LSQ_OK;
+}
+
+// Rows per block and columns per CTA.  Double-float: 128 rows for one column, 64 rows and up to 4
+// columns for a block of right-hand sides (the same number of inverse entries per thread).  FP64:
+// 64 rows, because the product of a block costs B^2 / 2 FMAs per column at two a clock.
+template <typename MT, typename AR, bool FWD>
+static const void* sb_kernel(int K, int* B, int* KC) {
+    constexpr bool pair = std::is_same<AR, SbPair>::value;
+    if (K == 1) {
+        *KC = 1;
+        *B = pair ? 128 : 64;
+        if constexpr (pair) return (const void*)k_sweep_blocked<MT, AR, FWD, 128, 1>;
+        else return (const void*)k_sweep_blocked<MT, AR, FWD, 64, 1>;
+    }
+    *B = 64;
+    if (K == 2) { *KC = 2; return (const void*)k_sweep_blocked<MT, AR, FWD, 64, 2>; }
+    *KC = 4;
+    return (const void*)k_sweep_blocked<MT, AR, FWD, 64, 4>;
+}
+
+lsq_status sb_launch(const SbArgs& a, bool fwd, bool m32, bool pairs, cudaStream_t st) {
+    int B = 0, KC = 0;
+    const void* kern;
+    if (pairs) kern = fwd ? sb_kernel<float, SbPair, true>(a.K, &B, &KC) : sb_kernel<float, SbPair, false>(a.K, &B, &KC);
+    else if (m32) kern = fwd ? sb_kernel<float, SbDouble, true>(a.K, &B, &KC) : sb_kernel<float, SbDouble, false>(a.K, &B, &KC);
+    else kern = fwd ? sb_kernel<double, SbDouble, true>(a.K, &B, &KC) : sb_kernel<double, SbDouble, false>(a.K, &B, &KC);
+    int res = 0;
+    lsq_status r = resident_ctas(kern, SB_T, 0, &res);
+    if (r != LSQ_OK) return r;
+    const int64_t tasks = (a.n + B - 1) / B * ((a.K + KC - 1) / KC);
+    SbArgs av = a;
+    void* params[] = {&av};
+    LSQ_CUDA(cudaLaunchCooperativeKernel(kern, dim3((unsigned)std::min<int64_t>(tasks, res)), dim3(SB_T), params, 0, st));
+    count_launch();
+    return LSQ_OK;
+}
+
+lsq_status sb_build_inverse(SparseHandle* S, int64_t n, bool m32, cudaStream_t st) {
+    const int64_t nblk = (n + SB_ROWS - 1) / SB_ROWS;
+    const int64_t levels = S->nlev_f < S->nlev_b ? S->nlev_f : S->nlev_b;
+    // by blocks when the chain of blocks is shorter than the level schedule
+    if (nblk > levels) return LSQ_OK;
+    LSQ_CUDA(cudaMalloc(&S->inv, 8 * (size_t)nblk * SB_ROWS * SB_ROWS));
+    const unsigned g = (unsigned)std::min<int64_t>(nblk, 1 << 20);
+    if (m32) {
+        LSQ_CUDA(cudaFuncSetAttribute(k_block_inverse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SI_SMEM));
+        k_block_inverse<float><<<g, 1024, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval32, S->mval, S->mdiag, S->inv);
+    } else {
+        LSQ_CUDA(cudaFuncSetAttribute(k_block_inverse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SI_SMEM));
+        k_block_inverse<double><<<g, 1024, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval, S->mval, S->mdiag, S->inv);
+    }
+    count_launch();
+    LSQ_CUDA(cudaGetLastError());
+    return LSQ_OK;
+}
+
+lsq_status sb_levels(const SparseHandle* S, int64_t n, int* lev1_f, int* lev1_b, int* max_f, int* max_b,
+                     unsigned* err, cudaStream_t st) {
+    int res = 0;
+    lsq_status r = resident_ctas((const void*)k_levels_blocked, SL_T, 0, &res);
+    if (r != LSQ_OK) return r;
+    const int64_t nblk = (n + SB_ROWS - 1) / SB_ROWS;
+    unsigned grid = (unsigned)std::min<int64_t>(2 * nblk, res) & ~1u;
+    int64_t nn = n;
+    const int64_t *mptr = S->mptr, *mdiag = S->mdiag;
+    const int32_t* mcol = S->mcol;
+    unsigned max_polls = dep_wait_polls();
+    void* params[] = {&nn, (void*)&mptr, (void*)&mcol, (void*)&mdiag, &lev1_f, &lev1_b, &max_f, &max_b, &err, &max_polls};
+    LSQ_CUDA(cudaLaunchCooperativeKernel((const void*)k_levels_blocked, dim3(grid), dim3(SL_T), params, 0, st));
+    count_launch();
+    return LSQ_OK;
+}
+
+}  // namespace lsq
