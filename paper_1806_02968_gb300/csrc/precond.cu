@@ -1,95 +1,19 @@
-// Sec. 3.3 (sampled normal matrix) and Alg. 3 (symmetric Gauss-Seidel preconditioner).
+// Sec. 3.3 (sampled normal matrix) and Alg. 3 (symmetric Gauss-Seidel preconditioner): the
+// handle and its C entries.
 //
-// Dense path: M = A_s^T A_s is assembled by a split-K tiled product over the draws
-// (deterministic: partial tiles are summed in a fixed order), made exactly symmetric, and
-// its zero diagonal entries are replaced by 1.  The SGS operator of Alg. 3 is then
+// Dense path (dense_build.cu): M = A_s^T A_s is summed over the draws in a fixed order, exactly
+// symmetric, its zero diagonal entries replaced by 1.  The SGS operator of Alg. 3 is then
 // materialised: column j of the operator is the result of running the t forward and t
 // backward Gauss-Seidel sweeps, in the natural row order, on the unit vector e_j from a
 // zero start.  Inside PCG the preconditioner is one parallel matrix-vector product with
 // that operator instead of a 2n-step dependency chain per application.
 #include "common.cuh"
-#include "values.cuh"
+#include "dense_build.cuh"
 #include "sparse.cuh"
 
+#include <algorithm>
+
 namespace lsq {
-
-constexpr int MT = 64;   // M tile edge
-constexpr int MK = 16;   // draws per smem stage
-
-__global__ void k_gamma(const double* p, int64_t s, double* gam) {
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < s;
-         t += (int64_t)gridDim.x * blockDim.x)
-        gam[t] = __drcp_rn(__dmul_rn((double)s, p[t]));  // 1 / (s p_{i_t})
-}
-
-// part[z][j][k] = sum over draws t in split z of gam_t â_{i_t j} â_{i_t k}, for the tile
-// pair (blockIdx.x = j tile, blockIdx.y = k tile), k tile >= j tile.
-template <int DT>
-__global__ void __launch_bounds__(256) k_build_M_dense(lsq_matrix A, const int32_t* idx,
-                                                      const double* gam, const double* inv_d,
-                                                      int64_t s, int64_t per_split, double* part) {
-    if (blockIdx.y < blockIdx.x) return;
-    const int64_t n = A.n;
-    const int64_t j0 = (int64_t)blockIdx.x * MT, k0 = (int64_t)blockIdx.y * MT;
-    const int64_t t_begin = (int64_t)blockIdx.z * per_split;
-    const int64_t t_end = min(s, t_begin + per_split);
-    __shared__ double Xj[MK][MT], Xk[MK][MT];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double acc[4][4] = {};
-    for (int64_t t0 = t_begin; t0 < t_end; t0 += MK) {
-        for (int e = threadIdx.x; e < MK * MT; e += 256) {
-            int tt = e / MT, c = e % MT;
-            int64_t t = t0 + tt;
-            double vj = 0.0, vk = 0.0;
-            if (t < t_end) {
-                int64_t row = (int64_t)idx[t] * A.ld;
-                if (j0 + c < n) vj = __dmul_rn(__dmul_rn(Val<DT>::load(A.vals, row + j0 + c), inv_d[j0 + c]), gam[t]);
-                if (k0 + c < n) vk = __dmul_rn(Val<DT>::load(A.vals, row + k0 + c), inv_d[k0 + c]);
-            }
-            Xj[tt][c] = vj;
-            Xk[tt][c] = vk;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int tt = 0; tt < MK; ++tt) {
-            double a[4], b[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) { a[r] = Xj[tt][ty * 4 + r]; b[r] = Xk[tt][tx * 4 + r]; }
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[r][q] = fma(a[r], b[q], acc[r][q]);
-        }
-        __syncthreads();
-    }
-    double* out = part + (int64_t)blockIdx.z * n * n;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        int64_t j = j0 + ty * 4 + r;
-        if (j >= n) continue;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            int64_t k = k0 + tx * 4 + q;
-            if (k < n) out[j * n + k] = acc[r][q];
-        }
-    }
-}
-
-// M[j][k] = M[k][j] = sum_z part[z][j][k] for j <= k (fixed order); zero diagonal -> 1.
-__global__ void k_reduce_M(int64_t n, int splits, const double* part, double* M,
-                           unsigned long long* n_fixed) {
-    int64_t total = n * n;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        int64_t j = e / n, k = e % n;
-        if (k < j) continue;
-        double v = 0.0;
-        for (int z = 0; z < splits; ++z) v += part[(int64_t)z * total + e];
-        if (j == k && v == 0.0) { v = 1.0; atomicAdd(n_fixed, 1ull); }
-        M[j * n + k] = v;
-        M[k * n + j] = v;
-    }
-}
 
 // The identity operator (t = 0: CG on the column-normalised system, the paper's comparison
 // method in Sec. 5)
@@ -97,40 +21,6 @@ template <typename OT>
 __global__ void k_identity_op(int64_t n, OT* op) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * n; t += (int64_t)gridDim.x * blockDim.x)
         op[t] = (t / n == t % n) ? OT(1) : OT(0);
-}
-
-// Column j of the SGS operator: Alg. 3 on r = e_j from e = 0, t forward sweeps (rows
-// 0..n-1) then t backward sweeps (rows n-1..0), each the in-place Gauss-Seidel update
-// e_k <- (r_k - sum_{l != k} M_kl e_l) / M_kk (equal to e <- e + B^{-1}(r - M e) forward
-// and e <- e + B^{-T}(r - M e) backward).  One warp per column; e lives in shared memory.
-template <typename OT>
-__global__ void k_sgs_materialize(int64_t n, int sweeps, const double* M, OT* op) {
-    extern __shared__ double s_e[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t j = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid;
-    if (j >= n) return;
-    double* e = s_e + (int64_t)wid * n;
-    for (int64_t l = lane; l < n; l += 32) e[l] = 0.0;
-    __syncwarp();
-    for (int sw = 0; sw < 2 * sweeps; ++sw) {
-        const bool fwd = sw < sweeps;
-        for (int64_t kk = 0; kk < n; ++kk) {
-            const int64_t k = fwd ? kk : n - 1 - kk;
-            int64_t lo = 0, hi = n;
-            if (sw == 0) {  // first forward sweep from zero: only rows >= j move, and only
-                if (k < j) continue;  // already-updated entries l in [j, k) contribute
-                lo = j; hi = k;
-            }
-            const double* Mk = M + k * n;
-            double part = 0.0;
-            for (int64_t l = lo + lane; l < hi; l += 32)
-                if (l != k) part = fma(Mk[l], e[l], part);
-            double ssum = warp_sum(part);
-            if (lane == 0) e[k] = ((k == j ? 1.0 : 0.0) - ssum) / Mk[k];
-            __syncwarp();
-        }
-    }
-    for (int64_t k = lane; k < n; k += 32) op[k * n + j] = (OT)e[k];
 }
 
 template <typename OT>
@@ -164,52 +54,24 @@ __global__ void k_op_to_f64(int64_t count, const float* src, double* dst) {
         dst[e] = (double)src[e];
 }
 
-template <int DT>
 static lsq_status build_dense(const lsq_matrix* A, const int32_t* idx, const double* p,
                               int64_t s, lsq_precond* H, cudaStream_t st) {
     const int64_t n = A->n;
-    const int64_t ntj = (n + MT - 1) / MT;
-    const int64_t active = ntj * (ntj + 1) / 2;
-    int64_t splits = (4 * 152 + active - 1) / active;
-    int64_t max_splits = (s + 63) / 64;
-    if (splits > max_splits) splits = max_splits;
-    if (splits < 1) splits = 1;
-    if (splits > 64) splits = 64;
-    int64_t per_split = (s + splits - 1) / splits;
-    per_split = (per_split + MK - 1) / MK * MK;
-    splits = (s + per_split - 1) / per_split;
-
     Scratch sc;
-    size_t bytes = 256 + 8 * (size_t)s + 8 * (size_t)splits * n * n;
-    LSQ_CUDA(sc.alloc(bytes, st));
+    LSQ_CUDA(sc.alloc(256, st));
     unsigned long long* n_fixed = sc.as<unsigned long long>();
-    double* gam = (double*)(sc.as<char>() + 256);
-    double* part = gam + s;
     LSQ_CUDA(cudaMemsetAsync(n_fixed, 0, 16, st));
-
-    k_gamma<<<(unsigned)std::min<int64_t>((s + 255) / 256, 4096), 256, 0, st>>>(p, s, gam);
-    dim3 grid((unsigned)ntj, (unsigned)ntj, (unsigned)splits);
-    k_build_M_dense<DT><<<grid, 256, 0, st>>>(*A, idx, gam, H->inv_d, s, per_split, part);
-    k_reduce_M<<<(unsigned)std::min<int64_t>((n * n + 255) / 256, 152 * 16), 256, 0, st>>>(
-        n, (int)splits, part, H->M, n_fixed);
-    count_launch(3);
-    const int wpb = 4;
-    size_t smem = (size_t)wpb * n * sizeof(double);
-    unsigned g = (unsigned)((n + wpb - 1) / wpb);
+    lsq_status r = dense_normal_matrix(A, idx, p, H->inv_d, s, H->M, n_fixed, st);
+    if (r != LSQ_OK) return r;
     if (H->sweeps == 0) {   // the comparison method: P = I on the normalised system
         const unsigned gi = (unsigned)std::min<int64_t>((n * n + 255) / 256, 152 * 16);
         if (H->op_dtype == LSQ_F32) k_identity_op<float><<<gi, 256, 0, st>>>(n, (float*)H->op);
         else k_identity_op<double><<<gi, 256, 0, st>>>(n, (double*)H->op);
-    } else if (H->op_dtype == LSQ_F32) {
-        if (smem > 48 * 1024)
-            LSQ_CUDA(cudaFuncSetAttribute(k_sgs_materialize<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_sgs_materialize<float><<<g, 32 * wpb, smem, st>>>(n, H->sweeps, H->M, (float*)H->op);
+        count_launch();
     } else {
-        if (smem > 48 * 1024)
-            LSQ_CUDA(cudaFuncSetAttribute(k_sgs_materialize<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_sgs_materialize<double><<<g, 32 * wpb, smem, st>>>(n, H->sweeps, H->M, (double*)H->op);
+        r = dense_sgs_operator(n, H->sweeps, H->M, H->op, H->op_dtype, st);
+        if (r != LSQ_OK) return r;
     }
-    count_launch();
     LSQ_CUDA(cudaGetLastError());
     unsigned long long nf = 0;
     LSQ_CUDA(cudaMemcpyAsync(&nf, n_fixed, 8, cudaMemcpyDeviceToHost, st));
@@ -271,13 +133,7 @@ extern "C" lsq_status lsq_build_precond(const lsq_matrix* A, const int32_t* idx,
         set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
         return fail(LSQ_ERR_NOMEM);
     }
-    lsq_status r;
-    switch (A->dtype) {
-        case LSQ_F64: r = build_dense<LSQ_F64>(A, idx, p, s, H, st); break;
-        case LSQ_F32: r = build_dense<LSQ_F32>(A, idx, p, s, H, st); break;
-        case LSQ_BF16: r = build_dense<LSQ_BF16>(A, idx, p, s, H, st); break;
-        default: r = build_dense<LSQ_F32X2>(A, idx, p, s, H, st); break;
-    }
+    lsq_status r = build_dense(A, idx, p, s, H, st);
     if (r != LSQ_OK) return fail(r);
     *P_out = H;
     return LSQ_OK;
