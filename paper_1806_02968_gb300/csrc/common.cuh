@@ -86,6 +86,7 @@ struct Scratch {
 };
 
 // Reads the device error word (after a stream sync) and maps it to a status.
+lsq_status dev_error_status(unsigned bits);   // the status of an error word
 lsq_status read_dev_error(const unsigned* d_err, cudaStream_t st, unsigned* bits_out = nullptr);
 
 // ---------------------------------------------------------------------------------------

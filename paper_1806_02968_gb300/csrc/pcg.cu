@@ -4,6 +4,7 @@
 #include "values.cuh"
 #include "sparse.cuh"
 
+#include <algorithm>
 #include <vector>
 
 namespace lsq {
@@ -20,24 +21,36 @@ static int64_t pick_nmax(int dt, int dtr, int64_t n) {
 
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
+// Workspace of one dense solve: the control block (barriers, error word, per-column results)
+// and the vectors of the groups.
 struct SolveWork {
     Scratch sc;
-    double *y, *g, *z, *part_w, *part_s, *out_d;
-    unsigned *bar, *err;
+    double *vec, *part_w, *part_s, *out_d;
+    unsigned long long* bar;
+    unsigned* err;
     int32_t* out_i;
-    size_t ctl_bytes;
-    lsq_status alloc(int64_t n, cudaStream_t st) {
+    size_t o_i, o_d, res_bytes, ctl_bytes;   // results first (err, out_i, out_d), then the barriers
+    lsq_status alloc(int64_t n, int64_t k, cudaStream_t st) {
         const int Gmax = pcg_max_grid();
+        const int64_t groups = std::min<int64_t>(k, 16);
         size_t off = 0;
         auto take = [&](size_t b) { size_t at = off; off += (b + 255) & ~size_t(255); return at; };
-        size_t o_ctl = take(256), o_y = take(8 * n), o_g = take(8 * n), o_z = take(8 * n),
-               o_ps = take(8 * (size_t)Gmax * PART_S), o_pw = take(8 * (size_t)Gmax * n);
+        o_i = 16;
+        o_d = 16 + 16 * (size_t)k;
+        res_bytes = o_d + 32 * (size_t)k;
+        const size_t o_res = take(res_bytes), o_bar = take(8 * (size_t)PCG_BAR_STRIDE * groups);
+        ctl_bytes = off;
+        const size_t o_v = take(24 * (size_t)n * groups), o_ps = take(8 * (size_t)Gmax * PART_S),
+                     o_pw = take(8 * (size_t)Gmax * n);
         LSQ_CUDA(sc.alloc(off, st));
         char* b = sc.as<char>();
-        bar = (unsigned*)b; err = bar + 2; out_i = (int32_t*)(b + 16); out_d = (double*)(b + 64);
-        ctl_bytes = 256;
-        y = (double*)(b + o_y); g = (double*)(b + o_g); z = (double*)(b + o_z);
-        part_s = (double*)(b + o_ps); part_w = (double*)(b + o_pw);
+        err = (unsigned*)(b + o_res);
+        out_i = (int32_t*)(b + o_res + o_i);
+        out_d = (double*)(b + o_res + o_d);
+        bar = (unsigned long long*)(b + o_bar);
+        vec = (double*)(b + o_v);
+        part_s = (double*)(b + o_ps);
+        part_w = (double*)(b + o_pw);
         return LSQ_OK;
     }
 };
@@ -73,8 +86,8 @@ static lsq_status check_dense_solve(const lsq_matrix* A, const lsq_precond* P, i
     return LSQ_OK;
 }
 
-// One persistent-kernel solve per column.  h_cols (n-space right-hand sides) selects the
-// normal form used by the adjoint.
+// All columns in one launch of the persistent kernel.  Hcols (n-space right-hand sides)
+// selects the normal form used by the adjoint.
 static lsq_status solve_columns(const lsq_matrix* A, const lsq_precond* P, const double* B,
                                 const double* Hcols, int64_t k, int64_t ldb, double* X, int64_t ldx,
                                 const lsq_opts* o, lsq_info* info, cudaStream_t st) {
@@ -84,46 +97,47 @@ static lsq_status solve_columns(const lsq_matrix* A, const lsq_precond* P, const
     if (s0 != LSQ_OK) return s0;
     const int64_t m = A->m, n = A->n;
     SolveWork wk;
-    s0 = wk.alloc(n, st);
+    s0 = wk.alloc(n, k, st);
     if (s0 != LSQ_OK) return s0;
     cudaEvent_t e0, e1;
     LSQ_CUDA(cudaEventCreate(&e0));
     LSQ_CUDA(cudaEventCreate(&e1));
     LSQ_CUDA(cudaEventRecord(e0, st));
+    LSQ_CUDA(cudaMemsetAsync(wk.err, 0, wk.ctl_bytes, st));
+    PcgArgs a{};
+    a.m = m; a.n = n; a.ld = A->ld;
+    a.vals = A->vals;
+    a.vals_res = (dtr == LSQ_F64 && A->dtype != LSQ_F64) ? (const void*)A->vals_f64 : A->vals;
+    a.inv_d = P->inv_d;
+    a.op = P->op;
+    a.b = B;
+    a.h_in = Hcols;
+    a.x = X;
+    a.ncol = k; a.ldb = ldb; a.ldx = ldx;
+    a.vec = wk.vec;
+    a.part_w = wk.part_w; a.part_s = wk.part_s;
+    a.bar = wk.bar; a.err = wk.err;
+    a.tol = o->tol;
+    a.inner_tol = o->inner_tol > 0 ? o->inner_tol : 0.0;
+    a.maxit = o->maxit; a.max_outer = o->max_outer;
+    a.out_i = wk.out_i; a.out_d = wk.out_d;
+    a.max_polls = barrier_wait_polls();
+    lsq_status ls = dt == LSQ_F64 ? launch_pcg_f64(nmax, P->op_dtype, a, o->grid_ctas, st)
+                  : dt == LSQ_F32 ? launch_pcg_f32(nmax, dtr, P->op_dtype, a, o->grid_ctas, st)
+                  : dt == LSQ_BF16 ? launch_pcg_bf16(nmax, dtr, P->op_dtype, a, o->grid_ctas, st)
+                                  : launch_pcg_f32x2(nmax, dtr, P->op_dtype, a, o->grid_ctas, st);
+    if (ls != LSQ_OK) return ls;
+    LSQ_CUDA(cudaGetLastError());
+    LSQ_CUDA(cudaEventRecord(e1, st));
+    std::vector<char> res(wk.res_bytes);
+    LSQ_CUDA(cudaMemcpyAsync(res.data(), wk.err, wk.res_bytes, cudaMemcpyDeviceToHost, st));
+    LSQ_CUDA(cudaStreamSynchronize(st));
+    lsq_status es = dev_error_status(*reinterpret_cast<const unsigned*>(res.data()));
+    if (es != LSQ_OK) return es;
     lsq_status worst = LSQ_OK;
     for (int64_t c = 0; c < k; ++c) {
-        LSQ_CUDA(cudaMemsetAsync(wk.bar, 0, wk.ctl_bytes, st));
-        PcgArgs a{};
-        a.m = m; a.n = n; a.ld = A->ld;
-        a.vals = A->vals;
-        a.vals_res = (dtr == LSQ_F64 && A->dtype != LSQ_F64) ? (const void*)A->vals_f64 : A->vals;
-        a.inv_d = P->inv_d;
-        a.op = P->op;
-        a.b = B ? B + c * ldb : nullptr;
-        a.h_in = Hcols ? Hcols + c * ldb : nullptr;
-        a.x = X + c * ldx;
-        a.y = wk.y; a.g = wk.g; a.z = wk.z;
-        a.part_w = wk.part_w; a.part_s = wk.part_s;
-        a.bar = reinterpret_cast<unsigned long long*>(wk.bar); a.err = wk.err;
-        a.tol = o->tol;
-        a.inner_tol = o->inner_tol > 0 ? o->inner_tol : 0.0;
-        a.maxit = o->maxit; a.max_outer = o->max_outer;
-        a.out_i = wk.out_i; a.out_d = wk.out_d;
-        a.max_polls = barrier_wait_polls();
-        int G = 0;
-        lsq_status ls = dt == LSQ_F64 ? launch_pcg_f64(nmax, P->op_dtype, a, o->grid_ctas, st, &G)
-                      : dt == LSQ_F32 ? launch_pcg_f32(nmax, dtr, P->op_dtype, a, o->grid_ctas, st, &G)
-                      : dt == LSQ_BF16 ? launch_pcg_bf16(nmax, dtr, P->op_dtype, a, o->grid_ctas, st, &G)
-                                      : launch_pcg_f32x2(nmax, dtr, P->op_dtype, a, o->grid_ctas, st, &G);
-        if (ls != LSQ_OK) return ls;
-        LSQ_CUDA(cudaGetLastError());
-        int32_t oi[4];
-        double od[3];
-        unsigned bits = 0;
-        LSQ_CUDA(cudaMemcpyAsync(oi, wk.out_i, sizeof(oi), cudaMemcpyDeviceToHost, st));
-        LSQ_CUDA(cudaMemcpyAsync(od, wk.out_d, sizeof(od), cudaMemcpyDeviceToHost, st));
-        lsq_status es = read_dev_error(wk.err, st, &bits);
-        if (es != LSQ_OK) return es;
+        const int32_t* oi = reinterpret_cast<const int32_t*>(res.data() + wk.o_i) + 4 * c;
+        const double* od = reinterpret_cast<const double*>(res.data() + wk.o_d) + 4 * c;
         if (info && c < info->k) {
             if (info->iters) info->iters[c] = oi[0];
             if (info->outer) info->outer[c] = oi[1];
@@ -136,8 +150,6 @@ static lsq_status solve_columns(const lsq_matrix* A, const lsq_precond* P, const
         if (cs == LSQ_ERR_BREAKDOWN) worst = LSQ_ERR_BREAKDOWN;
         else if (cs != LSQ_OK && worst == LSQ_OK) worst = LSQ_ERR_NOT_CONVERGED;
     }
-    LSQ_CUDA(cudaEventRecord(e1, st));
-    LSQ_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
     cudaEventDestroy(e0);

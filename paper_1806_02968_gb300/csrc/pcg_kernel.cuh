@@ -2,7 +2,14 @@
 // run to completion (including restarts from the true residual) inside ONE persistent
 // cooperative kernel.
 //
-// Work split: CTA c owns the contiguous row block [c m/G, (c+1) m/G) of A for the fused
+// Several right-hand sides run side by side: the grid is cut into groups of G CTAs, each of
+// which solves one column at a time.  The columns are independent, so one group's barriers and
+// vector phases overlap the passes of the others, and groups that pass over the same rows
+// together share them in L2.  One column: one group of all CTAs.
+// Eight columns of 60,001 x 201 FP32 values (FP64 residuals): 3.2 ms, against 7.8 ms one column
+// after the other.
+//
+// Work split (inside a group): CTA c owns the contiguous row block [c m/G, (c+1) m/G) of A for the fused
 // pass w = Â^T (Â p) (each row is read from HBM once: its dot with p̃ = D^{-1} p gives q_i,
 // and the same registers are then scaled by q_i into the CTA's n-vector partial), and the
 // column slice [c n/G, (c+1) n/G) for the n-vector updates and for the rows of the
@@ -29,22 +36,27 @@ struct PcgArgs {
     const void* vals_res;  // values for h and the true residual (dtype DTR)
     const double* inv_d;   // 1 / d_j
     const void* op;        // n x n row-major SGS operator (OPT)
-    const double* b;       // m (least-squares form)
-    const double* h_in;    // n: right-hand side of Â^T Â y = h (normal form), or NULL
-    double* x;             // n (output)
-    double* y;             // n workspace
-    double* g;             // n workspace
-    double* z;             // n workspace
-    double* part_w;        // G x n
-    double* part_s;        // G x PART_S
-    unsigned long long* bar;  // grid barrier count (zeroed before the launch)
+    const double* b;       // k columns of m (least-squares form), column c at b + c ldb
+    const double* h_in;    // k right-hand sides of Â^T Â y = h (normal form, n each), or NULL
+    double* x;             // k columns of n (output), column c at x + c ldx
+    int64_t ncol, ldb, ldx;
+    double* vec;           // y, g and z of every group (3 n each)
+    double* part_w;        // grid x n
+    double* part_s;        // grid x PART_S
+    unsigned long long* bar;  // barrier counts of the groups, PCG_BAR_STRIDE apart (zeroed before the launch)
     unsigned* err;
     double tol, inner_tol;
     int32_t maxit, max_outer;
-    int32_t* out_i;        // iters, outer, converged, status
-    double* out_d;         // relres_rec, relres_true, relres_raw
+    int32_t* out_i;        // per column: iters, outer, converged, status
+    double* out_d;         // per column: relres_rec, relres_true, relres_raw, unused
     unsigned max_polls = 1u << 26;   // bound of every grid-barrier wait
+    int G;                 // CTAs of a group: group q = CTAs [q G, (q + 1) G) solves columns q, q + NG, ...
+    int NG;                // groups
+    // set by the kernel for its own CTA
+    int bid;               // CTA inside its group
+    double *y, *g, *z;     // the group's n-vectors
 };
+constexpr int PCG_BAR_STRIDE = 16;   // 64-bit words: one 128-byte line per group's barrier
 
 __device__ __forceinline__ int64_t imin64(int64_t x, int64_t y) { return x < y ? x : y; }
 
@@ -511,6 +523,17 @@ __device__ __forceinline__ void ring_prefetch(Ring& ring, const char* src, const
     ring.pre_count = cnt;
 }
 
+// part_s[cta][0] = the sum of the nw warps' q partials, by warp 0 in a tree (a dependent FP64
+// step takes ~64 cycles on GB300, so a serial sum of 16 would take half a microsecond)
+__device__ __forceinline__ void write_q_partial(const PcgArgs& a, const double* s_scal, int nw) {
+    if (threadIdx.x < 32) {
+        double t = (int)threadIdx.x < nw ? s_scal[threadIdx.x] : 0.0;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) a.part_s[(int64_t)a.bid * PART_S + 0] = t;
+    }
+}
+
 // Fused row pass over the CTA's rows [r0, r1), streamed HBM -> shared memory with 1D bulk
 // copies (the row block is one contiguous byte range):
 //   MATVEC: q_i = â_i . p̃      RHS: q_i = b_i      RESID: q_i = b_i - â_i . ỹ
@@ -551,16 +574,21 @@ __device__ __forceinline__ bool row_pass_rpw(const PcgArgs& a, const void* vals,
     Ops::zero(acc, qacc);
     bool ok = true;
     int slot = 0;
+    // b of this warp's rows, one stage ahead
+    auto load_b = [&](int i, int k) -> double {
+        const int64_t gi = r0 + (int64_t)i * g.R + wid * RPW + k;
+        return (MODE != PASS_MATVEC && k < RPW && wid * RPW + k < g.R && gi < r1) ? a.b[gi] : 0.0;
+    };
+    double nb0 = load_b(0, 0), nb1 = load_b(0, 1);
     for (int i = 0; i < nst; ++i) {
+        const double b0 = nb0, b1 = nb1;
+        if (MODE != PASS_MATVEC) { nb0 = load_b(i + 1, 0); nb1 = load_b(i + 1, 1); }
         if (!ring_wait(ring, slot)) ok = false;
         const int rows_here = min(g.R, nrows - i * g.R);
         const int lr = wid * RPW;    // first local row of this warp
         if (ok && lr < rows_here) {
             const char* base = ring.buf + slot * g.stage_bytes;
-            const int64_t gi = r0 + (int64_t)i * g.R + lr;
             const bool has1 = (RPW == 2) && (lr + 1 < rows_here);
-            const double b0 = (MODE == PASS_MATVEC) ? 0.0 : a.b[gi];
-            const double b1 = (MODE == PASS_MATVEC || !has1) ? 0.0 : a.b[gi + 1];
             const char* rp0 = base + lr * g.row_bytes;
             const char* rp1 = has1 ? rp0 + g.row_bytes : rp0;
             Ops::template row<MODE, RPW == 2>(rp0, rp1, has1, s_vc, lane, n, b0, b1, acc, qacc);
@@ -580,17 +608,13 @@ __device__ __forceinline__ bool row_pass_rpw(const PcgArgs& a, const void* vals,
     Ops::store(acc, s_red + (int64_t)wid * NMAX, lane);
     if (lane == 0) s_scal[wid] = Ops::q_out(qacc);
     __syncthreads();
-    double* pw = a.part_w + (int64_t)blockIdx.x * n;
+    double* pw = a.part_w + (int64_t)a.bid * n;
     for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
         RT sacc = Ops::red_zero();
         for (int w = 0; w < nwarps; ++w) Ops::red_add(sacc, s_red[(int64_t)w * NMAX + j]);
         pw[j] = Ops::red_out(sacc);
     }
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < nwarps; ++w) t += s_scal[w];
-        a.part_s[(int64_t)blockIdx.x * PART_S + 0] = t;
-    }
+    write_q_partial(a, s_scal, nwarps);
     __syncthreads();
     return ok;
 }
@@ -746,26 +770,169 @@ __device__ __forceinline__ bool row_pass_split(const PcgArgs& a, const void* val
             ring.ephase ^= (1u << slot);
             slot = (slot + 1 == g.slots) ? 0 : slot + 1;
         }
-        double* pw = a.part_w + (int64_t)blockIdx.x * n;
+        double* pw = a.part_w + (int64_t)a.bid * n;
 #pragma unroll
         for (int c = 0; c < CPL; ++c)
             if (FULL || col0 + c < n) pw[col0 + c] = df_to_double(df_norm(acc[c]));
     }
     if (!ok) raise_grid_error(a.err, a.bar, DEV_ERR_TIMEOUT);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < 8; ++w) t += s_scal[w];
-        a.part_s[(int64_t)blockIdx.x * PART_S + 0] = t;
-    }
+    write_q_partial(a, s_scal, 8);
     __syncthreads();
     return ok;
+}
+
+// The fused row pass for FP64 values, rows straight into registers.  GB300 issues a warp's FP64
+// instruction every 64 cycles per scheduler, so the pass is bound by the number of FP64
+// instructions, not by loads: a group of WPR warps takes R rows at a time (each lane two columns of
+// every 64-column chunk), and the R dot products share one reduce-scatter (R = 4: 6 adds for 4
+// rows, where pairs of rows with four chains each took 26), one chain per row.  The products of
+// four warps per scheduler hide the loads, so nothing is staged and no barrier stands inside the
+// pass.  Rows wider than 512 columns are split over two warps, which exchange their halves' dot
+// products.  R is what the registers hold: 8 up to 128 columns, 4 up to 320, else 2.
+// 90,000 x 300: 137 us per PCG iteration, against 182 us by pairs of rows from the staging ring
+// (86 us of FMAs at the pipe's rate).
+template <int NCH, int R, int WPR>
+__device__ __noinline__ void row_pass_f64(int mode, const double* vals, int64_t ld, const double* b, int n, const double* s_v,
+                                          double* s_red, double* s_scal, double* pw, int64_t r0, int64_t r1) {
+    constexpr int LG = R == 8 ? 3 : (R == 4 ? 2 : 1);
+    __shared__ double s_x[WPR == 2 ? 2 : 1][16][R];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int grp = wid / WPR, half = wid % WPR;
+    constexpr int NG = 16 / WPR;
+    const int col0 = half * NCH * 64 + lane * 2;
+    const int ri = lane >> (5 - LG);                  // the row whose sum this lane ends up with
+    const bool lead = (lane & ((32 >> LG) - 1)) == 0 && half == 0;
+    double2 acc[NCH];
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) acc[c] = make_double2(0.0, 0.0);
+    double qs = 0.0;
+    int buf = 0;
+    for (int64_t r = r0 + grp * R; r < r1; r += NG * R) {
+        double2 v[R][NCH];
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const double* row = vals + (r + i < r1 ? r + i : r1 - 1) * ld;
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+                const int col = col0 + c * 64;
+                v[i][c] = col < n ? __ldcs(reinterpret_cast<const double2*>(row + col)) : make_double2(0.0, 0.0);
+                if (col + 1 >= n) v[i][c].y = 0.0;    // row padding never enters the sums
+            }
+        }
+        double q = 0.0;
+        if (mode != PASS_RHS) {
+            double d[R];
+#pragma unroll
+            for (int i = 0; i < R; ++i) d[i] = 0.0;
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+                const double2 x = *reinterpret_cast<const double2*>(s_v + col0 + c * 64);
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    d[i] = fma(v[i][c].x, x.x, d[i]);
+                    d[i] = fma(v[i][c].y, x.y, d[i]);
+                }
+            }
+            // reduce-scatter: each step sends half of the rows it still holds
+#pragma unroll
+            for (int st = 0; st < LG; ++st) {
+                const int o = 16 >> st;
+                const int hold = R >> (st + 1);
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int i = 0; i < hold; ++i) {
+                    const double send = up ? d[i] : d[i + hold];
+                    const double keep = up ? d[i + hold] : d[i];
+                    d[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+#pragma unroll
+            for (int o = 16 >> LG; o > 0; o >>= 1) d[0] += __shfl_xor_sync(0xffffffffu, d[0], o);
+            q = d[0];
+            if (WPR == 2) {
+                if ((lane & ((32 >> LG) - 1)) == 0) s_x[buf][wid][ri] = q;
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");
+                q = s_x[buf][wid & ~1][ri] + s_x[buf][wid | 1][ri];
+                buf ^= 1;
+            }
+        }
+        if (mode != PASS_MATVEC) {
+            const double bi = r + ri < r1 ? b[r + ri] : 0.0;
+            q = mode == PASS_RHS ? bi : bi - q;
+        }
+        if (r + ri >= r1) q = 0.0;
+        qs = fma(lead ? q : 0.0, q, qs);
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const double qi = __shfl_sync(0xffffffffu, q, i << (5 - LG));
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+                acc[c].x = fma(qi, v[i][c].x, acc[c].x);
+                acc[c].y = fma(qi, v[i][c].y, acc[c].y);
+            }
+        }
+    }
+    constexpr int W = WPR * NCH * 64;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) *reinterpret_cast<double2*>(s_red + (int64_t)grp * W + col0 + c * 64) = acc[c];
+    qs = warp_sum(qs);
+    if (lane == 0) s_scal[wid] = qs;
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        double t0 = 0.0, t1 = 0.0;
+#pragma unroll
+        for (int w = 0; w < NG; w += 2) {
+            t0 += s_red[w * W + j];
+            t1 += s_red[(w + 1) * W + j];
+        }
+        pw[j] = t0 + t1;
+    }
+}
+// Rows a CTA needs for the register form: two rounds of all its groups; below, the ring's
+// stages, which are fetched during the barriers before the pass, are the better start.
+__device__ __forceinline__ bool f64_direct(int n, int64_t rows) {
+    if (n > 1024) return false;
+    return rows >= (n <= 128 ? 256 : (n <= 320 ? 128 : (n <= 512 ? 64 : 32)));
+}
+template <int NMAX, int MODE>
+__device__ __forceinline__ bool row_pass_direct(const PcgArgs& a, const void* vals, const double* s_v, double* s_scal,
+                                                int64_t r0, int64_t r1, Ring& ring) {
+    if (ring.pre_count > 0) ring_drain(ring);
+    const double* A = reinterpret_cast<const double*>(vals);
+    double* red = reinterpret_cast<double*>(ring.buf);
+    double* pw = a.part_w + (int64_t)a.bid * a.n;
+    const int n = (int)a.n;
+#define LSQ_F64_PASS(NCH, R, WPR) row_pass_f64<NCH, R, WPR>(MODE, A, a.ld, a.b, n, s_v, red, s_scal, pw, r0, r1)
+    if constexpr (NMAX == 128) {
+        if (n <= 64) LSQ_F64_PASS(1, 8, 1); else LSQ_F64_PASS(2, 8, 1);
+    } else if constexpr (NMAX == 256) {
+        if (n <= 192) LSQ_F64_PASS(3, 4, 1); else LSQ_F64_PASS(4, 4, 1);
+    } else if constexpr (NMAX == 512) {
+        if (n <= 320) LSQ_F64_PASS(5, 4, 1);
+        else if (n <= 384) LSQ_F64_PASS(6, 2, 1);
+        else if (n <= 448) LSQ_F64_PASS(7, 2, 1);
+        else LSQ_F64_PASS(8, 2, 1);
+    } else {
+        if (n <= 640) LSQ_F64_PASS(5, 2, 2);
+        else if (n <= 768) LSQ_F64_PASS(6, 2, 2);
+        else if (n <= 896) LSQ_F64_PASS(7, 2, 2);
+        else LSQ_F64_PASS(8, 2, 2);
+    }
+#undef LSQ_F64_PASS
+    write_q_partial(a, s_scal, 16);
+    __syncthreads();
+    return true;
 }
 
 template <int DT, int NMAX, int MODE>
 __device__ __forceinline__ bool row_pass(const PcgArgs& a, const void* vals, const double* s_v,
                                          void* s_vc_raw, double* s_scal, int64_t r0, int64_t r1,
                                          Ring& ring) {
+    if constexpr (DT == LSQ_F64 && NMAX <= 1024) {
+        if (blockDim.x == 512 && f64_direct((int)a.n, r1 - r0))
+            return row_pass_direct<NMAX, MODE>(a, vals, s_v, s_scal, r0, r1, ring);
+    }
     const Geo g = geometry(a.ld, RowOps<DT, NMAX>::ES, blockDim.x >> 5, ring.bytes);
     if constexpr (DT == LSQ_F32X2 && MODE == PASS_MATVEC && (NMAX == 256 || NMAX == 512)) {
         if (g.rpw == 1 && g.R == 16 && g.slots >= 2 && blockDim.x == 512) {
@@ -781,7 +948,7 @@ __device__ __forceinline__ bool row_pass(const PcgArgs& a, const void* vals, con
 // CTA sums in the same order, so all agree bit for bit); no block barrier.  Four loads per
 // lane are in flight together.
 __device__ __forceinline__ double warp_grid_scalar(const PcgArgs& a, int slot) {
-    const int lane = threadIdx.x & 31, G = (int)gridDim.x;
+    const int lane = threadIdx.x & 31, G = a.G;
     const double* ps = a.part_s + slot;
     double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
     int g = lane;
@@ -795,19 +962,51 @@ __device__ __forceinline__ double warp_grid_scalar(const PcgArgs& a, int slot) {
     return warp_sum((t0 + t1) + (t2 + t3));
 }
 
-// Writes the CTA partials pa, pb (one per warp, in s_scal) to part_s[cta][slot_a/slot_b].
-__device__ __forceinline__ void cta_partials(const PcgArgs& a, double pa, double pb, int slot_a,
-                                             int slot_b, double* s_scal) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    if (lane == 0) { s_scal[wid] = pa; s_scal[32 + wid] = pb; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double ta = 0.0, tb = 0.0;
-        for (int w = 0; w < nwarps; ++w) { ta += s_scal[w]; tb += s_scal[32 + w]; }
-        a.part_s[(int64_t)blockIdx.x * PART_S + slot_a] = ta;
-        a.part_s[(int64_t)blockIdx.x * PART_S + slot_b] = tb;
+// Scalars are computed by warp 0 alone and handed to the others through shared memory: an FP64
+// instruction holds its scheduler for ~64 cycles per warp, so a square root and a division done
+// by all 16 warps cost several us of every iteration (262,144 x 512 double-float: 195.6 us per
+// iteration before, 187.5 us now).  s_bc holds two sets used in turn, so that the
+// one being read is never the one being written.
+struct Scalars {
+    double (*set)[4];
+    int at;
+};
+// f(out) fills up to four values in warp 0 (all its lanes run it, lane 0 stores); returns the set after
+// a block barrier.
+template <typename F>
+__device__ __forceinline__ const double* warp0_scalars(Scalars& sc, F f) {
+    double* s = sc.set[sc.at];
+    sc.at ^= 1;
+    if (threadIdx.x < 32) {
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        f(v);
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s[k] = v[k];
+        }
     }
     __syncthreads();
+    return s;
+}
+
+// Writes the CTA partials pa, pb (one per warp, of the first nw warps) to part_s[cta][slot_a/slot_b].
+__device__ __forceinline__ void cta_partials(const PcgArgs& a, double pa, double pb, int slot_a,
+                                             int slot_b, double* s_scal, int nw) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane == 0) { s_scal[wid] = pa; s_scal[32 + wid] = pb; }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        const double* v = s_scal + 32 * threadIdx.x;
+        double t = 0.0;
+        for (int w = 0; w < nw; ++w) t += v[w];
+        a.part_s[(int64_t)a.bid * PART_S + (threadIdx.x ? slot_b : slot_a)] = t;
+    }
+    __syncthreads();
+}
+// warps that own a column of [c0, c1)
+__device__ __forceinline__ int owner_warps(int64_t c0, int64_t c1) {
+    const int64_t c = c1 - c0;
+    return (int)(c < (blockDim.x >> 5) ? c : (blockDim.x >> 5));
 }
 
 // w_j = (1/d_j) sum_g part_w[g][j] for the owned columns (one warp per column), handed on
@@ -819,7 +1018,7 @@ __device__ __forceinline__ void slice_reduce(const PcgArgs& a, int64_t c0, int64
     double pa = 0.0, pb = 0.0;
     for (int64_t j = c0 + wid; j < c1; j += nwarps) {
         double t = 0.0;
-        for (int g = lane; g < (int)gridDim.x; g += 32) t += a.part_w[(int64_t)g * a.n + j];
+        for (int g = lane; g < a.G; g += 32) t += a.part_w[(int64_t)g * a.n + j];
         t = warp_sum(t);
         if (lane == 0) {
             double2 r = fn(j, t * s_invd[j]);
@@ -827,7 +1026,7 @@ __device__ __forceinline__ void slice_reduce(const PcgArgs& a, int64_t c0, int64
             pb += r.y;
         }
     }
-    cta_partials(a, pa, pb, slot_a, slot_b, s_scal);
+    cta_partials(a, pa, pb, slot_a, slot_b, s_scal, owner_warps(c0, c1));
 }
 
 // z_j = sum_k op_jk g_k for the owned rows (g staged in s_v); partial g^T z -> slot 2.
@@ -856,101 +1055,108 @@ __device__ __forceinline__ void op_rows(const PcgArgs& a, int64_t c0, int64_t c1
             part = fma(s_v[j], zj, part);
         }
     }
-    cta_partials(a, part, 0.0, 2, 7, s_scal);
+    cta_partials(a, part, 0.0, 2, 7, s_scal, owner_warps(c0, c1));
 }
 
-// The phase after the fused pass: p^T w as the grid sum of the CTAs' ||Â p||^2 partials
-// (computed by every warp), then for the owned columns w_j = (1/d_j) sum_g part_w[g][j],
-// y_j += alpha p_j, g_j -= alpha w_j and the CTA's partial of ||g||^2 (slot 1).  The loads
-// of p^T w's partials, of a warp's first column's partials and of its y_j and g_j are all
-// issued before any of them is used.  Returns false on a PCG breakdown (non-positive or
-// non-finite p^T w or rho), the same decision in every thread of the grid.
+// The phase after the fused pass: p^T w as the grid sum of the CTAs' ||Â p||^2 partials, then
+// for the owned columns w_j = (1/d_j) sum_g part_w[g][j], y_j += alpha p_j, g_j -= alpha w_j and
+// the CTA's partial of ||g||^2 (slot 1).  Only the warps that own a column (and warp 0, for the
+// decision) work: the loads of p^T w's partials, of a warp's first column's partials and of its y_j
+// and g_j are all issued before any of them is used.  Returns false on a PCG breakdown
+// (non-positive or non-finite p^T w or rho), the same decision in every thread of the grid.
 __device__ __forceinline__ bool step_update(const PcgArgs& a, int64_t c0, int64_t c1, double rho,
-                                            const double* s_p, const double* s_invd, double* s_scal) {
+                                            const double* s_p, const double* s_invd, double* s_scal, Scalars& sc) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int G = (int)gridDim.x;
+    const int G = a.G;
     const int64_t n = a.n;
     const int64_t j0 = c0 + wid;
     const bool own = j0 < c1;
-    double yj = 0.0, gj = 0.0;
-    if (own && lane == 0) { yj = a.y[j0]; gj = a.g[j0]; }
-    const double* ps = a.part_s;
-    const double* pw = a.part_w + (own ? j0 : 0);
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0, u0 = 0.0, u1 = 0.0, u2 = 0.0, u3 = 0.0;
-    int g = lane;
-    for (; g + 96 < G; g += 128) {
-        t0 += ps[(int64_t)g * PART_S];
-        t1 += ps[(int64_t)(g + 32) * PART_S];
-        t2 += ps[(int64_t)(g + 64) * PART_S];
-        t3 += ps[(int64_t)(g + 96) * PART_S];
-        if (own) {
-            u0 += pw[(int64_t)g * n];
-            u1 += pw[(int64_t)(g + 32) * n];
-            u2 += pw[(int64_t)(g + 64) * n];
-            u3 += pw[(int64_t)(g + 96) * n];
-        }
-    }
-    for (; g < G; g += 32) {
-        t0 += ps[(int64_t)g * PART_S];
-        if (own) u0 += pw[(int64_t)g * n];
-    }
-    const double pTw = warp_sum((t0 + t1) + (t2 + t3));
-    const double wsum = warp_sum((u0 + u1) + (u2 + u3));
-    if (!(pTw > 0.0) || !(rho > 0.0) || !isfinite(pTw) || !isfinite(rho)) return false;
-    const double alpha = rho / pTw;
     double part = 0.0;
-    if (own && lane == 0) {
-        const double w = wsum * s_invd[j0];
-        yj = fma(alpha, s_p[j0], yj);
-        gj = fma(-alpha, w, gj);
-        a.y[j0] = yj;
-        a.g[j0] = gj;
-        part = gj * gj;
-    }
-    for (int64_t j = j0 + nwarps; j < c1; j += nwarps) {   // more columns than warps
-        double t = 0.0;
-        for (int gg = lane; gg < G; gg += 32) t += a.part_w[(int64_t)gg * n + j];
-        t = warp_sum(t);
-        if (lane == 0) {
-            const double w = t * s_invd[j];
-            a.y[j] = fma(alpha, s_p[j], a.y[j]);
-            const double gn = fma(-alpha, w, a.g[j]);
-            a.g[j] = gn;
-            part += gn * gn;
+    double* flag = sc.set[sc.at];
+    sc.at ^= 1;
+    if (own || wid == 0) {
+        double yj = 0.0, gj = 0.0;
+        if (own && lane == 0) { yj = a.y[j0]; gj = a.g[j0]; }
+        const double* ps = a.part_s;
+        const double* pw = a.part_w + (own ? j0 : 0);
+        double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0, u0 = 0.0, u1 = 0.0, u2 = 0.0, u3 = 0.0;
+        int g = lane;
+        for (; g + 96 < G; g += 128) {
+            t0 += ps[(int64_t)g * PART_S];
+            t1 += ps[(int64_t)(g + 32) * PART_S];
+            t2 += ps[(int64_t)(g + 64) * PART_S];
+            t3 += ps[(int64_t)(g + 96) * PART_S];
+            if (own) {
+                u0 += pw[(int64_t)g * n];
+                u1 += pw[(int64_t)(g + 32) * n];
+                u2 += pw[(int64_t)(g + 64) * n];
+                u3 += pw[(int64_t)(g + 96) * n];
+            }
+        }
+        for (; g < G; g += 32) {
+            t0 += ps[(int64_t)g * PART_S];
+            if (own) u0 += pw[(int64_t)g * n];
+        }
+        const double pTw = warp_sum((t0 + t1) + (t2 + t3));
+        const double wsum = own ? warp_sum((u0 + u1) + (u2 + u3)) : 0.0;
+        const bool ok = pTw > 0.0 && rho > 0.0 && isfinite(pTw) && isfinite(rho);
+        if (wid == 0 && lane == 0) flag[0] = ok ? 1.0 : 0.0;
+        if (ok && own) {
+            const double alpha = rho / pTw;
+            if (lane == 0) {
+                const double w = wsum * s_invd[j0];
+                yj = fma(alpha, s_p[j0], yj);
+                gj = fma(-alpha, w, gj);
+                a.y[j0] = yj;
+                a.g[j0] = gj;
+                part = gj * gj;
+            }
+            for (int64_t j = j0 + nwarps; j < c1; j += nwarps) {   // more columns than warps
+                double t = 0.0;
+                for (int gg = lane; gg < G; gg += 32) t += a.part_w[(int64_t)gg * n + j];
+                t = warp_sum(t);
+                if (lane == 0) {
+                    const double w = t * s_invd[j];
+                    a.y[j] = fma(alpha, s_p[j], a.y[j]);
+                    const double gn = fma(-alpha, w, a.g[j]);
+                    a.g[j] = gn;
+                    part += gn * gn;
+                }
+            }
         }
     }
-    cta_partials(a, part, 0.0, 1, 6, s_scal);
-    return true;
+    cta_partials(a, part, 0.0, 1, 6, s_scal, owner_warps(c0, c1));
+    return flag[0] != 0.0;
 }
 
-// Copies the n-vector src (global) into s_dst and returns the grid sum of part_s[][slot];
-// the vector's loads and the partials' loads are in flight together.
-template <int NMAX>
-__device__ __forceinline__ double stage_with_scalar(const PcgArgs& a, const double* src, double* s_dst, int slot) {
-    constexpr int PER = (NMAX + 511) / 512;
-    double v[PER];
-#pragma unroll
-    for (int r = 0; r < PER; ++r) {
-        const int64_t j = threadIdx.x + (int64_t)r * blockDim.x;
-        v[r] = j < a.n ? src[j] : 0.0;
-    }
-    const double s = warp_grid_scalar(a, slot);
-#pragma unroll
-    for (int r = 0; r < PER; ++r) {
-        const int64_t j = threadIdx.x + (int64_t)r * blockDim.x;
-        if (j < a.n) s_dst[j] = v[r];
-    }
-    return s;
+// The stop test after an update, by warp 0: out[0] = ||g||^2, out[1] = rec = ||g|| / ||h||,
+// out[2] = 1 when rec meets tol or ||g|| meets the inner tolerance.  The square root and the
+// division are only needed near a threshold or for the report, so they run once the squares are
+// within a rounding of it; rec is -1 otherwise.
+struct StopRule { double tol, inner, hn, thr2; };
+__device__ __forceinline__ StopRule stop_rule(double tol, double inner, double hn) {
+    const double t = tol * hn;
+    const double thr = t > inner ? t : inner;
+    return StopRule{tol, inner, hn, thr * thr * (1.0 + 1e-12) + 1e-300};
 }
 
 template <int DT, int DTR, int NMAX, typename OPT>
-__global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
+__global__ void __launch_bounds__(512, 1) k_pcg_dense(const PcgArgs args) {
+    PcgArgs a = args;
+    const int grp = (int)blockIdx.x / a.G;
+    a.bid = (int)blockIdx.x - grp * a.G;
+    a.bar += grp * PCG_BAR_STRIDE;
+    a.y = a.vec + (int64_t)grp * 3 * a.n; a.g = a.y + a.n; a.z = a.g + a.n;
+    a.part_w += (int64_t)grp * a.G * a.n;
+    a.part_s += (int64_t)grp * a.G * PART_S;
     extern __shared__ __align__(128) char smem_raw[];
     __shared__ double s_scal[64];
     __shared__ __align__(8) uint64_t s_bars[RING_SLOTS];
     __shared__ __align__(8) uint64_t s_qbars[RING_SLOTS];
     __shared__ __align__(8) uint64_t s_ebars[RING_SLOTS];
     __shared__ __align__(16) f2 s_q[RING_SLOTS * 16];
+    __shared__ double s_bc[2][4];
+    Scalars sc{s_bc, 0};
     const int64_t n = a.n;
     const int nwarps = blockDim.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -974,11 +1180,19 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
         s_invd[j] = j < n ? a.inv_d[j] : 0.0;
     }
     __syncthreads();
-    const unsigned G = gridDim.x;
-    const int64_t r0 = (int64_t)blockIdx.x * a.m / G, r1 = (int64_t)(blockIdx.x + 1) * a.m / G;
-    const int64_t c0 = (int64_t)blockIdx.x * n / G, c1 = (int64_t)(blockIdx.x + 1) * n / G;
+    const unsigned G = (unsigned)a.G;
+    const int64_t r0 = (int64_t)a.bid * a.m / G, r1 = (int64_t)(a.bid + 1) * a.m / G;
+    const int64_t c0 = (int64_t)a.bid * n / G, c1 = (int64_t)(a.bid + 1) * n / G;
     const Geo gmv = geometry(a.ld, RowOps<DT, NMAX>::ES, nwarps, RB);
     const char* mv_src = reinterpret_cast<const char*>(a.vals) + r0 * (int64_t)gmv.row_bytes;
+    // the first stages of the next matvec pass, fetched during the barriers before it (FP64 rows
+    // that go straight to registers have no stages)
+    auto prefetch = [&]() {
+        if constexpr (DT == LSQ_F64 && NMAX <= 1024) {
+            if (f64_direct((int)n, r1 - r0)) return;
+        }
+        ring_prefetch(ring, mv_src, gmv, r1 - r0);
+    };
 #define LSQ_BARRIER()                                   \
     do {                                                \
         if (!grid_barrier(a.bar, G, a.err, bar_epoch, a.max_polls)) { \
@@ -987,6 +1201,11 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
         }                                               \
     } while (0)
 
+    for (int64_t col = grp; col < a.ncol; col += a.NG) {
+    // every CTA of the group has read the last column's vectors and partial sums
+    if (col != grp) LSQ_BARRIER();
+    a.b = args.b ? args.b + col * a.ldb : nullptr;
+    a.h_in = args.h_in ? args.h_in + col * a.ldb : nullptr;
     int iters = 0, outer_used = 0, converged = 0, status = LSQ_ERR_NOT_CONVERGED;
     double rec = 1.0, tru = 1.0, gg = 0.0;
     bool dirty = false;  // iterations since the last true residual
@@ -999,10 +1218,10 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
             a.g[j] = h; a.y[j] = 0.0;
             ha = fma(h, h, ha); hb = fma(hr, hr, hb);
         }
-        cta_partials(a, warp_sum(ha), warp_sum(hb), 1, 4, s_scal);
+        cta_partials(a, warp_sum(ha), warp_sum(hb), 1, 4, s_scal, nwarps);
     } else {
         row_pass<DTR, NMAX, PASS_RHS>(a, a.vals_res, s_v, s_vc, s_scal, r0, r1, ring);
-        ring_prefetch(ring, mv_src, gmv, r1 - r0);
+        prefetch();
         LSQ_BARRIER();
         slice_reduce(a, c0, c1, 1, 4, s_scal, s_invd, [&](int64_t j, double h) {
             a.g[j] = h; a.y[j] = 0.0;
@@ -1010,9 +1229,13 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
             return make_double2(h * h, hr * hr); });
     }
     LSQ_BARRIER();
-    gg = warp_grid_scalar(a, 1);
-    const double hn = sqrt(gg);
-    const double hn_raw = sqrt(warp_grid_scalar(a, 4));
+    const double* s0 = warp0_scalars(sc, [&](double (&v)[4]) {
+        v[0] = warp_grid_scalar(a, 1);
+        v[1] = sqrt(v[0]);
+        v[2] = sqrt(warp_grid_scalar(a, 4));
+    });
+    gg = s0[0];
+    const double hn = s0[1], hn_raw = s0[2];
     double raw = 1.0;
     if (hn == 0.0) {
         converged = 1; status = LSQ_OK; rec = 0.0; tru = 0.0;
@@ -1024,7 +1247,7 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
                 __syncthreads();
                 if (a.h_in) row_pass<DTR, NMAX, PASS_MATVEC>(a, a.vals_res, s_v, s_vc, s_scal, r0, r1, ring);
                 else row_pass<DTR, NMAX, PASS_RESID>(a, a.vals_res, s_v, s_vc, s_scal, r0, r1, ring);
-                ring_prefetch(ring, mv_src, gmv, r1 - r0);
+                prefetch();
                 LSQ_BARRIER();
                 slice_reduce(a, c0, c1, 1, 5, s_scal, s_invd, [&](int64_t j, double t) {
                     if (a.h_in) t = a.h_in[j] - t;
@@ -1032,22 +1255,31 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
                     const double tr = t / s_invd[j];
                     return make_double2(t * t, tr * tr); });
                 LSQ_BARRIER();
-                gg = warp_grid_scalar(a, 1);
-                raw = sqrt(warp_grid_scalar(a, 5)) / hn_raw;
+                const double* sr = warp0_scalars(sc, [&](double (&v)[4]) {
+                    v[0] = warp_grid_scalar(a, 1);
+                    v[1] = sqrt(warp_grid_scalar(a, 5)) / hn_raw;
+                });
+                gg = sr[0];
+                raw = sr[1];
                 dirty = false;
             }
-            tru = sqrt(gg) / hn;
+            const double* st = warp0_scalars(sc, [&](double (&v)[4]) {
+                v[0] = sqrt(gg);
+                v[1] = v[0] / hn;
+            });
+            const double gstart = st[0];
+            tru = st[1];
             if (outer == 0) rec = tru;
             if (tru <= a.tol) { converged = 1; status = LSQ_OK; break; }
             if (iters >= a.maxit) break;
             outer_used = outer + 1;
-            const double gstart = sqrt(gg);
+            const StopRule rule = stop_rule(a.tol, a.inner_tol * gstart, hn);
             // z = P g, rho = g^T z, p = z
             for (int64_t j = threadIdx.x; j < n; j += blockDim.x) s_v[j] = a.g[j];
             __syncthreads();
             op_rows<OPT>(a, c0, c1, s_v, s_scal);
             LSQ_BARRIER();
-            double rho = warp_grid_scalar(a, 2);
+            double rho = warp0_scalars(sc, [&](double (&v)[4]) { v[0] = warp_grid_scalar(a, 2); })[0];
             for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
                 const double pj = a.z[j];
                 s_p[j] = pj;
@@ -1058,18 +1290,29 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
             while (true) {
                 // fused pass: w = Â^T (Â p), ||Â p||^2 = p^T w
                 row_pass<DT, NMAX, PASS_MATVEC>(a, a.vals, s_v, s_vc, s_scal, r0, r1, ring);
-                ring_prefetch(ring, mv_src, gmv, r1 - r0);
+                prefetch();
                 LSQ_BARRIER();
-                if (!step_update(a, c0, c1, rho, s_p, s_invd, s_scal)) {
+                if (!step_update(a, c0, c1, rho, s_p, s_invd, s_scal, sc)) {
+                    if (dirty) rec = sqrt(gg) / hn;
                     status = LSQ_ERR_BREAKDOWN; broke = true; break;
                 }
                 LSQ_BARRIER();
                 ++iters;
                 dirty = true;
-                gg = stage_with_scalar<NMAX>(a, a.g, s_v, 1);
-                rec = sqrt(gg) / hn;
-                __syncthreads();
-                if (rec <= a.tol || sqrt(gg) <= a.inner_tol * gstart) break;
+                // g into shared memory by all warps, ||g||^2 and the stop test by warp 0
+                for (int64_t j = threadIdx.x; j < n; j += blockDim.x) s_v[j] = a.g[j];
+                const double* su = warp0_scalars(sc, [&](double (&v)[4]) {
+                    v[0] = warp_grid_scalar(a, 1);
+                    v[1] = -1.0;
+                    if (v[0] <= rule.thr2 || iters >= a.maxit) {
+                        const double gn = sqrt(v[0]);
+                        v[1] = gn / hn;
+                        v[2] = (v[1] <= a.tol || gn <= rule.inner) ? 1.0 : 0.0;
+                    }
+                });
+                gg = su[0];
+                if (su[1] >= 0.0) rec = su[1];
+                if (su[2] != 0.0) break;
                 if (iters >= a.maxit) break;
                 op_rows<OPT>(a, c0, c1, s_v, s_scal);
                 LSQ_BARRIER();
@@ -1082,9 +1325,12 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
                         const int64_t j = threadIdx.x + (int64_t)r * blockDim.x;
                         zv[r] = j < n ? a.z[j] : 0.0;
                     }
-                    const double rho_new = warp_grid_scalar(a, 2);
-                    const double beta = rho_new / rho;
-                    rho = rho_new;
+                    const double* sb = warp0_scalars(sc, [&](double (&v)[4]) {
+                        v[0] = warp_grid_scalar(a, 2);
+                        v[1] = v[0] / rho;
+                    });
+                    const double beta = sb[1];
+                    rho = sb[0];
 #pragma unroll
                     for (int r = 0; r < PER; ++r) {
                         const int64_t j = threadIdx.x + (int64_t)r * blockDim.x;
@@ -1111,18 +1357,28 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(PcgArgs a) {
                 const double tr = t / s_invd[j];
                 return make_double2(t * t, tr * tr); });
             LSQ_BARRIER();
-            tru = sqrt(warp_grid_scalar(a, 3)) / hn;
-            raw = sqrt(warp_grid_scalar(a, 5)) / hn_raw;
+            const double* sf = warp0_scalars(sc, [&](double (&v)[4]) {
+                v[0] = sqrt(warp_grid_scalar(a, 3)) / hn;
+                v[1] = sqrt(warp_grid_scalar(a, 5)) / hn_raw;
+            });
+            tru = sf[0];
+            raw = sf[1];
             if (tru <= a.tol) { converged = 1; status = LSQ_OK; }
         }
     }
-#undef LSQ_BARRIER
     ring_drain(ring);
-    for (int64_t j = c0 + threadIdx.x; j < c1; j += blockDim.x) a.x[j] = a.y[j] * s_invd[j];
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        a.out_i[0] = iters; a.out_i[1] = outer_used; a.out_i[2] = converged; a.out_i[3] = status;
-        a.out_d[0] = rec; a.out_d[1] = tru; a.out_d[2] = (hn == 0.0) ? 0.0 : raw;
+    {
+        double* x = args.x + col * a.ldx;
+        for (int64_t j = c0 + threadIdx.x; j < c1; j += blockDim.x) x[j] = a.y[j] * s_invd[j];
+        if (a.bid == 0 && threadIdx.x == 0) {
+            int32_t* oi = a.out_i + 4 * col;
+            double* od = a.out_d + 4 * col;
+            oi[0] = iters; oi[1] = outer_used; oi[2] = converged; oi[3] = status;
+            od[0] = rec; od[1] = tru; od[2] = (hn == 0.0) ? 0.0 : raw;
+        }
     }
+    }
+#undef LSQ_BARRIER
     (void)lane;
 }
 

@@ -36,6 +36,10 @@ lsq_status read_dev_error(const unsigned* d_err, cudaStream_t st, unsigned* bits
     LSQ_CUDA(cudaMemcpyAsync(&bits, d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
     LSQ_CUDA(cudaStreamSynchronize(st));
     if (bits_out) *bits_out = bits;
+    return dev_error_status(bits);
+}
+
+lsq_status dev_error_status(unsigned bits) {
     if (bits & DEV_ERR_TIMEOUT) { set_error("device-side wait timed out"); return LSQ_ERR_TIMEOUT; }
     if (bits & DEV_ERR_RANGE) { set_error("values must be finite with max a_ij^2 in [2^-900, 2^900]"); return LSQ_ERR_INVALID; }
     if (bits & DEV_ERR_EMPTY) { set_error("no row has positive sampling weight"); return LSQ_ERR_INVALID; }
