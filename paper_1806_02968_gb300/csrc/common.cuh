@@ -5,6 +5,7 @@
 #include <stdint.h>
 #include <string>
 #include <atomic>
+#include <initializer_list>
 
 #include "../../include/lsq.h"
 
@@ -68,6 +69,19 @@ inline size_t elem_size(int dtype) {
 
 lsq_status check_matrix(const lsq_matrix* A);
 
+// Device memory of scratch buffers and handles: stream-ordered allocations from a pool of the
+// library's own (one per device), which keeps up to POOL_KEEP bytes of freed memory mapped. The
+// device's default pool gives everything back at every synchronisation, and mapping it again
+// cost 0.1 to 1 ms per call. The pool gives all it holds back when an allocation fails (which is
+// then tried again), and the rest above POOL_KEEP at every synchronisation.
+constexpr uint64_t POOL_KEEP = 1ull << 30;   // 0.35 % of the device's memory
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t st);
+template <typename T>
+inline cudaError_t pool_alloc(T** p, size_t bytes, cudaStream_t st) { return pool_alloc((void**)p, bytes, st); }
+// Frees a handle's arrays (NULL entries are skipped) once all work on the device has ended:
+// the handle may have been used on any stream.
+void pool_free(std::initializer_list<void*> ptrs);
+
 // Stream-ordered scratch that is released on the same stream when it goes out of scope.
 struct Scratch {
     void* ptr = nullptr;
@@ -77,7 +91,7 @@ struct Scratch {
     Scratch& operator=(const Scratch&) = delete;
     cudaError_t alloc(size_t bytes, cudaStream_t s) {
         st = s;
-        return cudaMallocAsync(&ptr, bytes ? bytes : 16, s);
+        return pool_alloc(&ptr, bytes ? bytes : 16, s);
     }
     ~Scratch() {
         if (ptr) cudaFreeAsync(ptr, st);

@@ -84,10 +84,7 @@ static lsq_status build_dense(const lsq_matrix* A, const int32_t* idx, const dou
 
 static void free_handle(lsq_precond* H) {
     if (!H) return;
-    if (H->M) cudaFree(H->M);
-    if (H->op) cudaFree(H->op);
-    if (H->colscale) cudaFree(H->colscale);
-    if (H->inv_d) cudaFree(H->inv_d);
+    pool_free({H->M, H->op, H->colscale, H->inv_d});
     if (H->sp) free_sparse(H->sp);
     delete H;
 }
@@ -115,9 +112,9 @@ extern "C" lsq_status lsq_build_precond(const lsq_matrix* A, const int32_t* idx,
     H->stream = st;
     auto fail = [&](lsq_status code) { free_handle(H); return code; };
     cudaError_t e;
-    if ((e = cudaMalloc(&H->colscale, sizeof(double) * n)) != cudaSuccess ||
-        (e = cudaMalloc(&H->inv_d, sizeof(double) * n)) != cudaSuccess) {
-        set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    if ((e = pool_alloc(&H->colscale, sizeof(double) * n, st)) != cudaSuccess ||
+        (e = pool_alloc(&H->inv_d, sizeof(double) * n, st)) != cudaSuccess) {
+        set_error(std::string("device memory: ") + cudaGetErrorString(e));
         return fail(LSQ_ERR_NOMEM);
     }
     k_inv<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, colscale, H->colscale, H->inv_d);
@@ -128,9 +125,9 @@ extern "C" lsq_status lsq_build_precond(const lsq_matrix* A, const int32_t* idx,
         *P_out = H;
         return LSQ_OK;
     }
-    if ((e = cudaMalloc(&H->M, sizeof(double) * n * n)) != cudaSuccess ||
-        (e = cudaMalloc(&H->op, elem_size(o->precond_dtype) * n * n)) != cudaSuccess) {
-        set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    if ((e = pool_alloc(&H->M, sizeof(double) * n * n, st)) != cudaSuccess ||
+        (e = pool_alloc(&H->op, elem_size(o->precond_dtype) * n * n, st)) != cudaSuccess) {
+        set_error(std::string("device memory: ") + cudaGetErrorString(e));
         return fail(LSQ_ERR_NOMEM);
     }
     lsq_status r = build_dense(A, idx, p, s, H, st);

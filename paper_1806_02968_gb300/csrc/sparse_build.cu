@@ -659,8 +659,8 @@ static lsq_status levels_by_row(const SparseHandle* S, int64_t n, int* lev1, int
 // offsets into sched).
 static lsq_status level_schedule(int64_t n, const int* lev1, int64_t L, int32_t** sched, int64_t** loff,
                                  cudaStream_t st) {
-    LSQ_CUDA(cudaMalloc(sched, 4 * (size_t)n));
-    LSQ_CUDA(cudaMalloc(loff, 8 * (size_t)(L + 1)));
+    LSQ_CUDA(pool_alloc(sched, 4 * (size_t)n, st));
+    LSQ_CUDA(pool_alloc(loff, 8 * (size_t)(L + 1), st));
     Scratch sc2;
     const int64_t nt = (L + SC_T - 1) / SC_T;   // scan_i64: out[0..L], ceil(L / 512) scratch
     LSQ_CUDA(sc2.alloc(8 * (size_t)(2 * L + nt + 1), st));
@@ -786,7 +786,7 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
     int64_t* ts4 = mcnt + n + 16;
     int32_t* cand = reinterpret_cast<int32_t*>(ts4 + ntn);
     LSQ_CUDA(cudaMemsetAsync(nfix, 0, 32, st));
-    LSQ_CUDA(cudaMalloc(&S->mptr, 8 * (size_t)(n + 1)));
+    LSQ_CUDA(pool_alloc(&S->mptr, 8 * (size_t)(n + 1), st));
     int dev = 0, sms = 0;
     LSQ_CUDA(cudaGetDevice(&dev));
     LSQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -811,11 +811,11 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
     LSQ_CUDA(cudaMemcpyAsync(&mnnz, S->mptr + n, 8, cudaMemcpyDeviceToHost, st));
     LSQ_CUDA(cudaMemcpyAsync(hmax, mmax, 8, cudaMemcpyDeviceToHost, st));
     LSQ_CUDA(cudaStreamSynchronize(st));
-    LSQ_CUDA(cudaMalloc(&S->mcol, 4 * (size_t)mnnz));
-    LSQ_CUDA(cudaMalloc(&S->mval, 8 * (size_t)mnnz));
-    if (H->op_dtype == LSQ_F32) LSQ_CUDA(cudaMalloc(&S->mval32, 4 * (size_t)mnnz));
-    LSQ_CUDA(cudaMalloc(&S->dinv, 8 * (size_t)n));
-    LSQ_CUDA(cudaMalloc(&S->mdiag, 8 * (size_t)n));
+    LSQ_CUDA(pool_alloc(&S->mcol, 4 * (size_t)mnnz, st));
+    LSQ_CUDA(pool_alloc(&S->mval, 8 * (size_t)mnnz, st));
+    if (H->op_dtype == LSQ_F32) LSQ_CUDA(pool_alloc(&S->mval32, 4 * (size_t)mnnz, st));
+    LSQ_CUDA(pool_alloc(&S->dinv, 8 * (size_t)n, st));
+    LSQ_CUDA(pool_alloc(&S->mdiag, 8 * (size_t)n, st));
     ga.mptr = S->mptr; ga.mcol = S->mcol; ga.mval = S->mval; ga.mval32 = S->mval32;
     ga.dinv = S->dinv; ga.mdiag = S->mdiag; ga.acap = (hmax[1] + 1) & ~1;
     r = spgemm_pass<true>(ga, hmax[0], sms, st);
@@ -830,9 +830,9 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
     r = sb_build_inverse(S, n, H->op_dtype == LSQ_F32, st);
     if (r != LSQ_OK) return r;
     // 5. transposed pattern of A for the A^T q pass (values are gathered at solve time)
-    LSQ_CUDA(cudaMalloc(&S->atptr, 8 * (size_t)(n + 1)));
-    LSQ_CUDA(cudaMalloc(&S->atrow, 4 * (size_t)A->nnz));
-    LSQ_CUDA(cudaMalloc(&S->atperm, 8 * (size_t)A->nnz));
+    LSQ_CUDA(pool_alloc(&S->atptr, 8 * (size_t)(n + 1), st));
+    LSQ_CUDA(pool_alloc(&S->atrow, 4 * (size_t)A->nnz, st));
+    LSQ_CUDA(pool_alloc(&S->atperm, 8 * (size_t)A->nnz, st));
     r = transpose_pattern(A->row_ptr, A->col_idx, m, n, A->nnz, S->atptr, S->atrow, S->atperm, st);
     if (r != LSQ_OK) return r;
     LSQ_CUDA(cudaStreamSynchronize(st));
@@ -848,10 +848,8 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
 
 void free_sparse(SparseHandle* S) {
     if (!S) return;
-    cudaFree(S->mptr); cudaFree(S->mcol); cudaFree(S->mval); cudaFree(S->mval32); cudaFree(S->dinv); cudaFree(S->mdiag);
-    cudaFree(S->sched_f); cudaFree(S->sched_b); cudaFree(S->inv);
-    cudaFree(S->atptr); cudaFree(S->atrow);
-    cudaFree(S->atperm); cudaFree(S->loff_f); cudaFree(S->loff_b);
+    pool_free({S->mptr, S->mcol, S->mval, S->mval32, S->dinv, S->mdiag, S->sched_f, S->sched_b, S->inv,
+               S->atptr, S->atrow, S->atperm, S->loff_f, S->loff_b});
     delete S;
 }
 

@@ -530,7 +530,7 @@ lsq_status sb_build_inverse(SparseHandle* S, int64_t n, bool m32, cudaStream_t s
     const int64_t levels = S->nlev_f < S->nlev_b ? S->nlev_f : S->nlev_b;
     // by blocks when the chain of blocks is shorter than the level schedule
     if (nblk > levels) return LSQ_OK;
-    LSQ_CUDA(cudaMalloc(&S->inv, 8 * (size_t)nblk * SB_ROWS * SB_ROWS));
+    LSQ_CUDA(pool_alloc(&S->inv, 8 * (size_t)nblk * SB_ROWS * SB_ROWS, st));
     const unsigned g = (unsigned)std::min<int64_t>(nblk, 1 << 20);
     if (m32) {
         LSQ_CUDA(cudaFuncSetAttribute(k_block_inverse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SI_SMEM));
