@@ -4,6 +4,26 @@
 
 namespace lsq {
 
+// A float as the same double, by integer operations alone: GB300 converts to and from 64-bit types
+// (and does every other FP64 operation) at 2 lanes a clock and SM, integers at 64.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), mag = u & 0x7fffffffu, ex = mag >> 23;
+    unsigned hi = (mag >> 3) + 0x38000000u, lo = u << 29;    // normal: rebias the exponent
+    if (ex - 1u >= 254u) {
+        if (ex == 255u) {
+            hi = (mag >> 3) + 0x70000000u;                   // infinity, NaN
+        } else if (mag == 0u) {
+            hi = lo = 0u;
+        } else {                                             // subnormal: a normal double
+            const int sh = __clz((int)mag) - 8;
+            const unsigned m = mag << sh;
+            hi = ((unsigned)(897 - sh) << 20) | ((m & 0x7fffffu) >> 3);
+            lo = m << 29;
+        }
+    }
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
+}
+
 template <int DT> struct Val;
 template <> struct Val<LSQ_F64> {
     typedef double T;
@@ -14,13 +34,13 @@ template <> struct Val<LSQ_F64> {
 template <> struct Val<LSQ_F32> {
     typedef float T;
     static __device__ __forceinline__ double load(const void* p, int64_t e) {
-        return (double)reinterpret_cast<const float*>(p)[e];
+        return widen(reinterpret_cast<const float*>(p)[e]);
     }
 };
 template <> struct Val<LSQ_BF16> {
     typedef __nv_bfloat16 T;
     static __device__ __forceinline__ double load(const void* p, int64_t e) {
-        return (double)__bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[e]);
+        return widen(__bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[e]));
     }
 };
 template <> struct Val<LSQ_F32X2> {
