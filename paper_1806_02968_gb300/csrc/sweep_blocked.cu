@@ -17,8 +17,8 @@
 // ES sums and the product.  The inverse sits in registers (each thread holds the part of its row
 // it multiplies), loaded while the CTA waits.
 // Measured per sweep: 40,000 rows of 380 dependencies in 1583 levels, one column, double-float:
-// 0.75 ms (2.4 us per block of 128 rows), against 1.75 ms forward and 3.5 ms backward by rows;
-// 10,000 rows of 350 dependencies in 1227 levels, 16 columns: 0.48 ms (3.1 us per block of 64),
+// 0.54 ms (1.7 us per block of 128 rows), against 1.75 ms forward and 3.5 ms backward by rows;
+// 10,000 rows of 350 dependencies in 1227 levels, 16 columns: 0.42 ms (2.7 us per block of 64),
 // against 5.3 and 6.1 ms.
 // Columns are independent chains, so a block of right-hand sides is split over CTAs by KC
 // columns.
@@ -38,7 +38,7 @@ namespace lsq {
 constexpr unsigned long long SB_EMPTY = 0xFFF7DEADBEEFCAFEull;   // the row forms' empty marker
 constexpr int SB_T = 512;
 constexpr int SB_SPAN = 4;          // blocks taken at once while catching up
-constexpr int SB_AHEAD = 4;         // entries of its row a thread holds ahead
+constexpr unsigned SB_FAR_NS = 100; // between the polls of a CTA that is far behind its block
 
 __device__ __forceinline__ unsigned long long sb_ldv(const unsigned long long* p) {
     unsigned long long v;
@@ -47,6 +47,14 @@ __device__ __forceinline__ unsigned long long sb_ldv(const unsigned long long* p
 }
 __device__ __forceinline__ void sb_stv(unsigned long long* p, unsigned long long v) {
     asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// one 4- or 8-byte element global -> shared, asynchronously
+template <typename T>
+__device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if (sizeof(T) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
 }
 
 // Arithmetic of a sweep: double-float pairs for FP32 M, or FP64 sums for either type of M.
@@ -102,6 +110,9 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
     static_assert(ES >= 1 && ES * KC <= 32 && SB_ROWS % B == 0, "thread layout");
     __shared__ V s_x[2][SB_SPAN * B * KC];
     __shared__ V s_s[B * KC];
+    constexpr int AHEAD = sizeof(MT) == 4 ? 6 : 4;       // entries under way per thread
+    __shared__ int s_qc[AHEAD][SB_T];
+    __shared__ MT s_qv[AHEAD][SB_T];
     __shared__ double s_red[SB_T / 32];
     __shared__ int s_stop;
     if (*a.done) return;
@@ -129,7 +140,12 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
     const int32_t* __restrict__ mc = a.mcol;
     unsigned long long* xnew = reinterpret_cast<unsigned long long*>(a.e_new);
     const unsigned long long* xold = reinterpret_cast<const unsigned long long*>(a.e_old);
-    const int c = tid % KC, h = (tid / KC) % ES, row = tid / (KC * ES);
+    // a warp takes RW consecutive rows; the row groups are dealt so that the triangles of the four
+    // schedulers (warps s, s + 4, s + 8, s + 12) are the same size
+    constexpr int RW = 32 / (KC * ES);
+    const int wg = (tid >> 7) & 3, wsch = (tid >> 5) & 3;
+    const int wrow0 = RW * (wg * 4 + ((wg & 1) ? 3 - wsch : wsch)), wrow1 = wrow0 + RW - 1;
+    const int c = tid % KC, h = (tid / KC) % ES, row = wrow0 + lane / (KC * ES);
     const int nblk = (int)((a.n + B - 1) / B);
     const int ngrp = (a.K + KC - 1) / KC;
     const int64_t ntask = (int64_t)nblk * ngrp;
@@ -177,23 +193,32 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
             if (FWD) { e = p0 + h; e_end = pd; }
             else { e = p1 - 1 - h; e_end = pd; }
         }
-        // the cursor holds SB_AHEAD entries: M streams from L2 or HBM, and a load that is waited
-        // for inside the walk stands in the chain; a column past every block ends the walk
+        // The cursor: this thread's entries of M, AHEAD of them under way to its own slots of
+        // shared memory.  M streams from L2 or HBM, and an entry waited for inside the walk stands in
+        // the chain; a queue in registers waits as well, because moving a register up needs the load
+        // that fills it.  A column past every block ends the walk.
         constexpr int PAST = FWD ? 0x7fffffff : -1;
-        int cq[SB_AHEAD];
-        MT vq[SB_AHEAD];
-        auto fetch = [&](int& cc, MT& vv) {
+        auto fetch = [&](int at) {
             const bool in = FWD ? e < e_end : e > e_end;
-            cc = PAST;
-            vv = MT(0);
-            if (in) { cc = mc[e]; vv = mv[e]; e += FWD ? ES : -ES; }
+            if (in) {
+                cp_async_elem(&s_qc[at][tid], mc + e);
+                cp_async_elem(&s_qv[at][tid], mv + e);
+                e += FWD ? ES : -ES;
+            } else {
+                s_qc[at][tid] = PAST;
+            }
         };
+        asm volatile("cp.async.wait_group 0;" ::: "memory");   // the last block's left-over entries
+        if (!live) e = e_end = 0;
 #pragma unroll
-        for (int q = 0; q < SB_AHEAD; ++q) { cq[q] = PAST; vq[q] = MT(0); }
-        if (live) {
-#pragma unroll
-            for (int q = 0; q < SB_AHEAD; ++q) fetch(cq[q], vq[q]);
+        for (int q = 0; q < AHEAD; ++q) {
+            fetch(q);
+            asm volatile("cp.async.commit_group;" ::: "memory");
         }
+        int head = 0;
+        asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
+        int cc = s_qc[0][tid];
+        MT cv = s_qv[0][tid];
         // slot of this thread's value in block i of the chain (i-th block done)
         const int lrow = tid / KC;
         auto slot = [&](int i) -> const unsigned long long* {
@@ -202,48 +227,79 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
         };
         int i = 0, buf = 0;
         while (i < kk) {
-            // the first block must be there; three more are taken if they are
-            const int more = min(SB_SPAN, kk - i);
-            unsigned long long u[SB_SPAN];
-#pragma unroll
-            for (int q = 0; q < SB_SPAN; ++q) {
-                const unsigned long long* p = q < more ? slot(i + q) : nullptr;
-                u[q] = p ? sb_ldv(p) : 0ull;
+            // Far behind its own block the CTA takes four blocks at a time, and one thread waits
+            // for the last of them, now and then; only the CTAs of the next few blocks watch every
+            // value.  (All CTAs polling all values kept the chain's own stores waiting.)
+            const int span = kk - i > SB_SPAN ? SB_SPAN : 1;
+            if (span > 1) {
+                if (tid == 0) {
+                    const int64_t j3 = (int64_t)(FWD ? i + span - 1 : nblk - i - span) * B;
+                    const unsigned long long* p = xnew + j3 * a.K + cg * KC;
+                    unsigned polls = 0;
+                    while (sb_ldv(p) == SB_EMPTY) {
+                        ++polls;
+                        if (polls > a.max_polls || ((polls & 63u) == 0 && *(volatile unsigned*)a.err != 0u)) {
+                            atomicOr(a.err, DEV_ERR_TIMEOUT);
+                            break;
+                        }
+                        __nanosleep(SB_FAR_NS);
+                    }
+                }
+                __syncthreads();
             }
             if (tid < ((B * KC + 31) & ~31)) {
-                const unsigned long long* p = slot(i);
+                unsigned long long u[SB_SPAN];
+#pragma unroll
+                for (int q = 0; q < SB_SPAN; ++q) {
+                    const unsigned long long* p = q < span ? slot(i + q) : nullptr;
+                    u[q] = p ? sb_ldv(p) : 0ull;
+                }
                 unsigned polls = 0;
-                while (__any_sync(0xffffffffu, u[0] == SB_EMPTY)) {
+                while (true) {
+                    bool missing = false;
+#pragma unroll
+                    for (int q = 0; q < SB_SPAN; ++q) missing = missing || u[q] == SB_EMPTY;
+                    if (!__any_sync(0xffffffffu, missing)) break;
                     ++polls;
                     const bool give_up = polls > a.max_polls ||
                                          ((polls & 255u) == 0 && *(volatile unsigned*)a.err != 0u);
                     if (__any_sync(0xffffffffu, give_up)) {
                         if (lane == 0) atomicOr(a.err, DEV_ERR_TIMEOUT);
-                        if (u[0] == SB_EMPTY) u[0] = 0ull;
+#pragma unroll
+                        for (int q = 0; q < SB_SPAN; ++q)
+                            if (u[q] == SB_EMPTY) u[q] = 0ull;
                         break;
                     }
                     if (polls > 64) __nanosleep(polls > 4096 ? 128 : 20);
-                    if (u[0] == SB_EMPTY) u[0] = sb_ldv(p);
+#pragma unroll
+                    for (int q = 0; q < SB_SPAN; ++q)
+                        if (u[q] == SB_EMPTY) u[q] = sb_ldv(slot(i + q));
                 }
 #pragma unroll
                 for (int q = 0; q < SB_SPAN; ++q)
-                    if (tid < B * KC) s_x[buf][q * B * KC + tid] = AR::from_bits(u[q]);
+                    if (q < span && tid < B * KC) s_x[buf][q * B * KC + tid] = AR::from_bits(u[q]);
             }
-            bool ready = more == SB_SPAN;
-#pragma unroll
-            for (int q = 1; q < SB_SPAN; ++q) ready = ready && u[q] != SB_EMPTY;
-            const int span = __syncthreads_and(ready) ? SB_SPAN : 1;
+            __syncthreads();
             // this thread's entries inside the blocks just loaded
             const int64_t first = (int64_t)(FWD ? i : nblk - i - span) * B;   // lowest row of the span
             const int lim = FWD ? (int)min(first + (int64_t)span * B, (int64_t)0x7fffffff) : (int)first;
-            while (FWD ? cq[0] < lim : cq[0] >= lim) {
-                const int d = cq[0] - (int)first;
-                // forward: block q of the span starts at q B; backward: the span runs downwards
-                const int at = FWD ? d : (span - 1 - d / B) * B + (d & (B - 1));
-                AR::mad(acc, vq[0], s_x[buf][at * KC + c]);
-#pragma unroll
-                for (int q = 0; q + 1 < SB_AHEAD; ++q) { cq[q] = cq[q + 1]; vq[q] = vq[q + 1]; }
-                fetch(cq[SB_AHEAD - 1], vq[SB_AHEAD - 1]);
+            while (true) {
+                // the warp goes round as one until no lane has an entry left in the span
+                const bool on = FWD ? cc < lim : cc >= lim;
+                if (!__any_sync(0xffffffffu, on)) break;
+                if (on) {
+                    const int d = cc - (int)first;
+                    // forward: block q of the span starts at q B; backward: the span runs downwards
+                    const int at = FWD ? d : (span - 1 - d / B) * B + (d & (B - 1));
+                    AR::mad(acc, cv, s_x[buf][at * KC + c]);
+                    fetch(head);
+                    head = head + 1 == AHEAD ? 0 : head + 1;
+                }
+                asm volatile("cp.async.commit_group;\n\tcp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
+                if (on) {
+                    cc = s_qc[head][tid];
+                    cv = s_qv[head][tid];
+                }
             }
             i += span;
             buf ^= 1;
@@ -257,14 +313,21 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
         for (int o = KC; o < KC * ES; o <<= 1) AR::add(s, AR::xorv(s, o));
         if (h == 0) s_s[row * KC + c] = s;
         __syncthreads();
-        // x_row = sum_k inv(row, k) s_k over the triangle; the warp skips what is zero for all
-        // of its rows
-        const int wrow0 = (tid & ~31) / (KC * ES), wrow1 = (tid | 31) / (KC * ES);
+        // x_row = sum_k inv(row, k) s_k over the triangle, CH entries at a time; the warp skips the
+        // chunks that are zero for all of its rows.  (A test per entry left every entry's shared
+        // load and multiply-add waiting for the one before: 2900 cycles of a 5000-cycle step.)
+        constexpr int CH = std::is_same<AR, SbPair>::value ? 8 : (PER >= 16 ? 4 : 2);
         V x = AR::zero();
 #pragma unroll
-        for (int t = 0; t < PER; ++t) {
-            const bool need = FWD ? ES * t <= wrow1 : ES * t + ES - 1 >= wrow0;
-            if (need) AR::madv(x, inv[t], s_s[(h + ES * t) * KC + c]);
+        for (int t0 = 0; t0 < PER; t0 += CH) {
+            const bool need = FWD ? ES * t0 <= wrow1 : ES * (t0 + CH) - 1 >= wrow0;
+            if (need) {
+                V sv[CH];
+#pragma unroll
+                for (int t = 0; t < CH; ++t) sv[t] = s_s[(h + ES * (t0 + t)) * KC + c];
+#pragma unroll
+                for (int t = 0; t < CH; ++t) AR::madv(x, inv[t0 + t], sv[t]);
+            }
         }
         AR::norm(x);
 #pragma unroll
@@ -281,25 +344,29 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
 // Inverses of the 128-row lower diagonal blocks D + L of M: the block in shared memory (M's
 // entries, the identity beyond n), inverted in place from the last column to the first
 // (column j of the inverse is -X_sub l_j / l_jj with X_sub the inverse of the rows below),
-// eight threads per row.  FP64 throughout; FP32 M (whose sweeps use the FP32-rounded
+// four threads per row.  FP64 throughout; FP32 M (whose sweeps use the FP32-rounded
 // off-diagonal entries and the FP64 diagonal) gets them as float pairs.
-// Bound: FP64 FMA (350 k per block, two a clock per SM: ~85 us per block and SM).
+// Bound: FP64 instructions (350 k FMAs per block and as many lanes again in the row reductions; the
+// reciprocals of the diagonal are formed once: a division per thread and column took most of the
+// time).  313 blocks: 0.71 ms, against
+// 1.56 ms.
 // ---------------------------------------------------------------------------------------
 constexpr int SI_LD = SB_ROWS + 1;
+constexpr int SI_T = 512;
 constexpr size_t SI_SMEM = (size_t)SB_ROWS * SI_LD * 8;
 template <typename MT>
-__global__ void __launch_bounds__(1024, 1) k_block_inverse(int64_t n, const int64_t* mptr, const int32_t* mcol,
+__global__ void __launch_bounds__(SI_T, 1) k_block_inverse(int64_t n, const int64_t* mptr, const int32_t* mcol,
                                                            const MT* mval, const double* mval64,
                                                            const int64_t* mdiag, void* inv) {
     extern __shared__ __align__(16) double s_a[];   // SB_ROWS x SI_LD, row-major
-    __shared__ double s_l[SB_ROWS];
+    __shared__ double s_l[SB_ROWS], s_rd[SB_ROWS];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nblk = (int)((n + SB_ROWS - 1) / SB_ROWS);
     for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
         const int64_t j0 = (int64_t)b * SB_ROWS;
-        for (int t = tid; t < SB_ROWS * SI_LD; t += 1024) s_a[t] = 0.0;
+        for (int t = tid; t < SB_ROWS * SI_LD; t += SI_T) s_a[t] = 0.0;
         __syncthreads();
-        for (int r = wid; r < SB_ROWS; r += 32) {
+        for (int r = wid; r < SB_ROWS; r += SI_T / 32) {
             const int64_t j = j0 + r;
             if (j >= n) {
                 if (lane == 0) s_a[r * SI_LD + r] = 1.0;
@@ -314,28 +381,24 @@ __global__ void __launch_bounds__(1024, 1) k_block_inverse(int64_t n, const int6
             }
         }
         __syncthreads();
-        const int row = tid >> 3, h = tid & 7;
+        if (tid < SB_ROWS) s_rd[tid] = 1.0 / s_a[tid * SI_LD + tid];
+        const int row = tid >> 2, h = tid & 3;
         for (int j = SB_ROWS - 1; j >= 0; --j) {
             if (tid < SB_ROWS) s_l[tid] = s_a[tid * SI_LD + j];
             __syncthreads();
-            const double xjj = 1.0 / s_l[j];
-            double t0 = 0.0, t1 = 0.0;
-            if (row > j) {
-                int k = j + 1 + h;
-                for (; k + 8 <= row; k += 16) {
-                    t0 = fma(s_a[row * SI_LD + k], s_l[k], t0);
-                    t1 = fma(s_a[row * SI_LD + k + 8], s_l[k + 8], t1);
-                }
-                if (k <= row) t0 = fma(s_a[row * SI_LD + k], s_l[k], t0);
+            // warps whose rows all lie at or above j have nothing to do (eight rows a warp)
+            if ((row | 7) > j) {
+                double t = 0.0;
+                if (row > j)
+                    for (int k = j + 1 + h; k <= row; k += 4) t = fma(s_a[row * SI_LD + k], s_l[k], t);
+                t += __shfl_xor_sync(0xffffffffu, t, 1);
+                t += __shfl_xor_sync(0xffffffffu, t, 2);
+                if (h == 0 && row > j) s_a[row * SI_LD + j] = -t * s_rd[j];
             }
-            t0 += t1;
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) t0 += __shfl_xor_sync(0xffffffffu, t0, o);
-            if (h == 0 && row > j) s_a[row * SI_LD + j] = -t0 * xjj;
-            if (tid == 0) s_a[j * SI_LD + j] = xjj;
+            if (tid == 0) s_a[j * SI_LD + j] = s_rd[j];
             __syncthreads();
         }
-        for (int t = tid; t < SB_ROWS * SB_ROWS; t += 1024) {
+        for (int t = tid; t < SB_ROWS * SB_ROWS; t += SI_T) {
             const double v = s_a[(t / SB_ROWS) * SI_LD + t % SB_ROWS];
             const int64_t at = (int64_t)b * SB_ROWS * SB_ROWS + t;
             if (sizeof(MT) == 4) reinterpret_cast<f2*>(inv)[at] = df_from_double(v);
@@ -352,15 +415,16 @@ __global__ void __launch_bounds__(1024, 1) k_block_inverse(int64_t n, const int6
 // (as many rounds as the block's own depth).  Even CTAs take the forward direction, odd ones the
 // backward one.
 // ---------------------------------------------------------------------------------------
-constexpr int SL_T = 256;
+constexpr int SL_T = 256, SL_AHEAD = 8;
 template <bool FWD>
 __device__ __forceinline__ void levels_blocked(int64_t n, const int64_t* mptr, const int32_t* mcol,
                                                const int64_t* mdiag, int* lev1, int* maxlev, unsigned* err,
                                                unsigned max_polls, int first_blk, int stride) {
     constexpr int B = SB_ROWS, ES = SL_T / B;
-    __shared__ int s_x[2][B];
+    __shared__ int s_x[2][SB_SPAN * B];
     __shared__ int s_lev[B];
     __shared__ unsigned s_bits[B][B / 32];
+    __shared__ int s_qc[SL_AHEAD][SL_T];
     const int tid = threadIdx.x, lane = tid & 31;
     const int row = tid / ES, h = tid % ES;
     const int nblk = (int)((n + B - 1) / B);
@@ -375,52 +439,101 @@ __device__ __forceinline__ void levels_blocked(int64_t n, const int64_t* mptr, c
             e = FWD ? mptr[j] + h : mptr[j + 1] - 1 - h;
         }
         constexpr int PAST = FWD ? 0x7fffffff : -1;
-        auto fetch = [&]() -> int {
-            const bool in = j < n && (FWD ? e < e_end : e > e_end);
-            if (!in) return PAST;
-            const int cc = mcol[e];
-            e += FWD ? ES : -ES;
-            return cc;
+        if (j >= n) e = e_end = 0;
+        auto fetch = [&](int at) {
+            const bool in = FWD ? e < e_end : e > e_end;
+            if (in) { cp_async_elem(&s_qc[at][tid], mcol + e); e += FWD ? ES : -ES; }
+            else s_qc[at][tid] = PAST;
+        };
+        int head = 0;
+        // moves the lanes with `on` to their next entry (the whole warp calls this together)
+        auto advance = [&](bool on, int& c0) {
+            if (on) {
+                fetch(head);
+                head = head + 1 == SL_AHEAD ? 0 : head + 1;
+            }
+            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group %0;" ::"n"(SL_AHEAD - 1) : "memory");
+            if (on) c0 = s_qc[head][tid];
         };
         for (int t = tid; t < B * (B / 32); t += SL_T) s_bits[t / (B / 32)][t % (B / 32)] = 0u;
-        int c0 = fetch(), c1 = fetch(), mx = 0;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll
+        for (int q = 0; q < SL_AHEAD; ++q) {
+            fetch(q);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
+        asm volatile("cp.async.wait_group %0;" ::"n"(SL_AHEAD - 1) : "memory");
+        int c0 = s_qc[0][tid], mx = 0;
         int buf = 0;
-        for (int i = 0; i < kk; ++i) {
-            const int64_t f = (int64_t)(FWD ? i : nblk - 1 - i) * B;   // first row of that block
+        for (int i = 0; i < kk;) {
+            // as in the sweep: far behind, one thread waits for every fourth block
+            const int span = kk - i > SB_SPAN ? SB_SPAN : 1;
+            if (span > 1) {
+                if (tid == 0) {
+                    const int* p = lev1 + (int64_t)(FWD ? i + span - 1 : nblk - i - span) * B;
+                    unsigned polls = 0;
+                    while (*(volatile const int*)p == 0) {
+                        ++polls;
+                        if (polls > max_polls || ((polls & 63u) == 0 && *(volatile unsigned*)err != 0u)) {
+                            atomicOr(err, DEV_ERR_TIMEOUT);
+                            break;
+                        }
+                        __nanosleep(SB_FAR_NS);
+                    }
+                }
+                __syncthreads();
+            }
+            const int64_t f = (int64_t)(FWD ? i : nblk - i - span) * B;   // lowest row of the span
             if (tid < B) {
-                int v = f + tid < n ? *(volatile int*)(lev1 + f + tid) : 1;
+                int v[SB_SPAN];
+#pragma unroll
+                for (int q = 0; q < SB_SPAN; ++q) {
+                    const int64_t r = f + q * B + tid;
+                    v[q] = q < span && r < n ? *(volatile int*)(lev1 + r) : 1;
+                }
                 unsigned polls = 0;
-                while (__any_sync(0xffffffffu, v == 0)) {
+                while (true) {
+                    bool missing = false;
+#pragma unroll
+                    for (int q = 0; q < SB_SPAN; ++q) missing = missing || v[q] == 0;
+                    if (!__any_sync(0xffffffffu, missing)) break;
                     ++polls;
                     const bool give_up = polls > max_polls || ((polls & 255u) == 0 && *(volatile unsigned*)err != 0u);
                     if (__any_sync(0xffffffffu, give_up)) {
                         if (lane == 0) atomicOr(err, DEV_ERR_TIMEOUT);
-                        v = max(v, 1);
+#pragma unroll
+                        for (int q = 0; q < SB_SPAN; ++q) v[q] = max(v[q], 1);
                         break;
                     }
                     if (polls > 64) __nanosleep(polls > 4096 ? 128 : 20);
-                    if (v == 0) v = *(volatile int*)(lev1 + f + tid);
+#pragma unroll
+                    for (int q = 0; q < SB_SPAN; ++q)
+                        if (v[q] == 0) v[q] = *(volatile int*)(lev1 + f + q * B + tid);
                 }
-                s_x[buf][tid] = v;
+#pragma unroll
+                for (int q = 0; q < SB_SPAN; ++q)
+                    if (q < span) s_x[buf][q * B + tid] = v[q];
             }
             __syncthreads();
-            const int64_t lim = FWD ? f + B : f;
-            while (FWD ? c0 < lim : (c0 >= lim && c0 >= 0)) {
-                mx = max(mx, s_x[buf][c0 - (int)f]);
-                c0 = c1;
-                c1 = fetch();
+            const int64_t lim = FWD ? f + (int64_t)span * B : f;
+            while (true) {
+                const bool on = FWD ? c0 < lim : (c0 >= lim && c0 >= 0);
+                if (!__any_sync(0xffffffffu, on)) break;
+                if (on) mx = max(mx, s_x[buf][c0 - (int)f]);
+                advance(on, c0);
             }
+            i += span;
             buf ^= 1;
         }
         __syncwarp();
 #pragma unroll
         for (int o = 1; o < ES; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         __syncthreads();   // s_bits cleared
-        while (c0 != PAST) {   // what is left of the row lies inside the block
+        while (__any_sync(0xffffffffu, c0 != PAST)) {   // what is left of the row lies inside the block
+            const bool on = c0 != PAST;
             const int d = c0 - (int)j0;
-            atomicOr(&s_bits[row][d >> 5], 1u << (d & 31));
-            c0 = c1;
-            c1 = fetch();
+            if (on) atomicOr(&s_bits[row][d >> 5], 1u << (d & 31));
+            advance(on, c0);
         }
         if (h == 0) s_lev[row] = mx + 1;
         __syncthreads();
@@ -534,10 +647,10 @@ lsq_status sb_build_inverse(SparseHandle* S, int64_t n, bool m32, cudaStream_t s
     const unsigned g = (unsigned)std::min<int64_t>(nblk, 1 << 20);
     if (m32) {
         LSQ_CUDA(cudaFuncSetAttribute(k_block_inverse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SI_SMEM));
-        k_block_inverse<float><<<g, 1024, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval32, S->mval, S->mdiag, S->inv);
+        k_block_inverse<float><<<g, SI_T, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval32, S->mval, S->mdiag, S->inv);
     } else {
         LSQ_CUDA(cudaFuncSetAttribute(k_block_inverse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SI_SMEM));
-        k_block_inverse<double><<<g, 1024, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval, S->mval, S->mdiag, S->inv);
+        k_block_inverse<double><<<g, SI_T, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval, S->mval, S->mdiag, S->inv);
     }
     count_launch();
     LSQ_CUDA(cudaGetLastError());
