@@ -1243,38 +1243,96 @@ lsq_status sparse_apply(const lsq_precond* P, const double* r, double* e, int64_
     return LSQ_OK;
 }
 
-// grad_b = A lambda, r = b - A x and grad_vals[e] = sum_c r_i lambda_j - (A lambda)_i x_j
-template <int DT>
-__global__ void k_csr_rowdot(int64_t m, const int64_t* rp, const int32_t* ci, const void* vals,
-                             const double* v, const double* b, double sb, double sa, double* out) {
-    const int sub = threadIdx.x & 7;
-    const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-    const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) >> 3;
+// Up to GK columns of the adjoint's products in one pass over A: a group of GK lanes per row, lane
+// c its column c.  The row's products A lambda and r = b - A x come first (lambda and x row-major,
+// so a group gathers one line per entry), then grad[e] (+)= sum_c r_c lambda_jc - (A lambda)_c x_jc
+// for the row's entries, eight at a time: their sums over the group share one reduce-scatter.
+// Bound: FP64 operations, five per entry and column.  1e6 x 10,000 with 16 columns, FP32 values:
+// 1.24 ms, against 6.3 ms by two products per column and a pass over all columns.
+constexpr int AJ_E = 8;
+template <int DT, int GK>
+__global__ void __launch_bounds__(SP_T) k_csr_adjoint(int64_t m, const int64_t* rp, const int32_t* ci, const void* vals,
+                                                      const double* lam, const double* x, int kc, const double* b,
+                                                      int64_t ldb, double* al_out, double* grad, int accumulate) {
+    const int c = threadIdx.x & (GK - 1);
+    const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / GK;
+    const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) / GK;
+    const bool on = c < kc;
+    // one batch of the row's entries: columns, values, and this lane's lambda and x
+    auto batch = [&](int64_t e, int64_t e1, int32_t (&col)[AJ_E], double (&lv)[AJ_E], double (&xv)[AJ_E]) {
+#pragma unroll
+        for (int u = 0; u < AJ_E; ++u) col[u] = e + u < e1 ? ci[e + u] : -1;
+#pragma unroll
+        for (int u = 0; u < AJ_E; ++u) {
+            const bool in = col[u] >= 0 && on;
+            lv[u] = in ? lam[(int64_t)col[u] * kc + c] : 0.0;
+            xv[u] = in ? x[(int64_t)col[u] * kc + c] : 0.0;
+        }
+    };
+    // the trip count is the same for every group of a warp (the shuffles need all 32 lanes)
     for (int64_t i0 = 0; i0 < m; i0 += ngrp) {
         const int64_t i = i0 + grp;
-        double t = 0.0;
-        if (i < m)
-            for (int64_t e = rp[i] + sub; e < rp[i + 1]; e += 8) t = fma(Val<DT>::load(vals, e), v[ci[e]], t);
+        const int64_t e0 = i < m ? rp[i] : 0, e1 = i < m ? rp[i + 1] : 0;
+        int32_t col[AJ_E];
+        double lv[AJ_E], xv[AJ_E];
+        double al = 0.0, ax = 0.0;
+        for (int64_t e = e0; e < e1; e += AJ_E) {
+            batch(e, e1, col, lv, xv);
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (i < m && sub == 0) out[i] = (b ? sb * b[i] : 0.0) + sa * t;
-    }
-}
-__global__ void k_sddmm_csr(int64_t m, const int64_t* rp, const int32_t* ci, int64_t kcols,
-                            const double* r, const double* al, int64_t ldm, const double* lam,
-                            const double* x, int64_t ldn, double* grad) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = warp; i < m; i += nw) {
-        for (int64_t e = rp[i] + lane; e < rp[i + 1]; e += 32) {
-            const int64_t j = ci[e];
-            double acc = 0.0;
-            for (int64_t c = 0; c < kcols; ++c)
-                acc += r[c * ldm + i] * lam[c * ldn + j] - al[c * ldm + i] * x[c * ldn + j];
-            grad[e] = acc;
+            for (int u = 0; u < AJ_E; ++u) {
+                if (col[u] >= 0) {
+                    const double v = Val<DT>::load(vals, e + u);
+                    al = fma(v, lv[u], al);
+                    ax = fma(v, xv[u], ax);
+                }
+            }
+        }
+        double r = 0.0;
+        if (i < m && on) {
+            r = b[(int64_t)c * ldb + i] - ax;
+            if (al_out) al_out[(int64_t)c * ldb + i] = al;
+        }
+        if (!grad) continue;
+        int64_t len = e1 - e0;   // the longest row of the warp sets the number of batches
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) len = max(len, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)len, o));
+        for (int64_t k0 = 0; k0 < len; k0 += AJ_E) {
+            const int64_t e = e0 + k0;
+            if (len > AJ_E) batch(e, e1, col, lv, xv);   // else still in registers
+            double t[AJ_E];
+#pragma unroll
+            for (int u = 0; u < AJ_E; ++u) t[u] = e + u < e1 ? r * lv[u] - al * xv[u] : 0.0;
+            int first = 0, hold = AJ_E;                   // this lane ends with entries first ... first + hold - 1
+#pragma unroll
+            for (int o = GK / 2; o > 0; o >>= 1) {
+                if (hold > 1) {
+                    hold >>= 1;
+                    const bool up = (c & o) != 0;
+#pragma unroll
+                    for (int u = 0; u < AJ_E / 2; ++u) {
+                        if (u < hold) {
+                            const double send = up ? t[u] : t[u + hold];
+                            const double keep = up ? t[u + hold] : t[u];
+                            t[u] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                        }
+                    }
+                    if (up) first += hold;
+                } else {
+                    t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+                }
+            }
+            constexpr int KEEP = GK >= AJ_E ? 1 : AJ_E / GK;      // entries a lane is left with
+            const bool writer = GK <= AJ_E || (c & (GK / AJ_E - 1)) == 0;
+#pragma unroll
+            for (int u = 0; u < KEEP; ++u)
+                if (writer && e + first + u < e1) grad[e + first + u] = accumulate ? grad[e + first + u] + t[u] : t[u];
         }
     }
+}
+// column-major (leading dimension ld) -> row-major n x kc
+__global__ void k_cols_to_rows(const double* src, int64_t ld, int64_t n, int kc, double* dst) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * kc; t += (int64_t)gridDim.x * blockDim.x)
+        dst[t] = src[(t % kc) * ld + t / kc];
 }
 __global__ void k_scale_into(const double* src, int64_t lds, const double* s, double* dst, int64_t n, int64_t kcols) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * kcols; t += (int64_t)gridDim.x * blockDim.x) {
@@ -1290,27 +1348,37 @@ static lsq_status sp_adjoint_impl(const lsq_matrix* A, const lsq_precond* P, con
                                   cudaStream_t st) {
     const int64_t m = A->m, n = A->n;
     Scratch sc;
-    LSQ_CUDA(sc.alloc(8 * (size_t)(2 * n * k + 2 * m * k) + 256, st));
+    LSQ_CUDA(sc.alloc(8 * (size_t)(2 * n * k + 32 * n) + 256, st));
     double* h = sc.as<double>();
     double* lam = h + n * k;
-    double* r = lam + n * k;
-    double* al = r + m * k;
+    double* lamr = lam + n * k;   // 16 columns of lambda and x, row-major
+    double* xr = lamr + 16 * n;
     k_scale_into<<<gridn(n * k), SP_T, 0, st>>>(G, ldx, P->inv_d, h, n, k);
     count_launch();
     // A^T A lambda = G  <=>  Â^T Â mu = D^{-1} G, lambda = D^{-1} mu (the solver's output)
     lsq_status s = sparse_solve(A, P, nullptr, h, k, n, lam, n, o, info, st);
     if (s != LSQ_OK && s != LSQ_ERR_NOT_CONVERGED) return s;
-    const void* vals = A->vals;
-    for (int64_t c = 0; c < k; ++c) {
-        k_csr_rowdot<DT><<<gridn(m * 8), SP_T, 0, st>>>(m, A->row_ptr, A->col_idx, vals, lam + c * n, nullptr, 0.0, 1.0, al + c * m);
-        k_csr_rowdot<DT><<<gridn(m * 8), SP_T, 0, st>>>(m, A->row_ptr, A->col_idx, vals, X + c * ldx, B + c * ldb, 1.0, -1.0, r + c * m);
-        count_launch(2);
-        if (grad_b) LSQ_CUDA(cudaMemcpyAsync(grad_b + c * ldb, al + c * m, 8 * (size_t)m, cudaMemcpyDeviceToDevice, st));
-        if (Lambda) LSQ_CUDA(cudaMemcpyAsync(Lambda + c * ldx, lam + c * n, 8 * (size_t)n, cudaMemcpyDeviceToDevice, st));
-    }
-    if (grad_vals) {
-        k_sddmm_csr<<<gridn(m * 32), SP_T, 0, st>>>(m, A->row_ptr, A->col_idx, k, r, al, m, lam, X, ldx, grad_vals);
-        count_launch();
+    for (int64_t c = 0; c < k; c += 16) {
+        const int kc = (int)std::min<int64_t>(16, k - c);
+        double* gb = grad_b ? grad_b + c * ldb : nullptr;
+        if (gb || grad_vals) {
+            k_cols_to_rows<<<gridn(n * kc), SP_T, 0, st>>>(lam + c * n, n, n, kc, lamr);
+            k_cols_to_rows<<<gridn(n * kc), SP_T, 0, st>>>(X + c * ldx, ldx, n, kc, xr);
+            const double* Bc = B + c * ldb;
+            const int more = c > 0 ? 1 : 0;
+            auto pass = [&](auto kern, int gk) {
+                kern<<<gridn(m * gk, 152 * 16), SP_T, 0, st>>>(m, A->row_ptr, A->col_idx, A->vals, lamr, xr, kc, Bc, ldb,
+                                                               gb, grad_vals, more);
+            };
+            if (kc <= 2) pass(k_csr_adjoint<DT, 2>, 2);
+            else if (kc <= 4) pass(k_csr_adjoint<DT, 4>, 4);
+            else if (kc <= 8) pass(k_csr_adjoint<DT, 8>, 8);
+            else pass(k_csr_adjoint<DT, 16>, 16);
+            count_launch(3);
+        }
+        if (Lambda)
+            for (int q = 0; q < kc; ++q)
+                LSQ_CUDA(cudaMemcpyAsync(Lambda + (c + q) * ldx, lam + (c + q) * n, 8 * (size_t)n, cudaMemcpyDeviceToDevice, st));
     }
     LSQ_CUDA(cudaGetLastError());
     LSQ_CUDA(cudaStreamSynchronize(st));
