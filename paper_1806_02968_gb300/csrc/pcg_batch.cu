@@ -17,6 +17,13 @@
 // scalars are FP64.  Restarts (outer steps) recompute g from the residual D^{-1} A^T (b - A x)
 // in double-float on the FP32 units (about 48 bits; A's values are exact in FP32), which also
 // refines x.
+// Bound: the largest problem's cluster (the FP32 passes' shared-memory reads and the double-float
+// products).  What stood beside them were FP64 instructions, each of which holds a scheduler for ~64
+// cycles, and barriers: one lane in four ended all columns of a row of Q, so the warp paid the
+// conversions and the subtraction once per column (now every lane ends one column, once per warp), a
+// column's partial sums were one chain of 32 FP64 additions (now four warps), the padding of A was
+// cleared by an extra pass and barrier per tile (now masked as it is read), and the first residual
+// multiplied A by zero.  64 problems up to 11803 x 255 with 16 columns: 12.70 -> 9.60 ms.
 // Every decision (alpha, masks, loop exits) is computed identically by all CTAs of a cluster
 // from the same sums in the same order, so their control flow cannot diverge.
 #include "batch.cuh"
@@ -64,9 +71,27 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 
-// Rows [r_lo, r_hi) of problem P, KC columns, arithmetic type T (float: inner iteration;
-// double: FP64 residual):
-//   Q = A X          (mode 0)   or   Q = b - A X   (mode 1, T = double)
+// A's padding columns n..npad-1 may hold anything: they enter no dot product (what they put into W
+// belongs to rows j >= n, which nothing reads)
+__device__ __forceinline__ void bt_mask_padding(float (&av)[4], int col, int n) {
+    if (col + 4 > n) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (col + u >= n) av[u] = 0.f;
+    }
+}
+// v[i] for a lane-dependent i without local memory
+template <typename V, int N>
+__device__ __forceinline__ V bt_pick(const V (&v)[N], int i) {
+    V r = v[0];
+#pragma unroll
+    for (int k = 1; k < N; ++k)
+        if (i == k) r = v[k];
+    return r;
+}
+
+// Rows [r_lo, r_hi) of problem P, KC columns, arithmetic type T (float: inner iteration):
+//   Q = A X
 //   Wp = A^T Q over these rows, qq_out[c] = sum of Q_ic^2 over these rows (c < k)
 // X (npad x KC, rows j >= n zero) is in shared memory.  Tiles of BR rows are streamed with
 // cp.async into two buffers; the next tile is in flight while the current one is used.
@@ -74,7 +99,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // shuffles.  W step: a thread owns 4 consecutive j and CQ columns (RS threads split the rows
 // when there are fewer such units than threads) and accumulates over all tiles in registers.
 template <int KC, typename T>
-__device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int mode, int k,
+__device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int k,
                             float* As, const T* Xs, T* Qs, T* Wp, double* qq_out, double* red) {
     constexpr int CQ = KC < 4 ? KC : 4;
     constexpr int CG = KC / CQ;
@@ -94,9 +119,7 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
 #pragma unroll
         for (int c = 0; c < CQ; ++c) acc[u][c] = T(0);
     // ||Q||^2 in double-float on the FP32 units (the FP64 pipe runs at 1/64 of their rate)
-    f2 qq[CQ];
-#pragma unroll
-    for (int c = 0; c < CQ; ++c) qq[c] = f2{0.f, 0.f};
+    f2 qq{0.f, 0.f};   // this lane's column of its row group
     const int qr = tid / TPR, qsub = tid % TPR, qcg = qsub % CG, qjs = qsub / CG;
 
     auto load_tile = [&](int t, int buf) {
@@ -116,18 +139,14 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
         __syncthreads();   // tile t has landed; every thread is done with tile t-1
         if (t + 1 < ntile) load_tile(t + 1, (t + 1) & 1);
         float* At = As + (t & 1) * BR * LDS;
-        if (n < npad) {    // A's padding columns n..npad-1 may hold anything
-            const int pw = npad - n;
-            for (int q = tid; q < BR * pw; q += BT) At[(q / pw) * LDS + n + q % pw] = 0.f;
-            __syncthreads();
-        }
         {   // Q step
             T sacc[CQ];
 #pragma unroll
             for (int c = 0; c < CQ; ++c) sacc[c] = T(0);
             for (int ch = qjs; ch < nch; ch += JS) {
                 const float4 a4 = *reinterpret_cast<const float4*>(At + qr * LDS + 4 * ch);
-                const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+                float av[4] = {a4.x, a4.y, a4.z, a4.w};
+                bt_mask_padding(av, 4 * ch, n);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const T* xr = Xs + (4 * ch + u) * XPitch<KC>::v + qcg * CQ;
@@ -147,20 +166,16 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
             for (int o = CG; o < TPR; o <<= 1)
 #pragma unroll
                 for (int c = 0; c < CQ; ++c) sacc[c] += __shfl_xor_sync(0xffffffffu, sacc[c], o);
-            if (qjs == 0) {
+            // every lane of the row holds the totals: lane qjs takes column qjs
+            if (qjs < CQ) {
                 const int64_t i = r_lo + (int64_t)t * BR + qr;
-                const bool ok = i < r_hi;
-#pragma unroll
-                for (int cc = 0; cc < CQ; ++cc) {
-                    const int c = qcg * CQ + cc;
-                    T q = T(0);
-                    if (ok && c < k) {
-                        q = sacc[cc];
-                        if (mode == 1) q = (T)(P.B[(int64_t)c * P.ldb + i] - (double)sacc[cc]);
-                        df_add_sq(qq[cc], (float)q);
-                    }
-                    Qs[qr * KC + c] = q;
+                const int c = qcg * CQ + qjs;
+                T q = T(0);
+                if (i < r_hi && c < k) {
+                    q = bt_pick(sacc, qjs);
+                    df_add_sq(qq, (float)q);
                 }
+                Qs[qr * KC + c] = q;
             }
         }
         __syncthreads();
@@ -192,15 +207,12 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
         }
         __syncthreads();
     }
-    // ||Q||^2 per column: the js == 0 threads of every tile row, in row order
-#pragma unroll
-    for (int c = 0; c < CQ; ++c) red[tid * CQ + c] = (qjs == 0) ? df_to_double(qq[c]) : 0.0;
+    // ||Q||^2 per column: the tile rows' sums, a warp per column
+    red[tid] = qjs < CQ ? df_to_double(qq) : 0.0;
     __syncthreads();
-    if (tid < KC) {
-        const int g = tid / CQ, cc = tid % CQ;
-        double sum = 0.0;
-        for (int r = 0; r < BR; ++r) sum += red[(r * TPR + g) * CQ + cc];
-        qq_out[tid] = sum;
+    for (int c = tid >> 5; c < KC; c += BT / 32) {
+        const double sum = warp_sum(red[(tid & 31) * TPR + (c % CQ) * CG + c / CQ]);
+        if ((tid & 31) == 0) qq_out[c] = sum;
     }
     __syncthreads();
 }
@@ -219,7 +231,7 @@ __device__ __forceinline__ void bt_cascade(f2& acc, float a, f2 x) {
     acc.lo += e + pe;
 }
 template <int KC>
-__device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int k, float* As,
+__device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int k, bool from_zero, float* As,
                                  const f2* Xs, f2* Qs, f2* Wp) {
     constexpr int CQ = KC < 4 ? KC : 4;
     constexpr int CG = KC / CQ;
@@ -256,18 +268,19 @@ __device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi,
         __syncthreads();
         if (t + 1 < ntile) load_tile(t + 1, (t + 1) & 1);
         float* At = As + (t & 1) * BR * LDS;
-        if (n < npad) {
-            const int pw = npad - n;
-            for (int q = tid; q < BR * pw; q += BT) At[(q / pw) * LDS + n + q % pw] = 0.f;
-            __syncthreads();
-        }
-        {   // Q = b - A x for this tile's rows
+        {   // Q = b - A x for this tile's rows (Q = b from x = 0)
+            const int64_t qi = r_lo + (int64_t)t * BR + qr;
+            const int qc = qcg * CQ + qjs;                  // the column this lane takes in the end
+            const bool mine = qjs < CQ && qi < r_hi && qc < k;
+            const double bq = mine ? P.B[(int64_t)qc * P.ldb + qi] : 0.0;
             f2 sacc[CQ];
 #pragma unroll
             for (int c = 0; c < CQ; ++c) sacc[c] = f2{0.f, 0.f};
+            if (!from_zero)
             for (int ch = qjs; ch < nch; ch += JS) {
                 const float4 a4 = *reinterpret_cast<const float4*>(At + qr * LDS + 4 * ch);
-                const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+                float av[4] = {a4.x, a4.y, a4.z, a4.w};
+                bt_mask_padding(av, 4 * ch, n);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const f2* xr = Xs + (4 * ch + u) * XPitch<KC>::v + qcg * CQ;
@@ -281,17 +294,9 @@ __device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi,
             for (int o = CG; o < TPR; o <<= 1)
 #pragma unroll
                 for (int c = 0; c < CQ; ++c) df_add(sacc[c], df_shfl_xor(sacc[c], o));
-            if (qjs == 0) {
-                const int64_t i = r_lo + (int64_t)t * BR + qr;
-                const bool ok = i < r_hi;
-#pragma unroll
-                for (int cc = 0; cc < CQ; ++cc) {
-                    const int c = qcg * CQ + cc;
-                    f2 q = f2{0.f, 0.f};
-                    if (ok && c < k) q = df_from_double(P.B[(int64_t)c * P.ldb + i] - df_to_double(sacc[cc]));
-                    Qs[qr * KC + c] = q;
-                }
-            }
+            // FP64 once per column and row: every lane holds the totals, lane qjs takes column qjs
+            if (qjs < CQ)
+                Qs[qr * KC + qc] = mine ? df_from_double(bq - df_to_double(bt_pick(sacc, qjs))) : f2{0.f, 0.f};
         }
         __syncthreads();
         if (wact) {   // W += A^T Q
@@ -359,15 +364,23 @@ __device__ __forceinline__ void bt_cluster_sum(cg::cluster_group& cl, BtState* S
 // column t % KC), written into slot `sl` in thread order.
 template <int KC>
 __device__ __forceinline__ void bt_slice_partials(double a, double b, BtState* S, int sl, double* red) {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     red[tid] = a;
     red[BT + tid] = b;
     __syncthreads();
-    if (tid < 2 * KC) {
-        const int which = tid / KC, c = tid % KC;
+    // four warps (one per scheduler) sum a quarter of every column each, one adds the quarters: a
+    // serial FP64 sum of a column takes ~64 cycles per term
+    constexpr int PER = BT / KC / 4;
+    const int which = lane / KC, c = lane % KC;
+    if (w < 4 && lane < 2 * KC) {
         double sum = 0.0;
-        for (int i = c; i < BT; i += KC) sum += red[which * BT + i];
-        S->slot[sl][which][c] = sum;
+        for (int i = 0; i < PER; ++i) sum += red[which * BT + c + KC * (w * PER + i)];
+        red[2 * BT + w * 32 + lane] = sum;
+    }
+    __syncthreads();
+    if (w == 0 && lane < 2 * KC) {
+        const double* q = red + 2 * BT + lane;
+        S->slot[sl][which][c] = (q[0] + q[32]) + (q[64] + q[96]);
     }
     __syncthreads();
 }
@@ -410,13 +423,14 @@ __device__ void bt_solve_problem(cg::cluster_group& cl, const BatchProb& P, int 
             Xp[j * XP + c] = df_from_double((!from_zero && j < n) ? __ldcg(y + e) * P.inv_d[j] : 0.0);
         }
         __syncthreads();
-        bt_residual_pass<KC>(P, r_lo, r_hi, k, As, Xp, Qp, Wpp);
+        bt_residual_pass<KC>(P, r_lo, r_hi, k, from_zero, As, Xp, Qp, Wpp);
         cl.sync();
         double a = 0.0, b = 0.0;
         for (int e = e_lo + tid; e < e_hi; e += BT) {
             const int j = e / KC;
             double sum = 0.0;
-            for (int r = 0; r < C; ++r) sum += df_to_double(cl.map_shared_rank(Wpp, r)[e]);
+            if (j < n)   // rows j >= n hold what A's padding made of them
+                for (int r = 0; r < C; ++r) sum += df_to_double(cl.map_shared_rank(Wpp, r)[e]);
             const double v = j < n ? sum * P.inv_d[j] : 0.0;
             dst[e] = v;
             a = fma(v, v, a);
@@ -440,9 +454,11 @@ __device__ void bt_solve_problem(cg::cluster_group& cl, const BatchProb& P, int 
                 float sacc = 0.f;
                 if (P.op_f32) {
                     const float* o = reinterpret_cast<const float*>(P.op) + (int64_t)j * n;
+#pragma unroll 8   // loads in flight: the sum itself stays one chain, as it was
                     for (int l = 0; l < n; ++l) sacc = fmaf(o[l], Xf[l * XP + c], sacc);
                 } else {
                     const double* o = reinterpret_cast<const double*>(P.op) + (int64_t)j * n;
+#pragma unroll 8
                     for (int l = 0; l < n; ++l) sacc = fmaf((float)o[l], Xf[l * XP + c], sacc);
                 }
                 zv = sacc;
@@ -528,7 +544,7 @@ __device__ void bt_solve_problem(cg::cluster_group& cl, const BatchProb& P, int 
         next_p(true);
         while (true) {
             // q = Â p, w = Â^T q (this CTA's rows), p^T w = ||q||^2
-            bt_row_pass<KC, float>(P, r_lo, r_hi, 0, k, As, Xf, Qf, Wf, S->qq, red);
+            bt_row_pass<KC, float>(P, r_lo, r_hi, k, As, Xf, Qf, Wf, S->qq, red);
             if (tid < KC) { S->slot[sl][0][tid] = S->qq[tid]; S->slot[sl][1][tid] = 0.0; }
             __syncthreads();
             cl.sync();
