@@ -20,7 +20,7 @@
 // Bound: the largest problem's cluster (the FP32 passes' shared-memory reads and the double-float
 // products).  What stood beside them were FP64 instructions, each of which holds a scheduler for ~64
 // cycles, and barriers: one lane in four ended all columns of a row of Q, so the warp paid the
-// conversions and the subtraction once per column (now every lane ends one column, once per warp), a
+// conversions and the subtraction once per column (now a thread ends one column of one row), a
 // column's partial sums were one chain of 32 FP64 additions (now four warps), the padding of A was
 // cleared by an extra pass and barrier per tile (now masked as it is read), and the first residual
 // multiplied A by zero.  64 problems up to 11803 x 255 with 16 columns: 12.70 -> 9.60 ms.
@@ -42,7 +42,7 @@ namespace lsq {
 
 constexpr int BT = 512;            // threads per CTA (16 warps; 128 registers each)
 constexpr int BR = 32;             // rows per tile
-constexpr int TPR = BT / BR;       // threads per tile row in the Q step (16)
+constexpr int JQ = 4;              // Q step: shares of the columns of A, each with BT / 32 / JQ = 4 warps of 8 rows
 constexpr int NPMAX = 256;         // largest padded n
 constexpr int LDS = NPMAX + 8;     // shared-memory pitch of a tile row (floats; 8 keeps
                                    // the float4 reads of 4 rows on distinct banks)
@@ -80,14 +80,102 @@ __device__ __forceinline__ void bt_mask_padding(float (&av)[4], int col, int n) 
             if (col + u >= n) av[u] = 0.f;
     }
 }
-// v[i] for a lane-dependent i without local memory
-template <typename V, int N>
-__device__ __forceinline__ V bt_pick(const V (&v)[N], int i) {
-    V r = v[0];
+// The 16-byte pieces of a tile that this thread copies, the same for every tile: row << 16 | piece, or -1
+template <int N>
+__device__ __forceinline__ void bt_tile_spots(int nch, int (&spot)[N]) {
 #pragma unroll
-    for (int k = 1; k < N; ++k)
-        if (i == k) r = v[k];
-    return r;
+    for (int u = 0; u < N; ++u) {
+        const int q = (int)threadIdx.x + u * BT;
+        spot[u] = q < BR * nch ? (q / nch) << 16 | q % nch : -1;
+    }
+}
+template <int N>
+__device__ __forceinline__ void bt_load_tile(const BatchProb& P, float* dst, int64_t r_lo, int64_t row0, int64_t r_hi,
+                                             int nch, const int (&spot)[N]) {
+#pragma unroll
+    for (int u = 0; u < N; ++u)
+        if (spot[u] >= 0) {
+            const int r = spot[u] >> 16, ch = spot[u] & 0xffff;
+            const int64_t i = row0 + r;
+            const bool ok = i < r_hi;
+            cp_async16(dst + r * LDS + 4 * ch, P.A + (ok ? i : r_lo) * P.ld + 4 * ch, ok);
+        }
+    cp_async_commit();
+}
+// (hi, lo) += a x in the cascaded Dot2 form of Ogita, Rump & Oishi
+__device__ __forceinline__ void bt_cascade(f2& acc, float a, f2 x) {
+    float p, pe;
+    two_prod(a, x.hi, p, pe);
+    pe = fmaf(a, x.lo, pe);
+    float s, e;
+    two_sum(acc.hi, p, s, e);
+    acc.hi = s;
+    acc.lo += e + pe;
+}
+__device__ __forceinline__ void bt_mac(float& s, float a, float x) { s = fmaf(a, x, s); }
+__device__ __forceinline__ void bt_mac(f2& s, float a, f2 x) { bt_cascade(s, a, x); }
+
+// A tile's products with X: part[share][row][column] for JQ shares of the columns of A, T = float or
+// (hi, lo) pairs.  Bound: shared-memory reads of X against the multiply-adds (16 per lane and chunk of four
+// columns at KC = 16).  A warp takes 8 rows of one share: a lane two rows, CQ columns and one in 8 / CG
+// of the chunks, so four rows share every read of X and each serves two: 6 wavefronts of reads for 8 cycles of
+// multiply-adds; two rows per warp and one per lane took 9 for 4.
+// 64 problems up to 11803 x 255 with 16 columns: 9.60 -> 8.81 ms (with the divisions of the tile loads
+// taken out of the loop).
+template <int KC, typename T>
+__device__ __forceinline__ void bt_q_products(const float* At, const T* Xs, int n, int nch, T* part) {
+    constexpr int CQ = KC < 4 ? KC : 4;
+    constexpr int CG = KC / CQ;
+    constexpr int JS = 8 / CG;
+    static_assert(BR == 32 && BT == 512 && JQ == 4, "four warps of eight rows for each share");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int cg = lane % CG, js = lane / CG % JS;
+    const int row = 8 * (w / JQ) + lane / 8;   // and row + 4
+    T acc[2][CQ];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int c = 0; c < CQ; ++c) acc[h][c] = T{};
+    for (int ch = (w % JQ) * JS + js; ch < nch; ch += JQ * JS) {
+        float av[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 a4 = *reinterpret_cast<const float4*>(At + (row + 4 * h) * LDS + 4 * ch);
+            av[h][0] = a4.x; av[h][1] = a4.y; av[h][2] = a4.z; av[h][3] = a4.w;
+            bt_mask_padding(av[h], 4 * ch, n);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const T* xr = Xs + (4 * ch + u) * XPitch<KC>::v + cg * CQ;
+            T xv[CQ];
+            if constexpr (CQ == 4 && sizeof(T) == 4) {
+                const float4 x4 = *reinterpret_cast<const float4*>(xr);
+                xv[0] = x4.x; xv[1] = x4.y; xv[2] = x4.z; xv[3] = x4.w;
+            } else {
+#pragma unroll
+                for (int c = 0; c < CQ; ++c) xv[c] = xr[c];
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int c = 0; c < CQ; ++c) bt_mac(acc[h][c], av[h][u], xv[c]);
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int c = 0; c < CQ; ++c) {
+            T v = acc[h][c];
+            if constexpr (sizeof(T) == 4) {
+#pragma unroll
+                for (int o = CG; o < 8; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            } else {
+                v = df_norm(v);
+#pragma unroll
+                for (int o = CG; o < 8; o <<= 1) df_add(v, df_shfl_xor(v, o));
+            }
+            if (js == 0) part[((w % JQ) * BR + row + 4 * h) * KC + cg * CQ + c] = v;
+        }
 }
 
 // Rows [r_lo, r_hi) of problem P, KC columns, arithmetic type T (float: inner iteration):
@@ -95,15 +183,13 @@ __device__ __forceinline__ V bt_pick(const V (&v)[N], int i) {
 //   Wp = A^T Q over these rows, qq_out[c] = sum of Q_ic^2 over these rows (c < k)
 // X (npad x KC, rows j >= n zero) is in shared memory.  Tiles of BR rows are streamed with
 // cp.async into two buffers; the next tile is in flight while the current one is used.
-// Q step: TPR threads per tile row, each CQ columns over a JS-th of the row, combined by
-// shuffles.  W step: a thread owns 4 consecutive j and CQ columns (RS threads split the rows
+// W step: a thread owns 4 consecutive j and CQ columns (RS threads split the rows
 // when there are fewer such units than threads) and accumulates over all tiles in registers.
 template <int KC, typename T>
 __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int k,
                             float* As, const T* Xs, T* Qs, T* Wp, double* qq_out, double* red) {
     constexpr int CQ = KC < 4 ? KC : 4;
     constexpr int CG = KC / CQ;
-    constexpr int JS = TPR / CG;
     const int tid = threadIdx.x;
     const int n = (int)P.n, npad = (int)P.npad, nch = npad / 4;
     const int64_t rows = r_hi > r_lo ? r_hi - r_lo : 0;
@@ -119,19 +205,11 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
 #pragma unroll
         for (int c = 0; c < CQ; ++c) acc[u][c] = T(0);
     // ||Q||^2 in double-float on the FP32 units (the FP64 pipe runs at 1/64 of their rate)
-    f2 qq{0.f, 0.f};   // this lane's column of its row group
-    const int qr = tid / TPR, qsub = tid % TPR, qcg = qsub % CG, qjs = qsub / CG;
-
+    f2 qq{0.f, 0.f};   // of this thread's tile row and column
+    int spot[NPMAX / 4 * BR / BT];
+    bt_tile_spots(nch, spot);
     auto load_tile = [&](int t, int buf) {
-        float* dst = As + buf * BR * LDS;
-        const int64_t row0 = r_lo + (int64_t)t * BR;
-        for (int q = tid; q < BR * nch; q += BT) {
-            const int r = q / nch, ch = q % nch;
-            const int64_t i = row0 + r;
-            const bool ok = i < r_hi;
-            cp_async16(dst + r * LDS + 4 * ch, P.A + (ok ? i : r_lo) * P.ld + 4 * ch, ok);
-        }
-        cp_async_commit();
+        bt_load_tile(P, As + buf * BR * LDS, r_lo, r_lo + (int64_t)t * BR, r_hi, nch, spot);
     };
     if (ntile > 0) load_tile(0, 0);
     for (int t = 0; t < ntile; ++t) {
@@ -139,44 +217,17 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
         __syncthreads();   // tile t has landed; every thread is done with tile t-1
         if (t + 1 < ntile) load_tile(t + 1, (t + 1) & 1);
         float* At = As + (t & 1) * BR * LDS;
-        {   // Q step
-            T sacc[CQ];
-#pragma unroll
-            for (int c = 0; c < CQ; ++c) sacc[c] = T(0);
-            for (int ch = qjs; ch < nch; ch += JS) {
-                const float4 a4 = *reinterpret_cast<const float4*>(At + qr * LDS + 4 * ch);
-                float av[4] = {a4.x, a4.y, a4.z, a4.w};
-                bt_mask_padding(av, 4 * ch, n);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const T* xr = Xs + (4 * ch + u) * XPitch<KC>::v + qcg * CQ;
-                    T xv[CQ];
-                    if constexpr (CQ == 4 && sizeof(T) == 4) {
-                        const float4 x4 = *reinterpret_cast<const float4*>(xr);
-                        xv[0] = x4.x; xv[1] = x4.y; xv[2] = x4.z; xv[3] = x4.w;
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < CQ; ++c) xv[c] = xr[c];
-                    }
-#pragma unroll
-                    for (int c = 0; c < CQ; ++c) sacc[c] = fma((T)av[u], xv[c], sacc[c]);
-                }
+        bt_q_products<KC, T>(At, Xs, n, nch, reinterpret_cast<T*>(red));
+        __syncthreads();
+        if (tid < BR * KC) {   // one tile row and column per thread
+            const int64_t i = r_lo + (int64_t)t * BR + tid / KC;
+            T q = T(0);
+            if (i < r_hi && tid % KC < k) {
+                const T* part = reinterpret_cast<const T*>(red) + tid;
+                q = (part[0] + part[BR * KC]) + (part[2 * BR * KC] + part[3 * BR * KC]);
+                df_add_sq(qq, q);
             }
-#pragma unroll
-            for (int o = CG; o < TPR; o <<= 1)
-#pragma unroll
-                for (int c = 0; c < CQ; ++c) sacc[c] += __shfl_xor_sync(0xffffffffu, sacc[c], o);
-            // every lane of the row holds the totals: lane qjs takes column qjs
-            if (qjs < CQ) {
-                const int64_t i = r_lo + (int64_t)t * BR + qr;
-                const int c = qcg * CQ + qjs;
-                T q = T(0);
-                if (i < r_hi && c < k) {
-                    q = bt_pick(sacc, qjs);
-                    df_add_sq(qq, (float)q);
-                }
-                Qs[qr * KC + c] = q;
-            }
+            Qs[tid] = q;
         }
         __syncthreads();
         if (wact) {   // W step
@@ -208,10 +259,10 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
         __syncthreads();
     }
     // ||Q||^2 per column: the tile rows' sums, a warp per column
-    red[tid] = qjs < CQ ? df_to_double(qq) : 0.0;
+    if (tid < BR * KC) red[tid] = df_to_double(qq);
     __syncthreads();
     for (int c = tid >> 5; c < KC; c += BT / 32) {
-        const double sum = warp_sum(red[(tid & 31) * TPR + (c % CQ) * CG + c / CQ]);
+        const double sum = warp_sum(red[(tid & 31) * KC + c]);
         if ((tid & 31) == 0) qq_out[c] = sum;
     }
     __syncthreads();
@@ -221,21 +272,11 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
 // in FP32; x and q are (hi, lo) float pairs; products and sums follow the cascaded Dot2 form
 // of Ogita, Rump & Oishi):  Q = b - A X, Wp = A^T Q over rows [r_lo, r_hi) (pairs), qq_out
 // unused.  Same tiling and thread roles as bt_row_pass.
-__device__ __forceinline__ void bt_cascade(f2& acc, float a, f2 x) {
-    float p, pe;
-    two_prod(a, x.hi, p, pe);
-    pe = fmaf(a, x.lo, pe);
-    float s, e;
-    two_sum(acc.hi, p, s, e);
-    acc.hi = s;
-    acc.lo += e + pe;
-}
 template <int KC>
 __device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int k, bool from_zero, float* As,
-                                 const f2* Xs, f2* Qs, f2* Wp) {
+                                 const f2* Xs, f2* Qs, f2* Wp, f2* red) {
     constexpr int CQ = KC < 4 ? KC : 4;
     constexpr int CG = KC / CQ;
-    constexpr int JS = TPR / CG;
     const int tid = threadIdx.x;
     const int n = (int)P.n, npad = (int)P.npad, nch = npad / 4;
     const int64_t rows = r_hi > r_lo ? r_hi - r_lo : 0;
@@ -250,17 +291,10 @@ __device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi,
     for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int c = 0; c < CQ; ++c) acc[u][c] = f2{0.f, 0.f};
-    const int qr = tid / TPR, qsub = tid % TPR, qcg = qsub % CG, qjs = qsub / CG;
+    int spot[NPMAX / 4 * BR / BT];
+    bt_tile_spots(nch, spot);
     auto load_tile = [&](int t, int buf) {
-        float* dst = As + buf * BR * LDS;
-        const int64_t row0 = r_lo + (int64_t)t * BR;
-        for (int q = tid; q < BR * nch; q += BT) {
-            const int r = q / nch, ch = q % nch;
-            const int64_t i = row0 + r;
-            const bool ok = i < r_hi;
-            cp_async16(dst + r * LDS + 4 * ch, P.A + (ok ? i : r_lo) * P.ld + 4 * ch, ok);
-        }
-        cp_async_commit();
+        bt_load_tile(P, As + buf * BR * LDS, r_lo, r_lo + (int64_t)t * BR, r_hi, nch, spot);
     };
     if (ntile > 0) load_tile(0, 0);
     for (int t = 0; t < ntile; ++t) {
@@ -268,35 +302,22 @@ __device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi,
         __syncthreads();
         if (t + 1 < ntile) load_tile(t + 1, (t + 1) & 1);
         float* At = As + (t & 1) * BR * LDS;
-        {   // Q = b - A x for this tile's rows (Q = b from x = 0)
-            const int64_t qi = r_lo + (int64_t)t * BR + qr;
-            const int qc = qcg * CQ + qjs;                  // the column this lane takes in the end
-            const bool mine = qjs < CQ && qi < r_hi && qc < k;
-            const double bq = mine ? P.B[(int64_t)qc * P.ldb + qi] : 0.0;
-            f2 sacc[CQ];
+        // Q = b - A x for this tile's rows (Q = b from x = 0): one tile row and column per thread
+        const int64_t qi = r_lo + (int64_t)t * BR + tid / KC;
+        const bool mine = tid < BR * KC && qi < r_hi && tid % KC < k;
+        const double bq = mine ? P.B[(int64_t)(tid % KC) * P.ldb + qi] : 0.0;
+        if (!from_zero) {
+            bt_q_products<KC, f2>(At, Xs, n, nch, red);
+            __syncthreads();
+        }
+        if (tid < BR * KC) {
+            f2 ax{0.f, 0.f};
+            if (!from_zero) {
+                ax = red[tid];
 #pragma unroll
-            for (int c = 0; c < CQ; ++c) sacc[c] = f2{0.f, 0.f};
-            if (!from_zero)
-            for (int ch = qjs; ch < nch; ch += JS) {
-                const float4 a4 = *reinterpret_cast<const float4*>(At + qr * LDS + 4 * ch);
-                float av[4] = {a4.x, a4.y, a4.z, a4.w};
-                bt_mask_padding(av, 4 * ch, n);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const f2* xr = Xs + (4 * ch + u) * XPitch<KC>::v + qcg * CQ;
-#pragma unroll
-                    for (int c = 0; c < CQ; ++c) bt_cascade(sacc[c], av[u], xr[c]);
-                }
+                for (int j = 1; j < JQ; ++j) df_add(ax, red[j * BR * KC + tid]);
             }
-#pragma unroll
-            for (int c = 0; c < CQ; ++c) sacc[c] = df_norm(sacc[c]);
-#pragma unroll
-            for (int o = CG; o < TPR; o <<= 1)
-#pragma unroll
-                for (int c = 0; c < CQ; ++c) df_add(sacc[c], df_shfl_xor(sacc[c], o));
-            // FP64 once per column and row: every lane holds the totals, lane qjs takes column qjs
-            if (qjs < CQ)
-                Qs[qr * KC + qc] = mine ? df_from_double(bq - df_to_double(bt_pick(sacc, qjs))) : f2{0.f, 0.f};
+            Qs[tid] = mine ? df_from_double(bq - df_to_double(ax)) : f2{0.f, 0.f};
         }
         __syncthreads();
         if (wact) {   // W += A^T Q
@@ -423,7 +444,7 @@ __device__ void bt_solve_problem(cg::cluster_group& cl, const BatchProb& P, int 
             Xp[j * XP + c] = df_from_double((!from_zero && j < n) ? __ldcg(y + e) * P.inv_d[j] : 0.0);
         }
         __syncthreads();
-        bt_residual_pass<KC>(P, r_lo, r_hi, k, from_zero, As, Xp, Qp, Wpp);
+        bt_residual_pass<KC>(P, r_lo, r_hi, k, from_zero, As, Xp, Qp, Wpp, reinterpret_cast<f2*>(red));
         cl.sync();
         double a = 0.0, b = 0.0;
         for (int e = e_lo + tid; e < e_hi; e += BT) {
