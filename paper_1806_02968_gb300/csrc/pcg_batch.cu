@@ -7,8 +7,8 @@
 // the problem's rows and meet at hardware cluster barriers, exchanging partial results through
 // distributed shared memory.  Per iteration (K = k columns advanced together, each with its
 // own alpha, beta, rho and convergence mask):
-//   row pass   every CTA streams its rows of A through shared memory (cp.async, double
-//              buffered) and computes Q = A P~ (P~ = D^{-1} P) then W += A^T Q on the tile,
+//   row pass   every CTA streams its rows of A through shared memory (cp.async, two or four
+//              tiles ahead) and computes Q = A P~ (P~ = D^{-1} P) then W += A^T Q on the tile,
 //              with ||Q||^2 = p^T w per column on the side
 //   cluster    CTA r sums its slice of W over the cluster (DSMEM, fixed order): alpha, y, g,
 //              ||g||^2; the masks; z = (materialised SGS operator) g on the slice; rho', beta,
@@ -17,8 +17,9 @@
 // scalars are FP64.  Restarts (outer steps) recompute g from the residual D^{-1} A^T (b - A x)
 // in double-float on the FP32 units (about 48 bits; A's values are exact in FP32), which also
 // refines x.
-// Bound: the largest problem's cluster (the FP32 passes' shared-memory reads and the double-float
-// products).  What stood beside them were FP64 instructions, each of which holds a scheduler for ~64
+// Bound: the double-float products of the residual passes and the FP32 passes, about half of the cycles
+// each, added over the problems of a cluster (16 of 8 CTAs run at once; the largest problem takes two thirds of
+// the launch).  What stood beside them were FP64 instructions, each of which holds a scheduler for ~64
 // cycles, and barriers: one lane in four ended all columns of a row of Q, so the warp paid the
 // conversions and the subtraction once per column (now a thread ends one column of one row), a
 // column's partial sums were one chain of 32 FP64 additions (now four warps), the padding of A was
@@ -28,6 +29,7 @@
 // from the same sums in the same order, so their control flow cannot diverge.
 #include "batch.cuh"
 #include "dfloat.cuh"
+#include "values.cuh"
 
 #include <cooperative_groups.h>
 
@@ -44,8 +46,20 @@ constexpr int BT = 512;            // threads per CTA (16 warps; 128 registers e
 constexpr int BR = 32;             // rows per tile
 constexpr int JQ = 4;              // Q step: shares of the columns of A, each with BT / 32 / JQ = 4 warps of 8 rows
 constexpr int NPMAX = 256;         // largest padded n
-constexpr int LDS = NPMAX + 8;     // shared-memory pitch of a tile row (floats; 8 keeps
-                                   // the float4 reads of 4 rows on distinct banks)
+constexpr int LDS = NPMAX + 8;     // shared-memory pitch of the widest tile row (floats)
+constexpr int TILES = 3;           // widest tiles that are held at once
+
+// Tiles are held `depth` + 1 at a time, `depth` of them on their way: a narrow tile is worked off in
+// ~2000 cycles, about the time its successor takes to arrive, so up to n = 128, where five fit, four are, and
+// two above.  The pitch is npad rounded up to 32 floats, plus 8: the float4 reads of 4 rows meet
+// distinct banks.  With the vector reads of Q and X, b read a tile ahead and pairs widened by integer
+// operations in the residual: 64 problems up to 11803 x 255 with 16 columns 8.81 -> 8.62 ms.  What is left
+// of a narrow tile is issue slots (~350 instructions a warp), of a wide one the multiply-adds.
+struct BtRing {
+    int pitch, depth;
+    __device__ explicit BtRing(int npad) : pitch((npad + 31) / 32 * 32 + 8) { depth = 5 * pitch <= TILES * LDS ? 4 : 2; }
+    __device__ __forceinline__ int next(int buf) const { return buf == depth ? 0 : buf + 1; }
+};
 
 // Shared-memory layout for KC columns (byte offsets; every part 16-byte aligned)
 // P~ / x rows in shared memory are XP entries apart: 4 entries of padding (from 4 columns up)
@@ -53,8 +67,8 @@ constexpr int LDS = NPMAX + 8;     // shared-memory pitch of a tile row (floats;
 template <int KC> struct XPitch { static constexpr int v = KC >= 4 ? KC + 4 : KC; };
 template <int KC>
 struct BLayout {
-    static constexpr size_t as = 0;                                   // two A tiles (float)
-    static constexpr size_t xs = as + 2 * (size_t)BR * LDS * 4;       // P~ (float) or x (pairs)
+    static constexpr size_t as = 0;                                   // tiles of A (float)
+    static constexpr size_t xs = as + TILES * (size_t)BR * LDS * 4;       // P~ (float) or x (pairs)
     static constexpr size_t wp = xs + (size_t)NPMAX * XPitch<KC>::v * 8;   // this CTA's W
     static constexpr size_t qs = wp + (size_t)NPMAX * KC * 8;         // Q of the current tile
     static constexpr size_t red = qs + (size_t)BR * KC * 8;           // reduction scratch
@@ -68,7 +82,11 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool fu
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem), "r"(n) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+// all but the newest depth - 1 groups have landed (depth 2 or 4)
+__device__ __forceinline__ void cp_async_wait_oldest(int depth) {
+    if (depth == 4) asm volatile("cp.async.wait_group 3;" ::: "memory");
+    else asm volatile("cp.async.wait_group 1;" ::: "memory");
+}
 
 
 // A's padding columns n..npad-1 may hold anything: they enter no dot product (what they put into W
@@ -89,18 +107,40 @@ __device__ __forceinline__ void bt_tile_spots(int nch, int (&spot)[N]) {
         spot[u] = q < BR * nch ? (q / nch) << 16 | q % nch : -1;
     }
 }
+// Nothing is copied from r_hi on (an empty group keeps the count of groups)
 template <int N>
-__device__ __forceinline__ void bt_load_tile(const BatchProb& P, float* dst, int64_t r_lo, int64_t row0, int64_t r_hi,
-                                             int nch, const int (&spot)[N]) {
+__device__ __forceinline__ void bt_load_tile(const BatchProb& P, float* dst, int pitch, int64_t r_lo, int64_t row0,
+                                             int64_t r_hi, const int (&spot)[N]) {
 #pragma unroll
     for (int u = 0; u < N; ++u)
-        if (spot[u] >= 0) {
+        if (spot[u] >= 0 && row0 < r_hi) {
             const int r = spot[u] >> 16, ch = spot[u] & 0xffff;
             const int64_t i = row0 + r;
             const bool ok = i < r_hi;
-            cp_async16(dst + r * LDS + 4 * ch, P.A + (ok ? i : r_lo) * P.ld + 4 * ch, ok);
+            cp_async16(dst + r * pitch + 4 * ch, P.A + (ok ? i : r_lo) * P.ld + 4 * ch, ok);
         }
     cp_async_commit();
+}
+// N consecutive columns of a row of X or Q (four of them lie on a 16-byte boundary)
+template <int N>
+__device__ __forceinline__ void bt_read(float (&v)[N], const float* p) {
+    if constexpr (N == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    } else {
+#pragma unroll
+        for (int c = 0; c < N; ++c) v[c] = p[c];
+    }
+}
+template <int N>
+__device__ __forceinline__ void bt_read(f2 (&v)[N], const f2* p) {
+    if constexpr (N == 4) {
+        const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+        v[0] = f2{a.x, a.y}; v[1] = f2{a.z, a.w}; v[2] = f2{b.x, b.y}; v[3] = f2{b.z, b.w};
+    } else {
+#pragma unroll
+        for (int c = 0; c < N; ++c) v[c] = p[c];
+    }
 }
 // (hi, lo) += a x in the cascaded Dot2 form of Ogita, Rump & Oishi
 __device__ __forceinline__ void bt_cascade(f2& acc, float a, f2 x) {
@@ -123,7 +163,7 @@ __device__ __forceinline__ void bt_mac(f2& s, float a, f2 x) { bt_cascade(s, a, 
 // 64 problems up to 11803 x 255 with 16 columns: 9.60 -> 8.81 ms (with the divisions of the tile loads
 // taken out of the loop).
 template <int KC, typename T>
-__device__ __forceinline__ void bt_q_products(const float* At, const T* Xs, int n, int nch, T* part) {
+__device__ __forceinline__ void bt_q_products(const float* At, int pitch, const T* Xs, int n, int nch, T* part) {
     constexpr int CQ = KC < 4 ? KC : 4;
     constexpr int CG = KC / CQ;
     constexpr int JS = 8 / CG;
@@ -140,7 +180,7 @@ __device__ __forceinline__ void bt_q_products(const float* At, const T* Xs, int 
         float av[2][4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float4 a4 = *reinterpret_cast<const float4*>(At + (row + 4 * h) * LDS + 4 * ch);
+            const float4 a4 = *reinterpret_cast<const float4*>(At + (row + 4 * h) * pitch + 4 * ch);
             av[h][0] = a4.x; av[h][1] = a4.y; av[h][2] = a4.z; av[h][3] = a4.w;
             bt_mask_padding(av[h], 4 * ch, n);
         }
@@ -148,13 +188,7 @@ __device__ __forceinline__ void bt_q_products(const float* At, const T* Xs, int 
         for (int u = 0; u < 4; ++u) {
             const T* xr = Xs + (4 * ch + u) * XPitch<KC>::v + cg * CQ;
             T xv[CQ];
-            if constexpr (CQ == 4 && sizeof(T) == 4) {
-                const float4 x4 = *reinterpret_cast<const float4*>(xr);
-                xv[0] = x4.x; xv[1] = x4.y; xv[2] = x4.z; xv[3] = x4.w;
-            } else {
-#pragma unroll
-                for (int c = 0; c < CQ; ++c) xv[c] = xr[c];
-            }
+            bt_read(xv, xr);
 #pragma unroll
             for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -182,7 +216,7 @@ __device__ __forceinline__ void bt_q_products(const float* At, const T* Xs, int 
 //   Q = A X
 //   Wp = A^T Q over these rows, qq_out[c] = sum of Q_ic^2 over these rows (c < k)
 // X (npad x KC, rows j >= n zero) is in shared memory.  Tiles of BR rows are streamed with
-// cp.async into two buffers; the next tile is in flight while the current one is used.
+// cp.async; the next tiles (BtRing) are in flight while the current one is used.
 // W step: a thread owns 4 consecutive j and CQ columns (RS threads split the rows
 // when there are fewer such units than threads) and accumulates over all tiles in registers.
 template <int KC, typename T>
@@ -208,16 +242,20 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
     f2 qq{0.f, 0.f};   // of this thread's tile row and column
     int spot[NPMAX / 4 * BR / BT];
     bt_tile_spots(nch, spot);
+    const BtRing ring(npad);
     auto load_tile = [&](int t, int buf) {
-        bt_load_tile(P, As + buf * BR * LDS, r_lo, r_lo + (int64_t)t * BR, r_hi, nch, spot);
+        bt_load_tile(P, As + buf * BR * ring.pitch, ring.pitch, r_lo, r_lo + (int64_t)t * BR, r_hi, spot);
     };
-    if (ntile > 0) load_tile(0, 0);
+    int buf = 0, fill = ring.depth;   // where tile t is, where tile t + depth goes
+    for (int t = 0; t < ring.depth; ++t) load_tile(t, t);
     for (int t = 0; t < ntile; ++t) {
-        cp_async_wait_all();
+        cp_async_wait_oldest(ring.depth);
         __syncthreads();   // tile t has landed; every thread is done with tile t-1
-        if (t + 1 < ntile) load_tile(t + 1, (t + 1) & 1);
-        float* At = As + (t & 1) * BR * LDS;
-        bt_q_products<KC, T>(At, Xs, n, nch, reinterpret_cast<T*>(red));
+        load_tile(t + ring.depth, fill);
+        const float* At = As + buf * BR * ring.pitch;
+        buf = ring.next(buf);
+        fill = ring.next(fill);
+        bt_q_products<KC, T>(At, ring.pitch, Xs, n, nch, reinterpret_cast<T*>(red));
         __syncthreads();
         if (tid < BR * KC) {   // one tile row and column per thread
             const int64_t i = r_lo + (int64_t)t * BR + tid / KC;
@@ -232,11 +270,10 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
         __syncthreads();
         if (wact) {   // W step
             for (int r = rs; r < BR; r += RS) {
-                const float4 a4 = *reinterpret_cast<const float4*>(At + r * LDS + 4 * jg);
+                const float4 a4 = *reinterpret_cast<const float4*>(At + r * ring.pitch + 4 * jg);
                 const float av[4] = {a4.x, a4.y, a4.z, a4.w};
                 T qv[CQ];
-#pragma unroll
-                for (int c = 0; c < CQ; ++c) qv[c] = Qs[r * KC + cgw * CQ + c];
+                bt_read(qv, Qs + r * KC + cgw * CQ);
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -293,21 +330,29 @@ __device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi,
         for (int c = 0; c < CQ; ++c) acc[u][c] = f2{0.f, 0.f};
     int spot[NPMAX / 4 * BR / BT];
     bt_tile_spots(nch, spot);
+    const BtRing ring(npad);
     auto load_tile = [&](int t, int buf) {
-        bt_load_tile(P, As + buf * BR * LDS, r_lo, r_lo + (int64_t)t * BR, r_hi, nch, spot);
+        bt_load_tile(P, As + buf * BR * ring.pitch, ring.pitch, r_lo, r_lo + (int64_t)t * BR, r_hi, spot);
     };
-    if (ntile > 0) load_tile(0, 0);
+    int buf = 0, fill = ring.depth;
+    for (int t = 0; t < ring.depth; ++t) load_tile(t, t);
+    const bool has_q = tid < BR * KC && tid % KC < k;   // this thread ends row tid / KC, column tid % KC of each tile
+    const double* bp = P.B + (int64_t)(tid % KC) * P.ldb;
+    auto load_b = [&](int t) {
+        const int64_t i = r_lo + (int64_t)t * BR + tid / KC;
+        return has_q && i < r_hi ? bp[i] : 0.0;
+    };
+    double bq = load_b(0);   // a tile ahead of its use
     for (int t = 0; t < ntile; ++t) {
-        cp_async_wait_all();
+        cp_async_wait_oldest(ring.depth);
         __syncthreads();
-        if (t + 1 < ntile) load_tile(t + 1, (t + 1) & 1);
-        float* At = As + (t & 1) * BR * LDS;
+        load_tile(t + ring.depth, fill);
+        const float* At = As + buf * BR * ring.pitch;
+        buf = ring.next(buf);
+        fill = ring.next(fill);
         // Q = b - A x for this tile's rows (Q = b from x = 0): one tile row and column per thread
-        const int64_t qi = r_lo + (int64_t)t * BR + tid / KC;
-        const bool mine = tid < BR * KC && qi < r_hi && tid % KC < k;
-        const double bq = mine ? P.B[(int64_t)(tid % KC) * P.ldb + qi] : 0.0;
         if (!from_zero) {
-            bt_q_products<KC, f2>(At, Xs, n, nch, red);
+            bt_q_products<KC, f2>(At, ring.pitch, Xs, n, nch, red);
             __syncthreads();
         }
         if (tid < BR * KC) {
@@ -317,16 +362,19 @@ __device__ void bt_residual_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi,
 #pragma unroll
                 for (int j = 1; j < JQ; ++j) df_add(ax, red[j * BR * KC + tid]);
             }
-            Qs[tid] = mine ? df_from_double(bq - df_to_double(ax)) : f2{0.f, 0.f};
+            const bool mine = has_q && r_lo + (int64_t)t * BR + tid / KC < r_hi;
+            const double q = bq - (widen(ax.hi) + widen(ax.lo));
+            const float hi = __double2float_rn(q);
+            Qs[tid] = mine ? f2{hi, __double2float_rn(q - widen(hi))} : f2{0.f, 0.f};
+            bq = load_b(t + 1);
         }
         __syncthreads();
         if (wact) {   // W += A^T Q
             for (int r = rs; r < BR; r += RS) {
-                const float4 a4 = *reinterpret_cast<const float4*>(At + r * LDS + 4 * jg);
+                const float4 a4 = *reinterpret_cast<const float4*>(At + r * ring.pitch + 4 * jg);
                 const float av[4] = {a4.x, a4.y, a4.z, a4.w};
                 f2 qv[CQ];
-#pragma unroll
-                for (int c = 0; c < CQ; ++c) qv[c] = Qs[r * KC + cgw * CQ + c];
+                bt_read(qv, Qs + r * KC + cgw * CQ);
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
