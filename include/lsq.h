@@ -21,8 +21,9 @@
  *     them and they must stay valid until the call returns (or, for stream-ordered
  *     outputs, until the stream reaches that point).  The library never frees them.
  *   - The only library-owned object is lsq_precond (free it with lsq_precond_destroy).
- *     Per-call scratch is taken with cudaMallocAsync on the given stream and released on
- *     the same stream before the call returns.
+ *     Per-call scratch is taken on the given stream from a memory pool of the library's own
+ *     (one per device, which keeps at most 1 GiB between calls and gives it back when an
+ *     allocation fails) and released on the same stream before the call returns.
  *   - Work is issued on the given stream (0 = legacy default stream).  Calls that report
  *     data-dependent status (every call below) synchronise that stream once at the end
  *     to read it.
@@ -397,16 +398,19 @@ LSQ_API int64_t lsq_kernel_launch_count(void);
 LSQ_API lsq_status lsq_set_wait_limit(int64_t max_polls);
 
 /* Form of the one-column sparse Gauss-Seidel sweeps (Alg. 3 on a CSR A_s^T A_s), a tuning and
- * test setting; every form computes the same rows in the same level order with the same
+ * test setting; forms 1 to 3 compute the same rows in the same level order with the same
  * per-row arithmetic:
- *   0  chosen from the level schedule's shape: one CTA or the grid (the default),
+ *   0  chosen from the level schedule's shape (the default): one CTA, the grid, or, where the
+ *      schedule is deep and rows are long, blocks of consecutive rows with inverted diagonal
+ *      blocks: the same sweep, rounded in another order.  Captured and persistent solves
+ *      keep the row forms,
  *   1  the grid: every row waits (bounded) for the values of its own dependencies,
  *   2  one CTA: levels meet at block barriers,
  *   3  one thread-block cluster of 8 CTAs: the sweep vector in the cluster's shared memory
  *      and levels at cluster barriers; where it does not fit (n > 204,800 or no cluster slot
  *      on the device) the grid form runs instead.
  * Blocks of k >= 2 right-hand sides (stream-ordered solves) take form 3 as well, where their
- * n x k vector fits (n k <= 204,800); every other value leaves them on their grid forms.
+ * n x k vector fits (n k <= 204,800); 1 and 2 leave them on their grid forms, 0 chooses as above.
  * Process-wide, read when a solve or preconditioner application starts.  LSQ_ERR_INVALID
  * unless 0 <= form <= 3. */
 LSQ_API lsq_status lsq_set_sweep_form(int32_t form);
