@@ -208,8 +208,8 @@ LSQ_API lsq_status lsq_build_precond(const lsq_matrix* A, const int32_t* idx, co
                              const double* colscale, int64_t s, const lsq_opts* o,
                              lsq_precond** P_out, void* stream);
 
-/* Free a handle from lsq_build_precond (NULL is ignored).  Stream-ordered on the stream
- * the handle was built on. */
+/* Free a handle from lsq_build_precond (NULL is ignored).  Waits for all work on the device the
+ * handle was built on, whichever device is current, and leaves the current device as it is. */
 LSQ_API void lsq_precond_destroy(lsq_precond* P);
 
 /* Copy the assembled M = A_s^T A_s of Sec. 3.3 out of a dense handle (row-major n x n into

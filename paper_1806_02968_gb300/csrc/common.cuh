@@ -5,10 +5,9 @@
 #include <stdint.h>
 #include <string>
 #include <atomic>
-#include <initializer_list>
 
 #include "../../include/lsq.h"
-
+#include "pool.cuh"
 
 typedef unsigned __int128 u128;
 
@@ -68,19 +67,6 @@ inline size_t elem_size(int dtype) {
 }
 
 lsq_status check_matrix(const lsq_matrix* A);
-
-// Device memory of scratch buffers and handles: stream-ordered allocations from a pool of the
-// library's own (one per device), which keeps up to POOL_KEEP bytes of freed memory mapped. The
-// device's default pool gives everything back at every synchronisation, and mapping it again
-// cost 0.1 to 1 ms per call. The pool gives all it holds back when an allocation fails (which is
-// then tried again), and the rest above POOL_KEEP at every synchronisation.
-constexpr uint64_t POOL_KEEP = 1ull << 30;   // 0.35 % of the device's memory
-cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t st);
-template <typename T>
-inline cudaError_t pool_alloc(T** p, size_t bytes, cudaStream_t st) { return pool_alloc((void**)p, bytes, st); }
-// Frees a handle's arrays (NULL entries are skipped) once all work on the device has ended:
-// the handle may have been used on any stream.
-void pool_free(std::initializer_list<void*> ptrs);
 
 // Stream-ordered scratch that is released on the same stream when it goes out of scope.
 struct Scratch {
@@ -209,11 +195,11 @@ namespace lsq { struct SparseHandle; }
 // Library-owned preconditioner handle (definition shared by the translation units).
 struct lsq_precond {
     int64_t n = 0, s = 0;
+    int32_t device = 0;         // the device it was built on, which owns every array
     int32_t dense = 1;
     int32_t sweeps = 1;
     int32_t op_dtype = LSQ_F64;  // storage of the materialised operator
     int64_t nnz_M = 0, n_fixed_diag = 0, levels = 0;
-    cudaStream_t stream = 0;
     double* M = nullptr;        // dense n x n FP64 (row-major)
     void* op = nullptr;         // dense n x n materialised SGS operator, op_dtype
     double* colscale = nullptr; // d_j (n)

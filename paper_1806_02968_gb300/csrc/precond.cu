@@ -84,8 +84,8 @@ static lsq_status build_dense(const lsq_matrix* A, const int32_t* idx, const dou
 
 static void free_handle(lsq_precond* H) {
     if (!H) return;
-    pool_free({H->M, H->op, H->colscale, H->inv_d});
-    if (H->sp) free_sparse(H->sp);
+    pool_free(H->device, {H->M, H->op, H->colscale, H->inv_d});
+    if (H->sp) free_sparse(H->sp, H->device);
     delete H;
 }
 
@@ -107,9 +107,11 @@ extern "C" lsq_status lsq_build_precond(const lsq_matrix* A, const int32_t* idx,
     else LSQ_CHECK_ARG(o->sweeps <= 32, "sparse preconditioners support sweeps <= 32");
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t n = A->n;
+    int dev = 0;
+    LSQ_CUDA(cudaGetDevice(&dev));
     lsq_precond* H = new lsq_precond();
+    H->device = dev;
     H->n = n; H->s = s; H->dense = A->dense ? 1 : 0; H->sweeps = o->sweeps; H->op_dtype = o->precond_dtype;
-    H->stream = st;
     auto fail = [&](lsq_status code) { free_handle(H); return code; };
     cudaError_t e;
     if ((e = pool_alloc(&H->colscale, sizeof(double) * n, st)) != cudaSuccess ||

@@ -33,7 +33,7 @@ lsq_status transpose_pattern(const int64_t* rptr, const int32_t* col, int64_t nr
                              int64_t* cptr, int32_t* trow, int64_t* tperm, cudaStream_t st);
 lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p, int64_t s,
                         lsq_precond* H, cudaStream_t st);
-void free_sparse(SparseHandle* S);
+void free_sparse(SparseHandle* S, int device);
 // The sweep form set by lsq_set_sweep_form (0 by shape, 1 grid, 2 one CTA, 3 one cluster).
 int sweep_form_setting();
 // Blocks of a grid-form sweep: enough that every row of an average level has its own warp

@@ -846,10 +846,10 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
     return LSQ_OK;
 }
 
-void free_sparse(SparseHandle* S) {
+void free_sparse(SparseHandle* S, int device) {
     if (!S) return;
-    pool_free({S->mptr, S->mcol, S->mval, S->mval32, S->dinv, S->mdiag, S->sched_f, S->sched_b, S->inv,
-               S->atptr, S->atrow, S->atperm, S->loff_f, S->loff_b});
+    pool_free(device, {S->mptr, S->mcol, S->mval, S->mval32, S->dinv, S->mdiag, S->sched_f, S->sched_b, S->inv,
+                       S->atptr, S->atrow, S->atperm, S->loff_f, S->loff_b});
     delete S;
 }
 
