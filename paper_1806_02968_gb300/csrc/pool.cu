@@ -5,13 +5,24 @@
 
 namespace lsq {
 
-// The pools, by device.  A pool that no longer works (the device was reset) is made again.
+// The pools, by device.  A pool that no longer works (the device was reset) is made again; what
+// the dead one held went with the device's context.
 namespace {
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[64] = {};
-cudaError_t pool_of(int dev, bool renew, cudaMemPool_t* out) {
+// The device's pool, made if there is none.  `failed` is a pool that refused an allocation: it is
+// replaced if it is still the device's and does not answer any more.  A live pool refuses for the
+// caller's reason (a stream that is not one, say) and stays: *out is `failed` again.
+cudaError_t pool_of(int dev, cudaMemPool_t failed, cudaMemPool_t* out) {
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    if (!g_pool[dev] || renew) {
+    if (failed && g_pool[dev] == failed) {
+        uint64_t keep = 0;
+        if (cudaMemPoolGetAttribute(failed, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            g_pool[dev] = nullptr;
+        }
+    }
+    if (!g_pool[dev]) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
@@ -21,7 +32,10 @@ cudaError_t pool_of(int dev, bool renew, cudaMemPool_t* out) {
         if (e != cudaSuccess) return e;
         uint64_t keep = POOL_KEEP;
         e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(made);
+            return e;
+        }
         g_pool[dev] = made;
     }
     *out = g_pool[dev];
@@ -35,7 +49,7 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t st) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     cudaMemPool_t pool = nullptr;
-    if (dev >= 64 || pool_of(dev, false, &pool) != cudaSuccess) {
+    if (dev >= 64 || pool_of(dev, nullptr, &pool) != cudaSuccess) {
         cudaGetLastError();
         return cudaMallocAsync(p, bytes, st);   // no pool of our own: the device's
     }
@@ -46,7 +60,10 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t st) {
         e = cudaMallocFromPoolAsync(p, bytes, pool, st);
     } else if (e == cudaErrorInvalidValue || e == cudaErrorInvalidResourceHandle) {
         cudaGetLastError();
-        if ((e = pool_of(dev, true, &pool)) == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+        cudaMemPool_t now = nullptr;
+        cudaError_t made = pool_of(dev, pool, &now);
+        if (made != cudaSuccess) return made;
+        if (now != pool) e = cudaMallocFromPoolAsync(p, bytes, now, st);
     }
     return e;
 }

@@ -87,3 +87,21 @@ def test_free_waits_for_the_owning_device(tmp_path):
     assert out[:4] == ["create 1 on 0", "alloc 1", "create 2 on 1", "alloc 2"]
     assert out[4] == "sync 1" and out[5].startswith("free 1 ") and out[6] == "current 0"
     assert out[7] == "sync 0" and out[8].startswith("free 0 ") and len(out) == 9
+
+
+def test_a_refused_allocation_keeps_a_live_pool(tmp_path):
+    """A caller's bad stream gives the error codes of a dead pool: the pool stays the one it was."""
+    out = _run(tmp_path, '''
+    for (int i = 0; i < 3; ++i) printf("code %d\\n", (int)lsq::pool_alloc(&p, 16, (cudaStream_t)0xbad));
+    lsq::pool_alloc(&p, 16, (cudaStream_t)0);
+''')
+    assert out == ["create 1 on 0"] + ["code 400"] * 3 + ["alloc 1"]
+
+
+def test_a_dead_pool_is_replaced_once(tmp_path):
+    out = _run(tmp_path, '''
+    lsq::pool_alloc(&p, 16, (cudaStream_t)0);
+    alive[(cudaMemPool_t)1] = false;
+    for (int i = 0; i < 2; ++i) printf("code %d\\n", (int)lsq::pool_alloc(&p, 16, (cudaStream_t)0));
+''')
+    assert out == ["create 1 on 0", "alloc 1", "create 2 on 0", "alloc 2", "code 0", "alloc 2", "code 0"]
