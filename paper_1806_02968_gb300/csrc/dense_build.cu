@@ -441,11 +441,16 @@ __global__ void __launch_bounds__(SG_T) k_sgs_columns(int64_t n, int sweeps, con
     }
 }
 
+// Shared memory for n <= 2048 columns.  The limit is one for the whole process and set to the most,
+// so that threads that build handles of different sizes do not lower it under one another.
+constexpr size_t sg_bytes(int64_t n, int C) {
+    return 8 * ((size_t)((n + 31) / 32) * 32 * C + SG_W * 32 * C + 32 * C);
+}
 template <typename OT, int C>
 static lsq_status sgs_columns(int64_t n, int sweeps, const double* M, const double* lt, const double* lo, OT* op,
                               cudaStream_t st) {
-    const size_t smem = 8 * ((size_t)((n + 31) / 32) * 32 * C + SG_W * 32 * C + 32 * C);
-    LSQ_CUDA(cudaFuncSetAttribute(k_sgs_columns<OT, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = sg_bytes(n, C);
+    LSQ_CUDA(cudaFuncSetAttribute(k_sgs_columns<OT, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sg_bytes(2048, C)));
     k_sgs_columns<OT, C><<<(unsigned)((n + C - 1) / C), SG_T, smem, st>>>(n, sweeps, M, lt, lo, op);
     count_launch();
     LSQ_CUDA(cudaGetLastError());

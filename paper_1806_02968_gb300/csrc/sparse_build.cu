@@ -538,6 +538,12 @@ __global__ void __launch_bounds__(32) k_spgemm_long(SpgArgs a) {
     }
     if (!FILL && lane == 0 && longest > 0) atomicMax(a.maxrow, longest);
 }
+// Shared memory of the long-row kernel, and the most any call needs.  The limit that a kernel is
+// given is one for the whole process, so it is set to the most: two threads that build handles of
+// different sizes must not lower it under one another.
+constexpr size_t spg_bytes(bool fill, size_t win, size_t acap) {
+    return (fill ? 12 * acap : 0) + 6 * ((win + 31) / 32) + 16;
+}
 // Both kernels of one pass; the long-row kernel only when there is a long row.
 template <bool FILL>
 static lsq_status spgemm_pass(SpgArgs a, int maxcand, int sms, cudaStream_t st) {
@@ -545,9 +551,10 @@ static lsq_status spgemm_pass(SpgArgs a, int maxcand, int sms, cudaStream_t st) 
     count_launch();
     if (maxcand <= SPG_SHORT) return LSQ_OK;
     a.win = (int)std::min<int64_t>(a.n, SPG_WIN);
-    const size_t words = (size_t)(a.win + 31) / 32;
-    const size_t smem = (FILL ? 12 * (size_t)a.acap : 0) + 4 * words + 2 * words + 16;
-    LSQ_CUDA(cudaFuncSetAttribute(k_spgemm_long<FILL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = spg_bytes(FILL, (size_t)a.win, (size_t)a.acap);
+    constexpr size_t most = spg_bytes(FILL, (size_t)SPG_WIN, (size_t)SPG_CAP + 2);
+    static_assert(most <= 227 * 1024, "a row's sums and the window's bitmap fit an SM");
+    LSQ_CUDA(cudaFuncSetAttribute(k_spgemm_long<FILL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     int per = 0;
     LSQ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_spgemm_long<FILL>, 32, smem));
     if (per < 1) { set_error("SpGEMM kernel does not fit on an SM"); return LSQ_ERR_CUDA; }
