@@ -65,14 +65,20 @@ __global__ void __launch_bounds__(256) k_oz_max(lsq_matrix A, const int32_t* idx
     }
 }
 // e_j with |x_tj| < 2^e_j (x the product with the head, correctly rounded), and 1 / d_j scaled
-// so that the digits' integer is a_ij times it times the root
+// so that the digits' integer is a_ij times it times the root.  A column without a non-zero draw
+// has the scale 0, so that all its digits are zero; e_j is no smaller than what keeps the scale finite.
 __global__ void k_oz_exp(const unsigned long long* mx, const double* inv_d, int64_t n, int* e, double* sd) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     const int ex = (int)(mx[j] >> 52);
-    const int ej = ex == 0x7ff ? OZ_BAD : max(ex, 1) - 1022;
+    int ej = ex == 0x7ff ? OZ_BAD : 0;
+    double sj = 0.0;
+    if (mx[j] != 0 && ej != OZ_BAD) {
+        ej = max(max(ex, 1) - 1022, ilogb(inv_d[j]) + 55 - 1022);
+        sj = scalbn(inv_d[j], 55 - ej);
+    }
     e[j] = ej;
-    sd[j] = ej == OZ_BAD ? 0.0 : scalbn(inv_d[j], 55 - ej);
+    sd[j] = sj;
 }
 // Digits of the integer nearest x0 + x1, |x0| < 2^55, x1 the rounding error of x0.  Integer
 // arithmetic on the bits: FP64 operations and conversions run at 1/64 of the integer rate.
