@@ -9,11 +9,15 @@
 // products of digits p and q with p + q <= 7 are summed by bf16 MMAs with FP32 accumulators.
 // Digits are at most 128, so a sum of 128 rows over the at most seven pairs of one p + q stays
 // below 2^24 and is exact; it is then moved to 64-bit integers.  (The pairs with p + q = 7 join
-// the last sum scaled by 2^-8, with its rounding.)  The digits stop at 2^-56 of a column's
-// largest entry, and what is left out of the products lies at 2^-64 of the two largest.
+// the last sum scaled by 2^-8, with its rounding.)  What remains are the digits' end at 2^-56 of a
+// column's largest entry and the products that are left out, 2^-64 of the two largest: errors
+// against sqrt(M_jj M_kk).  An entry whose terms are all far below that (a column with one entry that
+// stands out) would keep fewer bits than an FP64 product gives it, so every entry's error is
+// bounded beside the products, and the tiles with one that may pass 8 roundings of its terms are
+// summed in FP64 (k_wide_check, k_wide_tiles).
 // 12,777 draws of 512 columns: 0.37 ms, and 0.11 ms for the digits; s = 9,586, n = 400: 0.23 ms
 // and 0.07, against 2.1 ms.  Error of M against extended precision (Frobenius, relative; FP64
-// product before): Gaussian 1.45e-16 (1.83e-16), 2 % heavy rows 1.44e-16 (1.88e-16), the same
+// product in brackets): Gaussian 1.45e-16 (1.83e-16), 2 % heavy rows 1.44e-16 (1.88e-16), the same
 // under uniform draws 1.75e-16 (2.95e-16), UDV 1.49e-16 (1.93e-16), FP32 values 1.42e-16
 // (2.32e-16), semi-Gaussian 1.82e-16 (2.57e-16).
 #include "dense_build.cuh"
@@ -24,13 +28,14 @@
 namespace lsq {
 
 constexpr int OZ_P = 7;           // digits
+constexpr int OZ_PL = OZ_P + 1;   // planes: the digits, and the magnitudes
 constexpr int OZ_TILE = 64;       // columns of M per tile edge
 constexpr int OZ_KC = 16;         // draws per stage
 constexpr int OZ_STAGES = 4;
 constexpr int OZ_FLUSH = 128;     // draws whose sums stay exact in FP32
 constexpr int OZ_PITCH = OZ_TILE + 8;   // bf16 per staged row (16 bytes of padding: distinct banks)
 constexpr int OZ_T = 256;
-constexpr size_t OZ_STAGE = (size_t)2 * OZ_P * OZ_KC * OZ_PITCH * 2;
+constexpr size_t OZ_STAGE = (size_t)2 * OZ_PL * OZ_KC * OZ_PITCH * 2;
 constexpr int OZ_BAD = 1 << 20;   // exponent of a column with a non-finite entry
 
 // sqrt(gamma_t), gamma_t = 1 / (s p_t), as a head and a tail: its square is gamma_t to far below
@@ -100,15 +105,24 @@ __device__ __forceinline__ void oz_digits(double x0, double x1, int (&d)[OZ_P]) 
     }
     d[0] = (int)y;                                // |d_0| <= 128
 }
+// |x0| 2^-55 cut to a bf16, from below; a non-zero one at least 2^-60, so that products stay normal
+__device__ __forceinline__ unsigned oz_magnitude(double x0) {
+    const unsigned hi = (unsigned)__double2hiint(x0) & 0x7fffffffu;
+    if (hi == 0u && __double2loint(x0) == 0) return 0u;
+    const int b = (int)(hi >> 13) - ((1023 + 55 - 127) << 7);   // rebias the exponent, keep 7 bits
+    return (unsigned)max(b, (127 - 60) << 7);
+}
 __device__ __forceinline__ unsigned bf16_of_int(int v) { return __float_as_uint((float)v) >> 16; }
 template <int DT>
 __device__ __forceinline__ void oz_entry(const lsq_matrix& A, int64_t row, int64_t j, double sd, double2 g,
-                                         int (&d)[OZ_P]) {
+                                         int (&d)[OZ_P], unsigned& mag) {
     const double t = oz_a<DT>(A, row, j, sd);
     const double x0 = __dmul_rn(t, g.x);
     oz_digits(x0, fma(t, g.y, fma(t, g.x, -x0)), d);
+    mag = oz_magnitude(x0);
 }
-// digits of draws [t0, t0 + rows) (zero beyond s and n): q[p][t - t0][j], two columns a thread
+// digits and magnitudes of draws [t0, t0 + rows) (zero beyond s and n): q[p][t - t0][j], two
+// columns a thread
 template <int DT>
 __global__ void __launch_bounds__(256) k_oz_slice(lsq_matrix A, const int32_t* idx, const double2* rg,
                                                   const double* sd, const int* e, int64_t s, int64_t t0,
@@ -119,14 +133,16 @@ __global__ void __launch_bounds__(256) k_oz_slice(lsq_matrix A, const int32_t* i
         const int64_t r = w / half, t = t0 + r;
         const int j = 2 * (int)(w - r * half);
         int d0[OZ_P] = {}, d1[OZ_P] = {};
+        unsigned m0 = 0, m1 = 0;
         if (t < s) {
             const int64_t row = idx[t];
             const double2 g = rg[t];
-            if (j < A.n && e[j] != OZ_BAD) oz_entry<DT>(A, row, j, sd[j], g, d0);
-            if (j + 1 < A.n && e[j + 1] != OZ_BAD) oz_entry<DT>(A, row, j + 1, sd[j + 1], g, d1);
+            if (j < A.n && e[j] != OZ_BAD) oz_entry<DT>(A, row, j, sd[j], g, d0, m0);
+            if (j + 1 < A.n && e[j + 1] != OZ_BAD) oz_entry<DT>(A, row, j + 1, sd[j + 1], g, d1, m1);
         }
 #pragma unroll
         for (int p = 0; p < OZ_P; ++p) q[p * plane + w] = bf16_of_int(d0[p]) | (bf16_of_int(d1[p]) << 16);
+        q[OZ_P * plane + w] = m0 | (m1 << 16);
     }
 }
 
@@ -151,10 +167,11 @@ __device__ __forceinline__ unsigned bf16x2_scale(unsigned v) {
 // part[z][i][j] (+)= sum over split z's draws of x_ti x_tj for tile pair (ti <= tj).  8 warps: 4
 // row groups of 16 by 2 column groups of 32; every warp keeps one FP32 accumulator tile per
 // p + q and moves it to its 64-bit totals every 128 draws.  Digits arrive by cp.async in four
-// stages of 16 draws.  Bound: MMA issue (34 MMAs per 16 x 8 x 16 block of M).
+// stages of 16 draws.  mag[z][i][j] (+)= the same sums of the magnitudes, a lower bound of sum |x_ti| |x_tj|
+// in units of 2^(e_i + e_j).  Bound: MMA issue (35 MMAs per 16 x 8 x 16 block of M).
 __global__ void __launch_bounds__(OZ_T, 1) k_oz_gemm(const unsigned short* q, int64_t rows, int npad, int64_t n,
                                                      const int* e, int64_t per_split, int ntile, double* part,
-                                                     int accumulate) {
+                                                     float* mag, int accumulate) {
     extern __shared__ __align__(16) unsigned char oz_smem[];
     int ti = 0, rest = blockIdx.x;
     while (rest >= ntile - ti) { rest -= ntile - ti; ++ti; }
@@ -166,22 +183,22 @@ __global__ void __launch_bounds__(OZ_T, 1) k_oz_gemm(const unsigned short* q, in
     auto stage = [&](int k) {
         unsigned char* dst = oz_smem + (size_t)(k % OZ_STAGES) * OZ_STAGE;
         const int64_t t = r0 + (int64_t)k * OZ_KC;
-        // 2 operands x 7 planes x 16 rows x 8 chunks of 16 bytes
-        for (int c = tid; c < 2 * OZ_P * OZ_KC * 8; c += OZ_T) {
-            const int ch = c & 7, r = (c >> 3) & (OZ_KC - 1), pl = c >> 7;    // plane index 0..13
-            const int side = pl >= OZ_P ? 1 : 0, p = pl - side * OZ_P;
+        // 2 operands x 8 planes x 16 rows x 8 chunks of 16 bytes
+        for (int c = tid; c < 2 * OZ_PL * OZ_KC * 8; c += OZ_T) {
+            const int ch = c & 7, r = (c >> 3) & (OZ_KC - 1), pl = c >> 7;    // plane index 0..15
+            const int side = pl >= OZ_PL ? 1 : 0, p = pl - side * OZ_PL;
             const unsigned short* src = q + ((int64_t)p * rows + t + r) * npad + (side ? tj : ti) * OZ_TILE + ch * 8;
             const unsigned s = (unsigned)__cvta_generic_to_shared(dst + ((size_t)(pl * OZ_KC + r) * OZ_PITCH + ch * 8) * 2);
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(src) : "memory");
         }
     };
-    float acc[OZ_P][4][4];
+    float acc[OZ_P][4][4], macc[4][4];
     long long hi[4][4], lo[4][4];
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            hi[nt][v] = 0; lo[nt][v] = 0;
+            hi[nt][v] = 0; lo[nt][v] = 0; macc[nt][v] = 0.f;
 #pragma unroll
             for (int d = 0; d < OZ_P; ++d) acc[d][nt][v] = 0.f;
         }
@@ -205,7 +222,7 @@ __global__ void __launch_bounds__(OZ_T, 1) k_oz_gemm(const unsigned short* q, in
 #pragma unroll
             for (int qq = 0; qq < OZ_P; ++qq) {
                 unsigned b[4];
-                ldsm4t(b, S + (size_t)((OZ_P + qq) * OZ_KC + (mid & 1) * 8 + mr) * OZ_PITCH + wj + jp * 16 + (mid >> 1) * 8);
+                ldsm4t(b, S + (size_t)((OZ_PL + qq) * OZ_KC + (mid & 1) * 8 + mr) * OZ_PITCH + wj + jp * 16 + (mid >> 1) * 8);
 #pragma unroll
                 for (int p = 0; p + qq < OZ_P; ++p) {
                     mma_bf16(acc[p + qq][2 * jp], a[p], b[0], b[1]);
@@ -218,6 +235,14 @@ __global__ void __launch_bounds__(OZ_T, 1) k_oz_gemm(const unsigned short* q, in
                     mma_bf16(acc[OZ_P - 1][2 * jp + 1], a[OZ_P - qq], b[2], b[3]);
                 }
             }
+        }
+        ldsm4t(a[0], S + (size_t)(OZ_P * OZ_KC + (mid >> 1) * 8 + mr) * OZ_PITCH + wi + (mid & 1) * 8);
+#pragma unroll
+        for (int jp = 0; jp < 2; ++jp) {
+            unsigned b[4];
+            ldsm4t(b, S + (size_t)((OZ_PL + OZ_P) * OZ_KC + (mid & 1) * 8 + mr) * OZ_PITCH + wj + jp * 16 + (mid >> 1) * 8);
+            mma_bf16(macc[2 * jp], a[0], b[0], b[1]);
+            mma_bf16(macc[2 * jp + 1], a[0], b[2], b[3]);
         }
         if ((k + 1) % (OZ_FLUSH / OZ_KC) == 0 || k + 1 == nst) {
 #pragma unroll
@@ -234,6 +259,7 @@ __global__ void __launch_bounds__(OZ_T, 1) k_oz_gemm(const unsigned short* q, in
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     double* out = part + (int64_t)blockIdx.y * n * n;
+    float* mout = mag + (int64_t)blockIdx.y * n * n;
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
@@ -246,7 +272,94 @@ __global__ void __launch_bounds__(OZ_T, 1) k_oz_gemm(const unsigned short* q, in
                 if (ei == OZ_BAD || ej == OZ_BAD) x = __longlong_as_double(0x7ff8000000000000ll);
                 else x = scalbn(x, ei + ej - 14);
                 out[i * n + j] = accumulate ? out[i * n + j] + x : x;
+                mout[i * n + j] = accumulate ? mout[i * n + j] + macc[nt][v] : macc[nt][v];
             }
+        }
+}
+
+// Column sums of the magnitudes, rounded up to multiples of 2^-24 (whole numbers, so that the sum
+// does not depend on the order), 64 draws per block.
+__global__ void __launch_bounds__(256) k_oz_sums(const unsigned short* mag, int64_t rows, int npad, int64_t n,
+                                                 unsigned long long* sum) {
+    const int64_t t0 = (int64_t)blockIdx.x * 64, t1 = min(rows, t0 + 64);
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+        unsigned v = 0;
+#pragma unroll 8
+        for (int64_t t = t0; t < t1; ++t)
+            v += (unsigned)__float2int_ru(__uint_as_float((unsigned)mag[t * npad + j] << 16) * 0x1p24f);
+        if (v) atomicAdd(&sum[j], (unsigned long long)v);
+    }
+}
+// Marks the tiles with an entry that the digits may leave less accurate than an FP64 product.  The
+// digits' errors in entry (i, j) are at most 2^-56 (sum |x_ti| + sum |x_tj|) from the digits' end and
+// 5 * 2^-64 a draw from the products left out, in units of 2^(e_i + e_j); an FP64 product rounds each term
+// four times before it adds them.  Accepted: 2^-50 sum |x_ti| |x_tj|, eight roundings of the terms, if all of
+// the digits' errors had one sign (they do not: where this bound is met the error measured is at most a
+// fifth of the FP64 product's, Gaussian, UDV, heavy rows and semi-Gaussian at n = 40 to 512, and
+// these meet it three times over).  No common draw: nothing to lose.  The magnitudes are cut to 8
+// bits: the sums of one column are taken 2^-7 higher.
+__global__ void k_wide_check(int64_t n, int64_t s, int splits, int ntile, const float* mag,
+                             const unsigned long long* sum, const int* e, int* wide) {
+    const int64_t total = n * n;
+    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < total; w += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = w / n, j = w - i * n;
+        if (j < i || e[i] == OZ_BAD || e[j] == OZ_BAD) continue;
+        float b = 0.f;
+        for (int z = 0; z < splits; ++z) b += mag[(int64_t)z * total + w];
+        if (b == 0.f) continue;
+        const float need = (1.f + 0x1p-6f) * 0x1p-24f * (float)(sum[i] + sum[j]) + 6 * 0x1p-8f * (float)s;
+        if (need > 64.f * b) wide[(i / OZ_TILE) * ntile + j / OZ_TILE] = 1;
+    }
+}
+// part[z][i][j] of a marked tile in FP64: 4 x 4 entries a thread, 16 draws at a time through shared
+// memory.  Bound: FP64 FMAs, two a clock and SM (all tiles of 12,777 draws of 512 columns: 4.0 ms).
+template <int DT>
+__global__ void __launch_bounds__(256) k_wide_tiles(lsq_matrix A, const int32_t* idx, const double* p,
+                                                    const double* inv_d, int64_t s, int64_t per_split, int ntile,
+                                                    const int* wide, double* part) {
+    int ti = 0, rest = blockIdx.x;
+    while (rest >= ntile - ti) { rest -= ntile - ti; ++ti; }
+    const int tj = ti + rest;
+    if (!wide[ti * ntile + tj]) return;
+    const int64_t n = A.n, i0 = (int64_t)ti * OZ_TILE, j0 = (int64_t)tj * OZ_TILE;
+    const int64_t t_begin = min(s, (int64_t)blockIdx.y * per_split), t_end = min(s, t_begin + per_split);
+    __shared__ double Xi[OZ_KC][OZ_TILE], Xj[OZ_KC][OZ_TILE];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    double acc[4][4] = {};
+    for (int64_t t0 = t_begin; t0 < t_end; t0 += OZ_KC) {
+        for (int w = threadIdx.x; w < OZ_KC * OZ_TILE; w += 256) {
+            const int tt = w / OZ_TILE, c = w % OZ_TILE;
+            const int64_t t = t0 + tt;
+            double vi = 0.0, vj = 0.0;
+            if (t < t_end) {
+                const int64_t row = idx[t];
+                const double g = __drcp_rn(__dmul_rn((double)s, p[t]));
+                if (i0 + c < n) vi = __dmul_rn(oz_a<DT>(A, row, i0 + c, inv_d[i0 + c]), g);
+                if (j0 + c < n) vj = oz_a<DT>(A, row, j0 + c, inv_d[j0 + c]);
+            }
+            Xi[tt][c] = vi;
+            Xj[tt][c] = vj;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int tt = 0; tt < OZ_KC; ++tt) {
+            double a[4], b[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) { a[r] = Xi[tt][ty * 4 + r]; b[r] = Xj[tt][tx * 4 + r]; }
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[r][q] = fma(a[r], b[q], acc[r][q]);
+        }
+        __syncthreads();
+    }
+    double* out = part + (int64_t)blockIdx.y * n * n;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + ty * 4 + r, j = j0 + tx * 4 + q;
+            if (i < n && j < n) out[i * n + j] = acc[r][q];
         }
 }
 
@@ -273,7 +386,7 @@ static lsq_status normal_matrix(const lsq_matrix* A, const int32_t* idx, const d
     const int tiles = ntile * (ntile + 1) / 2;
     // draws per chunk: digits of at most 96 MB, which stay in L2 between the two kernels
     const int64_t srows = (s + OZ_FLUSH - 1) / OZ_FLUSH * OZ_FLUSH;
-    int64_t chunk = std::max<int64_t>(((int64_t)96 << 20) / (2 * OZ_P * npad) / OZ_FLUSH * OZ_FLUSH, OZ_FLUSH);
+    int64_t chunk = std::max<int64_t>(((int64_t)96 << 20) / (2 * OZ_PL * npad) / OZ_FLUSH * OZ_FLUSH, OZ_FLUSH);
     chunk = std::min(chunk, srows);
     // about one CTA per SM: each split takes at least 128 draws of a chunk
     int64_t splits = std::max<int64_t>(152 / tiles, 1);
@@ -283,8 +396,10 @@ static lsq_status normal_matrix(const lsq_matrix* A, const int32_t* idx, const d
     Scratch sc;
     auto r256 = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t o_rg = 0, o_mx = r256(16 * (size_t)s), o_e = o_mx + r256(8 * (size_t)n),
-                 o_sd = o_e + r256(4 * (size_t)n), o_q = o_sd + r256(8 * (size_t)n),
-                 o_part = o_q + r256((size_t)2 * OZ_P * chunk * npad), total = o_part + 8 * (size_t)splits * n * n;
+                 o_sd = o_e + r256(4 * (size_t)n), o_sum = o_sd + r256(8 * (size_t)n),
+                 o_wide = o_sum + r256(8 * (size_t)n), o_q = o_wide + r256(4 * (size_t)ntile * ntile),
+                 o_part = o_q + r256((size_t)2 * OZ_PL * chunk * npad),
+                 o_mag = o_part + r256(8 * (size_t)splits * n * n), total = o_mag + 4 * (size_t)splits * n * n;
     LSQ_CUDA(sc.alloc(total, st));
     char* base = sc.as<char>();
     double2* rg = (double2*)(base + o_rg);
@@ -293,7 +408,11 @@ static lsq_status normal_matrix(const lsq_matrix* A, const int32_t* idx, const d
     int* e = (int*)(base + o_e);
     unsigned* q = (unsigned*)(base + o_q);
     double* part = (double*)(base + o_part);
+    float* mag = (float*)(base + o_mag);
+    unsigned long long* sum = (unsigned long long*)(base + o_sum);
+    int* wide = (int*)(base + o_wide);
     LSQ_CUDA(cudaMemsetAsync(mx, 0, 8 * (size_t)n, st));
+    LSQ_CUDA(cudaMemsetAsync(sum, 0, o_q - o_sum, st));   // and no tile marked
     k_oz_weight<<<(unsigned)std::min<int64_t>((s + 255) / 256, 4096), 256, 0, st>>>(p, s, rg);
     k_oz_max<DT><<<(unsigned)((s + 31) / 32), 256, 0, st>>>(*A, idx, rg, inv_d, s, mx);
     k_oz_exp<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(mx, inv_d, n, e, sd);
@@ -307,9 +426,16 @@ static lsq_status normal_matrix(const lsq_matrix* A, const int32_t* idx, const d
             *A, idx, rg, sd, e, s, t0, rows, npad, q);
         // every split runs in every chunk (a split past the chunk's rows adds nothing)
         k_oz_gemm<<<dim3((unsigned)tiles, (unsigned)splits), OZ_T, smem, st>>>(
-            reinterpret_cast<const unsigned short*>(q), rows, npad, n, e, per, ntile, part, t0 > 0 ? 1 : 0);
-        count_launch(2);
+            reinterpret_cast<const unsigned short*>(q), rows, npad, n, e, per, ntile, part, mag, t0 > 0 ? 1 : 0);
+        k_oz_sums<<<(unsigned)((rows + 63) / 64), 256, 0, st>>>(
+            reinterpret_cast<const unsigned short*>(q) + OZ_P * rows * npad, rows, npad, n, sum);
+        count_launch(3);
     }
+    k_wide_check<<<(unsigned)std::min<int64_t>((n * n + 255) / 256, 152 * 16), 256, 0, st>>>(n, s, (int)splits, ntile, mag,
+                                                                                            sum, e, wide);
+    k_wide_tiles<DT><<<dim3((unsigned)tiles, (unsigned)splits), 256, 0, st>>>(
+        *A, idx, p, inv_d, s, ((s + splits - 1) / splits + OZ_KC - 1) / OZ_KC * OZ_KC, ntile, wide, part);
+    count_launch(2);
     k_reduce_M<<<(unsigned)std::min<int64_t>((n * n + 255) / 256, 152 * 16), 256, 0, st>>>(n, (int)splits, part, M, n_fixed);
     count_launch();
     LSQ_CUDA(cudaGetLastError());
