@@ -50,6 +50,7 @@ struct SpArgs {
     int64_t cl_f, cl_b;         // level count when that direction runs in one cluster, else 0
     int64_t nlev_f, nlev_b;     // level counts of the two schedules
     const void* inv;            // inverted diagonal blocks when the sweeps run by blocks, else NULL
+    int inv64;
     const double* mval64;
     int cl_lg;                  // log2 of that cluster's size
     int lpr, lpc;               // lanes per row of A, lanes per column of A (powers of two <= 32)
@@ -871,7 +872,7 @@ static lsq_status launch_sweep(const SpArgs& a, const double* r, const double* e
         count_launch();
         SbArgs b{};
         b.n = a.n; b.K = 1; b.mptr = a.mptr; b.mcol = a.mcol; b.mval = a.mval; b.mdiag = a.mdiag;
-        b.mval64 = a.mval64; b.inv = a.inv; b.done = &a.S->done; b.err = &a.S->err; b.max_polls = a.max_polls;
+        b.mval64 = a.mval64; b.inv = a.inv; b.inv64 = a.inv64; b.done = &a.S->done; b.err = &a.S->err; b.max_polls = a.max_polls;
         b.r = r; b.e_old = eold; b.e_new = enew; b.out64 = out64; b.identity = identity;
         b.S = check ? a.S : nullptr; b.part = a.part + a.rblk; b.nparts = nparts;
         b.tol = a.tol; b.inner_tol = a.inner_tol; b.maxit = a.maxit;
@@ -926,6 +927,7 @@ static void choose_sweep_form(SpArgs& a, const SparseHandle* SH, int64_t n) {
     const int form = g_sweep_form.load(std::memory_order_relaxed);
     const bool fits = 8 * ((n + (1 << SC_LG) - 1) >> SC_LG) <= SC_SMEM;
     a.inv = form == 0 && sb_use(SH) ? SH->inv : nullptr;
+    a.inv64 = SH->inv64;
     a.mval64 = SH->mval;
     a.cl_lg = SC_LG;
     auto pick = [&](int64_t nlev, int64_t& one, int64_t& clv) {

@@ -443,10 +443,7 @@ static lsq_status bk_solve_impl(const lsq_matrix* A, const lsq_precond* P, const
         else k_bk_cols<DT><<<gcols, BK_T, 0, st>>>(a, 0, dst);
         count_launch();
     };
-    // the sweep form follows the mean length of a row's dependency side: lane per column up to
-    // 24 entries, lane per entry up to 96, a CTA per row beyond
-    const double dep = (double)(SH->nnz_M - n) / (2.0 * (double)n);
-    const int smode = dep > 96.0 ? 2 : (dep > 24.0 ? 1 : 0);
+    const int smode = block_sweep_mode(SH->nnz_M, n);
     const bool m32 = P->op_dtype == LSQ_F32;
     // one cluster on request (lsq_set_sweep_form 3) where the block vector fits in the
     // cluster's shared memory; the stream-ordered solve only (the persistent kernel keeps the
@@ -483,7 +480,7 @@ static lsq_status bk_solve_impl(const lsq_matrix* A, const lsq_precond* P, const
             count_launch();
             SbArgs b{};
             b.n = n; b.K = K; b.mptr = a.mptr; b.mcol = a.mcol; b.mval = a.mval; b.mdiag = a.mdiag;
-            b.mval64 = SH->mval; b.inv = SH->inv; b.done = &S->done; b.err = &S->err; b.max_polls = a.max_polls;
+            b.mval64 = SH->mval; b.inv = SH->inv; b.inv64 = SH->inv64; b.done = &S->done; b.err = &S->err; b.max_polls = a.max_polls;
             b.r = r; b.e_old = eold; b.e_new = enew; b.out64 = out64; b.identity = identity;
             q = sb_launch(b, fwd, m32, pairs, st);
         } else if (fwd && cl_f) q = bk_launch_sweep_cl(cf, a, r, eold, enew, identity, SH->loff_f, SH->nlev_f, st);

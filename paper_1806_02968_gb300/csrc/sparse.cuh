@@ -20,14 +20,22 @@ struct SparseHandle {
     int64_t* loff_f = nullptr;    // first schedule slot of every level (nlev + 1 entries)
     int64_t* loff_b = nullptr;
     // inverses of the 128-row lower diagonal blocks (sweep_blocked.cu), where the schedule is
-    // deep; NULL otherwise
+    // deep; NULL otherwise.  Doubles where any sweep of the handle sums in FP64, else float pairs.
     void* inv = nullptr;
+    bool inv64 = false;
     // transposed pattern of A: column pointers, row indices, source entry of each
     int64_t* atptr = nullptr;
     int32_t* atrow = nullptr;
     int64_t* atperm = nullptr;
 };
 
+// The sweep of a block of right-hand sides follows the mean length of a row's dependency side: 0 a
+// lane per column up to 24 entries, 1 a lane per entry up to 96, 2 a CTA per row beyond.  FP32 M is
+// summed in double-float by 2 and in FP64 by 0 and 1.
+inline int block_sweep_mode(int64_t nnz_M, int64_t n) {
+    const double dep = (double)(nnz_M - n) / (2.0 * (double)n);
+    return dep > 96.0 ? 2 : (dep > 24.0 ? 1 : 0);
+}
 lsq_status scan_i64(const int64_t* in, int64_t n, int64_t* out, int64_t* scratch, cudaStream_t st);
 lsq_status transpose_pattern(const int64_t* rptr, const int32_t* col, int64_t nr, int64_t nc, int64_t nnz,
                              int64_t* cptr, int32_t* trow, int64_t* tperm, cudaStream_t st);

@@ -831,6 +831,7 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
     LSQ_CUDA(cudaMemcpyAsync(&nf, nfix, 8, cudaMemcpyDeviceToHost, st));
     LSQ_CUDA(cudaGetLastError());
     LSQ_CUDA(cudaStreamSynchronize(st));
+    S->nnz_M = mnnz;
     // 4. level schedules of the forward and backward sweeps (device)
     r = device_levels(S, n, mnnz, st);
     if (r != LSQ_OK) return r;
@@ -848,7 +849,6 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
     H->n_fixed_diag = (int64_t)nf;
     H->nnz_M = mnnz;
     H->levels = S->nlev_f;
-    S->nnz_M = mnnz;
     S->n_unique = nu;
     return LSQ_OK;
 }

@@ -99,8 +99,7 @@ struct SbDouble {
     static __device__ __forceinline__ V neg(V v) { return -v; }
 };
 
-// MT: type of M's values; AR: arithmetic; INV: element of the inverse (f2 pairs for float M,
-// double otherwise); B rows per block, KC columns per CTA.  Thread (row, h, c) of the 512 owns
+// MT: type of M's values; AR: arithmetic; B rows per block, KC columns per CTA.  Thread (row, h, c) of the 512 owns
 // entries h, h + ES, ... of its row for column c.
 template <typename MT, typename AR, bool FWD, int B, int KC>
 __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
@@ -166,10 +165,9 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
             for (int t = 0; t < PER; ++t) {
                 const int ci = sub + h + ES * t;
                 const int64_t e = at + (FWD ? (int64_t)ri * SB_ROWS + ci : (int64_t)ci * SB_ROWS + ri);
-                if constexpr (sizeof(MT) == 4) {
-                    const f2 p = reinterpret_cast<const f2*>(a.inv)[e];
-                    if constexpr (std::is_same<AR, SbPair>::value) inv[t] = p;
-                    else inv[t] = df_to_double(p);
+                if constexpr (std::is_same<AR, SbPair>::value) {
+                    if (!a.inv64) inv[t] = reinterpret_cast<const f2*>(a.inv)[e];
+                    else inv[t] = df_from_double(reinterpret_cast<const double*>(a.inv)[e]);
                 } else {
                     inv[t] = reinterpret_cast<const double*>(a.inv)[e];
                 }
@@ -344,8 +342,9 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
 // Inverses of the 128-row lower diagonal blocks D + L of M: the block in shared memory (M's
 // entries, the identity beyond n), inverted in place from the last column to the first
 // (column j of the inverse is -X_sub l_j / l_jj with X_sub the inverse of the rows below),
-// four threads per row.  FP64 throughout; FP32 M (whose sweeps use the FP32-rounded
-// off-diagonal entries and the FP64 diagonal) gets them as float pairs.
+// four threads per row.  FP64 throughout, from the FP32-rounded off-diagonal entries and the FP64
+// diagonal for FP32 M.  Stored as doubles, or as float pairs where every sweep that uses them runs in
+// double-float.
 // Bound: FP64 instructions (350 k FMAs per block and as many lanes again in the row reductions; the
 // reciprocals of the diagonal are formed once: a division per thread and column took most of the
 // time).  313 blocks: 0.71 ms, against
@@ -357,7 +356,7 @@ constexpr size_t SI_SMEM = (size_t)SB_ROWS * SI_LD * 8;
 template <typename MT>
 __global__ void __launch_bounds__(SI_T, 1) k_block_inverse(int64_t n, const int64_t* mptr, const int32_t* mcol,
                                                            const MT* mval, const double* mval64,
-                                                           const int64_t* mdiag, void* inv) {
+                                                           const int64_t* mdiag, void* inv, int inv64) {
     extern __shared__ __align__(16) double s_a[];   // SB_ROWS x SI_LD, row-major
     __shared__ double s_l[SB_ROWS], s_rd[SB_ROWS];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -401,8 +400,8 @@ __global__ void __launch_bounds__(SI_T, 1) k_block_inverse(int64_t n, const int6
         for (int t = tid; t < SB_ROWS * SB_ROWS; t += SI_T) {
             const double v = s_a[(t / SB_ROWS) * SI_LD + t % SB_ROWS];
             const int64_t at = (int64_t)b * SB_ROWS * SB_ROWS + t;
-            if (sizeof(MT) == 4) reinterpret_cast<f2*>(inv)[at] = df_from_double(v);
-            else reinterpret_cast<double*>(inv)[at] = v;
+            if (inv64) reinterpret_cast<double*>(inv)[at] = v;
+            else reinterpret_cast<f2*>(inv)[at] = df_from_double(v);
         }
         __syncthreads();
     }
@@ -644,13 +643,14 @@ lsq_status sb_build_inverse(SparseHandle* S, int64_t n, bool m32, cudaStream_t s
     // by blocks when the chain of blocks is shorter than the level schedule
     if (nblk > levels) return LSQ_OK;
     LSQ_CUDA(pool_alloc(&S->inv, 8 * (size_t)nblk * SB_ROWS * SB_ROWS, st));
+    S->inv64 = !m32 || block_sweep_mode(S->nnz_M, n) == 1;
     const unsigned g = (unsigned)std::min<int64_t>(nblk, 1 << 20);
     if (m32) {
         LSQ_CUDA(cudaFuncSetAttribute(k_block_inverse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SI_SMEM));
-        k_block_inverse<float><<<g, SI_T, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval32, S->mval, S->mdiag, S->inv);
+        k_block_inverse<float><<<g, SI_T, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval32, S->mval, S->mdiag, S->inv, S->inv64);
     } else {
         LSQ_CUDA(cudaFuncSetAttribute(k_block_inverse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SI_SMEM));
-        k_block_inverse<double><<<g, SI_T, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval, S->mval, S->mdiag, S->inv);
+        k_block_inverse<double><<<g, SI_T, SI_SMEM, st>>>(n, S->mptr, S->mcol, S->mval, S->mval, S->mdiag, S->inv, 1);
     }
     count_launch();
     LSQ_CUDA(cudaGetLastError());

@@ -23,7 +23,8 @@ struct SbArgs {
     const void* mval;          // float or double (the operator's type)
     const int64_t* mdiag;
     const double* mval64;      // FP64 values (the diagonal)
-    const void* inv;           // inverses of the lower diagonal blocks: pairs for float M, else double
+    const void* inv;           // inverses of the lower diagonal blocks
+    int inv64;                 // they are doubles; else float pairs (double-float sums only)
     const int32_t* done;       // nothing to do once set
     unsigned* err;
     unsigned max_polls;
