@@ -913,8 +913,8 @@ static lsq_status launch_sweep(const SpArgs& a, const double* r, const double* e
     return LSQ_OK;
 }
 
-// The sweep form of each direction.  By shape (form 0): by blocks of rows where the handle
-// holds the inverted blocks (sb_build_inverse); otherwise one CTA when a level holds fewer than
+// The sweep form of each direction.  By shape (form 0): by blocks of rows where that is the faster
+// form (sb_pays); otherwise one CTA when a level holds fewer than
 // 2048 dependency entries on average: block barriers between levels are then cheaper than a
 // grid of warps polling for the values they depend on, and one SM's loads still keep up with
 // a level's gathers (at ~10,000 entries per level one SM is twice slower than the grid);
@@ -926,7 +926,7 @@ static void choose_sweep_form(SpArgs& a, const SparseHandle* SH, int64_t n) {
     const double dep = 0.5 * (double)(SH->nnz_M - n);   // dependency entries per direction
     const int form = g_sweep_form.load(std::memory_order_relaxed);
     const bool fits = 8 * ((n + (1 << SC_LG) - 1) >> SC_LG) <= SC_SMEM;
-    a.inv = form == 0 && sb_use(SH) ? SH->inv : nullptr;
+    a.inv = form == 0 && sb_use(SH, n, 1, a.mval != (const void*)SH->mval) ? SH->inv : nullptr;
     a.inv64 = SH->inv64;
     a.mval64 = SH->mval;
     a.cl_lg = SC_LG;

@@ -463,10 +463,10 @@ static lsq_status bk_solve_impl(const lsq_matrix* A, const lsq_precond* P, const
     // last sweep also writing z in FP64 (a dependent FP64 step costs ~64 cycles on GB300);
     // the cluster and persistent forms keep FP64 sums
     const bool pairs = m32 && smode == 2 && !cl_f && !cl_b;
-    // by shape, deep level schedules run by blocks of rows (the same arithmetic: pairs where
-    // the CTA-per-row form uses them, FP64 sums otherwise).  Short rows (graphs) stay with the
+    // by shape, deep level schedules run by blocks of rows where that is faster (the same arithmetic:
+    // pairs where the CTA-per-row form uses them, FP64 sums otherwise).  Short rows (graphs) stay with the
     // lane-per-column form, whose bits the persistent kernel shares.
-    const bool blocked = form == 0 && smode > 0 && sb_use(SH);
+    const bool blocked = form == 0 && smode > 0 && sb_use(SH, n, K, m32);
     const void* kf = pairs ? bk_sweep_kernel<float, true, true>(smode, K)
                            : (m32 ? bk_sweep_kernel<float, true>(smode, K) : bk_sweep_kernel<double, true>(smode, K));
     const void* kb = pairs ? bk_sweep_kernel<float, false, true>(smode, K)

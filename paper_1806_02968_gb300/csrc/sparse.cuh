@@ -19,10 +19,13 @@ struct SparseHandle {
     int64_t nlev_f = 0, nlev_b = 0;
     int64_t* loff_f = nullptr;    // first schedule slot of every level (nlev + 1 entries)
     int64_t* loff_b = nullptr;
-    // inverses of the 128-row lower diagonal blocks (sweep_blocked.cu), where the schedule is
-    // deep; NULL otherwise.  Doubles where any sweep of the handle sums in FP64, else float pairs.
+    // inverses of the 128-row lower diagonal blocks (sweep_blocked.cu) where some sweep of the handle
+    // runs by blocks (sb_pays) and memory allowed it; NULL otherwise.  Doubles where any sweep of the handle sums in FP64, else float pairs.
     void* inv = nullptr;
     bool inv64 = false;
+    // mean entries of a row in the 64- (128-) row block before its own: those a block of the blocked
+    // sweeps still has to add up when the one before it is done
+    double near64 = 0.0, near128 = 0.0;
     // transposed pattern of A: column pointers, row indices, source entry of each
     int64_t* atptr = nullptr;
     int32_t* atrow = nullptr;

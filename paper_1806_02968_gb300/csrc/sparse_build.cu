@@ -835,8 +835,10 @@ lsq_status build_sparse(const lsq_matrix* A, const int32_t* idx, const double* p
     // 4. level schedules of the forward and backward sweeps (device)
     r = device_levels(S, n, mnnz, st);
     if (r != LSQ_OK) return r;
-    r = sb_build_inverse(S, n, H->op_dtype == LSQ_F32, st);
-    if (r != LSQ_OK) return r;
+    if (H->sweeps > 0) {   // t = 0 (the identity) sweeps nothing
+        r = sb_build_inverse(S, n, H->op_dtype == LSQ_F32, st);
+        if (r != LSQ_OK) return r;
+    }
     // 5. transposed pattern of A for the A^T q pass (values are gathered at solve time)
     LSQ_CUDA(pool_alloc(&S->atptr, 8 * (size_t)(n + 1), st));
     LSQ_CUDA(pool_alloc(&S->atrow, 4 * (size_t)A->nnz, st));

@@ -637,12 +637,96 @@ lsq_status sb_launch(const SbArgs& a, bool fwd, bool m32, bool pairs, cudaStream
     return LSQ_OK;
 }
 
+// The rule: a sweep by blocks takes nblk steps of t_blk, or, with many blocks, the time in which
+// the resident CTAs walk all blocks before their own (0.75 us for every four); a sweep by rows takes
+// nlev levels of t_row.  Times in us, measured on layers of 40 to 128 nodes with 2 to 110
+// dependencies each, 10,000 to 1,000,000 rows:
+//   t_blk = base + slope * (entries of a thread in the block before its own),
+//   t_row  one column: 1.9 (FP64) or 1.3 (FP32 M) on the grid, 1.2 + 0.22 w or 1.1 + 0.125 w in one CTA,
+//          where levels of w rows hold less than 2048 entries; K columns: about 3.5 + 0.14 K with a CTA
+//          per row, 2.4 + 0.5 K and, from 4 on, more with the row's length, with a lane per entry.
+// At 1,000,000 rows in 10,000 layers of 100, short rows, the walk is the longer of the two (145 ms a sweep
+// in FP64, 235 ms in one CTA); at 102,400 rows of 60 dependencies in 1600 layers rows are the
+// better form (3.5 ms, blocks 6.5 ms); at 40,000 rows of 380 random dependencies (1583 levels) blocks
+// are (0.54 ms, rows 1.75 and 3.5 ms).
+bool sb_pays(const SparseHandle* S, int64_t n, int K, bool m32) {
+    const double levels = (double)std::min(S->nlev_f, S->nlev_b), dep = (double)(S->nnz_M - n) / (2.0 * (double)n);
+    const int mode = block_sweep_mode(S->nnz_M, n);
+    if (K > 1 && mode == 0) return false;
+    const bool pair = m32 && (K == 1 || mode == 2);
+    const int B = K == 1 && pair ? 128 : 64, KC = K == 1 ? 1 : (K == 2 ? 2 : 4), at = KC == 1 ? 0 : (KC == 2 ? 1 : 2);
+    static const double base[2][3] = {{2.95, 3.6, 5.4}, {1.75, 2.2, 2.5}};
+    static const double slope[2][3] = {{0.145, 0.18, 0.26}, {0.18, 0.13, 0.23}};
+    const double nblk = (double)((n + B - 1) / B), groups = (double)((K + KC - 1) / KC);
+    const double entries = (B == 128 ? S->near128 : S->near64) * (double)(B * KC) / (double)SB_T;
+    const double t_blk = std::max(base[pair][at] + slope[pair][at] * entries, 0.75 * nblk * groups / (4.0 * 2.0 * 152.0));
+    double t_row;
+    if (K == 1) {
+        const double w = (double)n / levels;
+        if (dep * w < 2048.0) t_row = m32 ? 1.1 + 0.125 * w : 1.2 + 0.22 * w;
+        else t_row = m32 ? 1.3 : 1.9;
+    } else if (mode == 2) {
+        t_row = 3.5 + 0.14 * K;
+    } else {
+        t_row = K <= 4 ? 2.4 + 0.5 * K : 4.4 + (K - 4) * (0.25 + 0.0095 * dep);
+    }
+    return nblk * t_blk <= levels * t_row;
+}
+
+// sums over the rows of their entries in the 64-row (sum[0]) and 128-row (sum[1]) block before their own
+__global__ void k_near_entries(int64_t n, const int64_t* mptr, const int32_t* mcol, const int64_t* mdiag,
+                               unsigned long long* sum) {
+    int c[2] = {0, 0};
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t p0 = mptr[j], pd = mdiag[j];
+        auto first_at = [&](int64_t col) {   // rows are sorted
+            int64_t lo = p0, hi = pd;
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (mcol[mid] < col) lo = mid + 1;
+                else hi = mid;
+            }
+            return lo;
+        };
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int64_t B = 64 << q, b0 = j / B * B;
+            c[q] += (int)(first_at(b0) - first_at(b0 - B));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int t = warp_sum(c[q]);
+        if ((threadIdx.x & 31) == 0 && t) atomicAdd(&sum[q], (unsigned long long)t);
+    }
+}
+
 lsq_status sb_build_inverse(SparseHandle* S, int64_t n, bool m32, cudaStream_t st) {
+    auto any = [&] {
+        return sb_pays(S, n, 1, m32) || sb_pays(S, n, 2, m32) || sb_pays(S, n, 4, m32) || sb_pays(S, n, 16, m32) ||
+               sb_pays(S, n, 32, m32);
+    };
+    if (!any()) return LSQ_OK;   // not even without entries in the block before
+    {
+        Scratch sc;
+        LSQ_CUDA(sc.alloc(16, st));
+        LSQ_CUDA(cudaMemsetAsync(sc.ptr, 0, 16, st));
+        k_near_entries<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, st>>>(
+            n, S->mptr, S->mcol, S->mdiag, sc.as<unsigned long long>());
+        count_launch();
+        unsigned long long sum[2] = {0, 0};
+        LSQ_CUDA(cudaMemcpyAsync(sum, sc.ptr, 16, cudaMemcpyDeviceToHost, st));
+        LSQ_CUDA(cudaStreamSynchronize(st));
+        S->near64 = (double)sum[0] / (double)n;
+        S->near128 = (double)sum[1] / (double)n;
+    }
+    if (!any()) return LSQ_OK;
     const int64_t nblk = (n + SB_ROWS - 1) / SB_ROWS;
-    const int64_t levels = S->nlev_f < S->nlev_b ? S->nlev_f : S->nlev_b;
-    // by blocks when the chain of blocks is shorter than the level schedule
-    if (nblk > levels) return LSQ_OK;
-    LSQ_CUDA(pool_alloc(&S->inv, 8 * (size_t)nblk * SB_ROWS * SB_ROWS, st));
+    if (pool_alloc(&S->inv, 8 * (size_t)nblk * SB_ROWS * SB_ROWS, st) != cudaSuccess) {
+        cudaGetLastError();
+        S->inv = nullptr;
+        return LSQ_OK;
+    }
     S->inv64 = !m32 || block_sweep_mode(S->nnz_M, n) == 1;
     const unsigned g = (unsigned)std::min<int64_t>(nblk, 1 << 20);
     if (m32) {

@@ -41,13 +41,17 @@ struct SbArgs {
     int32_t maxit;
 };
 
-// True when the sweeps of this handle run by blocks (its schedule is deep enough and the
-// inverted blocks were built).
-inline bool sb_use(const SparseHandle* S) { return S->inv != nullptr; }
+// True where sweeps over K columns are expected to take less time by blocks than by rows.
+bool sb_pays(const SparseHandle* S, int64_t n, int K, bool m32);
+// True when sweeps over K columns of this handle run by blocks.
+inline bool sb_use(const SparseHandle* S, int64_t n, int K, bool m32) {
+    return S->inv != nullptr && sb_pays(S, n, K, m32);
+}
 // One sweep in the arithmetic of the operator type: FP32 M with pairs = true in double-float
 // (vectors hold pairs), otherwise FP64 sums.  The caller has filled e_new with SB_EMPTY.
 lsq_status sb_launch(const SbArgs& a, bool fwd, bool m32, bool pairs, cudaStream_t st);
-// The inverted diagonal blocks of a handle whose M is complete (no-op where they would not pay).
+// The inverted diagonal blocks of a handle whose M and levels are complete: none where no number of
+// columns takes the block form, or where there is no memory for them (the row forms need none).
 lsq_status sb_build_inverse(SparseHandle* S, int64_t n, bool m32, cudaStream_t st);
 // lev1[j] = level + 1 of every row for the forward (lev1_f) and backward (lev1_b) dependencies,
 // both zero on entry; *max_f, *max_b the deepest levels.  By blocks, both directions at once.

@@ -68,3 +68,56 @@ def test_fp32_m_summed_in_fp64_uses_fp64_inverses(lsq, form, k):
     assert not by_blocks(solve)
     X1 = solve()
     assert float(((X0 - X1).abs() / X1.abs()).max()) <= 9 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("layers,width,reach,dtype,k,blocks", [
+    (200, 8, 1, 0, 1, True),        # narrow levels: 25 blocks of 64 rows against 200 levels in one CTA
+    (200, 60, 1, 0, 1, False),      # 188 blocks against 200 levels of 3600 entries on the grid
+    (200, 60, 1, 1, 1, False),
+    (200, 60, 1, 0, 2, False),
+    (200, 60, 1, 0, 16, True),      # a lane per entry: wide levels cost more than a block
+    (100, 110, 1, 0, 16, False),    # 172 blocks against 100 levels, a CTA per row
+    (400, 16, 8, 1, 16, True),      # 100 blocks against 400 levels
+])
+def test_form_follows_the_cost_of_blocks_and_levels(lsq, layers, width, reach, dtype, k, blocks):
+    A, P = layered(lsq, layers, width, reach, coupling=0.1, precond_dtype=dtype)
+    if k == 1:
+        r = torch.ones(A.n, dtype=torch.float64, device="cuda")
+        assert by_blocks(lambda: P.apply(r)) == blocks
+    else:
+        B = torch.ones(k, A.m, dtype=torch.float64, device="cuda")
+        assert by_blocks(lambda: lsq.lsq_pcg_solve(A, P, B, lsq.opts(maxit=1, max_outer=1))) == blocks
+
+
+def test_t0_builds_no_inverses(lsq):
+    assert any("k_block_inverse" in x for x in kernels(lambda: layered(lsq, 200, 8, 1)))
+    assert not any("k_block_inverse" in x for x in kernels(lambda: layered(lsq, 200, 8, 1, sweeps=0)))
+
+
+def test_no_memory_for_the_inverses_leaves_the_row_forms(lsq):
+    """3,000,000 rows in layers of 8 would take 3 GB of inverses; with 1.5 GB left the handle is built all
+    the same and applies by rows."""
+    n, width = 3000000, 8
+    node = torch.arange(width, n, device="cuda")
+    e = node.numel()
+    rp = torch.cat([torch.arange(n, device="cuda"), n + 2 * torch.arange(e + 1, device="cuda")])
+    ci = torch.cat([torch.arange(n, device="cuda"), torch.stack([node - width, node], 1).reshape(-1)]).to(torch.int32)
+    va = torch.ones(n + 2 * e, dtype=torch.float64, device="cuda")
+    va[n + 1::2] = -1.0
+    A = lsq.Matrix(row_ptr=rp, col_idx=ci, vals=va, n=n)
+    args = (torch.arange(A.m, dtype=torch.int32, device="cuda"),
+            torch.full((A.m,), 1.0 / A.m, dtype=torch.float64, device="cuda"), torch.ones(n, dtype=torch.float64, device="cuda"))
+    o = lsq.opts(precond_dtype=1)
+    r = torch.randn(n, dtype=torch.float64, device="cuda")
+    P = lsq.lsq_build_precond(A, *args, o)
+    assert by_blocks(lambda: P.apply(r))
+    E = P.apply(r)
+    del P
+    torch.cuda.empty_cache()
+    fill, left = [], 3 << 29
+    while torch.cuda.mem_get_info()[0] > left + (1 << 28):
+        fill.append(torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda"))
+    P = lsq.lsq_build_precond(A, *args, o)
+    del fill
+    assert not by_blocks(lambda: P.apply(r))
+    assert float((P.apply(r) - E).norm() / E.norm()) <= 1e-10
