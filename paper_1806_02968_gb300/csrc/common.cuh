@@ -181,6 +181,42 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* bar, unsigned n
     return s_ok != 0;
 }
 
+// Rows far longer than the others, set aside by a pass that gives every row a few lanes: the whole CTA
+// (of at most 8 warps) takes them one after the other when it is through with its own.  Every warp keeps
+// its own list, so what is set aside does not depend on timing; where the list is full a row stays with
+// its lanes.
+constexpr int LONG_CAP = 64;       // rows a warp sets aside at most
+constexpr int LONG_ROW = 1024;     // entries from which a row counts as long (passes raise it with their lanes)
+struct LongRows {
+    int n[8];
+    int64_t row[8][LONG_CAP];
+    __device__ __forceinline__ void init() {
+        if ((threadIdx.x & 31) == 0) n[threadIdx.x >> 5] = 0;
+        __syncwarp();
+    }
+    // Called by a whole warp, `want` in one lane of a row's L (a power of two): true in all lanes of a row
+    // that was taken.
+    __device__ __forceinline__ bool put(bool want, int64_t r, int L) {
+        const unsigned mask = __ballot_sync(0xffffffffu, want);
+        if (!mask) return false;
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, had = n[w];
+        const int at = had + __popc(mask & ((1u << lane) - 1u));
+        const bool took = want && at < LONG_CAP;
+        if (took) row[w][at] = r;
+        __syncwarp();
+        if (lane == 0) n[w] = min(had + __popc(mask), LONG_CAP);
+        __syncwarp();
+        return (__ballot_sync(0xffffffffu, took) >> (lane & ~(L - 1))) & (L == 32 ? 0xffffffffu : (1u << L) - 1u);
+    }
+    // f(row) for every row set aside, by the whole CTA
+    template <typename F>
+    __device__ __forceinline__ void each(F f) {
+        __syncthreads();
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+            for (int q = 0; q < n[w]; ++q) f(row[w][q]);
+    }
+};
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll

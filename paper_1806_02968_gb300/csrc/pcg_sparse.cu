@@ -20,6 +20,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 namespace lsq {
 
@@ -91,21 +92,6 @@ __device__ __forceinline__ double sum_parts(const double* part, int cnt, double*
 
 constexpr int SP_T = 256;
 enum { SPM_MATVEC = 0, SPM_RHS = 1, SPM_RESID = 2 };
-
-// an FP32 or BF16 value as FP32
-template <int DT>
-__device__ __forceinline__ float load_f32(const void* p, int64_t e) {
-    if constexpr (DT == LSQ_BF16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[e]);
-    else return reinterpret_cast<const float*>(p)[e];
-}
-
-// a value as FP64 by the hardware's conversion, for a pass that waits on memory and has FP64 slots
-// to spare (one column: 0.162 ms per column pass of 3.2e7 entries, 0.190 ms with integer widening)
-template <int DT>
-__device__ __forceinline__ double load_f64(const void* p, int64_t e) {
-    if constexpr (DT == LSQ_F32 || DT == LSQ_BF16) return (double)load_f32<DT>(p, e);
-    else return Val<DT>::load(p, e);
-}
 
 // q_i = sum_e a_e x_{col e} (x = D^{-1} p or D^{-1} y), or b_i, or b_i - that.  A group of
 // LPR lanes (a power of two, about the mean row length) takes 4 consecutive rows per step and
@@ -1250,14 +1236,22 @@ lsq_status sparse_apply(const lsq_precond* P, const double* r, double* e, int64_
 // so a group gathers one line per entry), then grad[e] (+)= sum_c r_c lambda_jc - (A lambda)_c x_jc
 // for the row's entries, eight at a time: their sums over the group share one reduce-scatter.
 // Bound: FP64 operations, five per entry and column.  1e6 x 10,000 with 16 columns, FP32 values:
-// 1.24 ms, against 6.3 ms by two products per column and a pass over all columns.
+// 1.24 ms, against 6.3 ms by two products per column and a pass over all columns.  Rows of more than
+// `lng` entries (far more than the mean) are set aside for the whole CTA, whose groups take every so many
+// of their batches (1e6 rows of 2 entries and 20 of 50,000 side by side, one column: 2 ms, 17 ms with two
+// lanes to every row).
 constexpr int AJ_E = 8;
 template <int DT, int GK>
 __global__ void __launch_bounds__(SP_T) k_csr_adjoint(int64_t m, const int64_t* rp, const int32_t* ci, const void* vals,
                                                       const double* lam, const double* x, int kc, const double* b,
-                                                      int64_t ldb, double* al_out, double* grad, int accumulate) {
+                                                      int64_t ldb, double* al_out, double* grad, int accumulate,
+                                                      int64_t lng) {
+    constexpr int GROUPS = SP_T / GK;   // of a CTA
+    __shared__ LongRows s_long;
+    __shared__ double s_sum[2][SP_T / 32][GK];
     const int c = threadIdx.x & (GK - 1);
-    const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / GK;
+    // the warps of a CTA take rows far from one another, so that long rows side by side go to several CTAs
+    const int64_t grp = (((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31)) / GK;
     const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) / GK;
     const bool on = c < kc;
     // one batch of the row's entries: columns, values, and this lane's lambda and x
@@ -1271,14 +1265,14 @@ __global__ void __launch_bounds__(SP_T) k_csr_adjoint(int64_t m, const int64_t* 
             xv[u] = in ? x[(int64_t)col[u] * kc + c] : 0.0;
         }
     };
-    // the trip count is the same for every group of a warp (the shuffles need all 32 lanes)
-    for (int64_t i0 = 0; i0 < m; i0 += ngrp) {
-        const int64_t i = i0 + grp;
-        const int64_t e0 = i < m ? rp[i] : 0, e1 = i < m ? rp[i + 1] : 0;
+    // Row i, entries [e0, e1), if `act`: batches part, part + PARTS, ...  The warp (with PARTS > 1 the CTA)
+    // calls this together, with the longest of its rows as len (every lane goes through the same shuffles).
+    auto row = [&](auto parts, bool act, int64_t i, int64_t e0, int64_t e1, int64_t len, int part) {
+        constexpr int PARTS = decltype(parts)::value;
         int32_t col[AJ_E];
         double lv[AJ_E], xv[AJ_E];
         double al = 0.0, ax = 0.0;
-        for (int64_t e = e0; e < e1; e += AJ_E) {
+        for (int64_t e = e0 + part * AJ_E; e < e1; e += PARTS * AJ_E) {
             batch(e, e1, col, lv, xv);
 #pragma unroll
             for (int u = 0; u < AJ_E; ++u) {
@@ -1289,18 +1283,28 @@ __global__ void __launch_bounds__(SP_T) k_csr_adjoint(int64_t m, const int64_t* 
                 }
             }
         }
-        double r = 0.0;
-        if (i < m && on) {
-            r = b[(int64_t)c * ldb + i] - ax;
-            if (al_out) al_out[(int64_t)c * ldb + i] = al;
-        }
-        if (!grad) continue;
-        int64_t len = e1 - e0;   // the longest row of the warp sets the number of batches
+        if constexpr (PARTS > 1) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) len = max(len, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)len, o));
-        for (int64_t k0 = 0; k0 < len; k0 += AJ_E) {
-            const int64_t e = e0 + k0;
-            if (len > AJ_E) batch(e, e1, col, lv, xv);   // else still in registers
+            for (int o = GK; o < 32; o <<= 1) {
+                al += __shfl_xor_sync(0xffffffffu, al, o);
+                ax += __shfl_xor_sync(0xffffffffu, ax, o);
+            }
+            if ((threadIdx.x & 31) < GK) { s_sum[0][threadIdx.x >> 5][c] = al; s_sum[1][threadIdx.x >> 5][c] = ax; }
+            __syncthreads();
+            al = 0.0; ax = 0.0;
+#pragma unroll
+            for (int v = 0; v < SP_T / 32; ++v) { al += s_sum[0][v][c]; ax += s_sum[1][v][c]; }
+            __syncthreads();
+        }
+        double r = 0.0;
+        if (act && on) {
+            r = b[(int64_t)c * ldb + i] - ax;
+            if (al_out && part == 0) al_out[(int64_t)c * ldb + i] = al;
+        }
+        if (!grad) return;
+        for (int64_t k0 = 0; k0 < len; k0 += PARTS * AJ_E) {
+            const int64_t e = e0 + k0 + part * AJ_E;
+            if (len > PARTS * AJ_E) batch(e, e1, col, lv, xv);   // else still in registers
             double t[AJ_E];
 #pragma unroll
             for (int u = 0; u < AJ_E; ++u) t[u] = e + u < e1 ? r * lv[u] - al * xv[u] : 0.0;
@@ -1329,7 +1333,23 @@ __global__ void __launch_bounds__(SP_T) k_csr_adjoint(int64_t m, const int64_t* 
             for (int u = 0; u < KEEP; ++u)
                 if (writer && e + first + u < e1) grad[e + first + u] = accumulate ? grad[e + first + u] + t[u] : t[u];
         }
+    };
+    s_long.init();
+    // the trip count is the same for every group of a warp (the shuffles need all 32 lanes)
+    for (int64_t i0 = 0; i0 < m; i0 += ngrp) {
+        const int64_t i = i0 + grp;
+        int64_t e0 = i < m ? rp[i] : 0, e1 = i < m ? rp[i + 1] : 0;
+        const bool aside = s_long.put(c == 0 && e1 - e0 > lng, i, GK);
+        if (aside) e1 = e0;
+        int64_t len = e1 - e0;   // the longest row of the warp sets the number of batches
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) len = max(len, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)len, o));
+        row(std::integral_constant<int, 1>{}, i < m && !aside, i, e0, e1, len, 0);
     }
+    s_long.each([&](int64_t i) {
+        const int64_t e0 = rp[i], e1 = rp[i + 1];
+        row(std::integral_constant<int, GROUPS>{}, true, i, e0, e1, e1 - e0, threadIdx.x / GK);
+    });
 }
 // column-major (leading dimension ld) -> row-major n x kc
 __global__ void k_cols_to_rows(const double* src, int64_t ld, int64_t n, int kc, double* dst) {
@@ -1368,9 +1388,10 @@ static lsq_status sp_adjoint_impl(const lsq_matrix* A, const lsq_precond* P, con
             k_cols_to_rows<<<gridn(n * kc), SP_T, 0, st>>>(X + c * ldx, ldx, n, kc, xr);
             const double* Bc = B + c * ldb;
             const int more = c > 0 ? 1 : 0;
+            const int64_t lng = std::max<int64_t>(LONG_ROW, 8 * (A->nnz / m));
             auto pass = [&](auto kern, int gk) {
                 kern<<<gridn(m * gk, 152 * 16), SP_T, 0, st>>>(m, A->row_ptr, A->col_idx, A->vals, lamr, xr, kc, Bc, ldb,
-                                                               gb, grad_vals, more);
+                                                               gb, grad_vals, more, lng);
             };
             if (kc <= 2) pass(k_csr_adjoint<DT, 2>, 2);
             else if (kc <= 4) pass(k_csr_adjoint<DT, 4>, 4);

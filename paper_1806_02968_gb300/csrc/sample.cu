@@ -186,51 +186,106 @@ __global__ void k_colscale(int64_t n, int normalize, const int* E1j, const unsig
 // S2: w_i = sum_j floor(2^51 fl(fl(a_ij^2) inv_d2_j)), a group of L lanes per row (about the mean
 // row length, a power of two up to a warp), exact.  Bound: two FP64 multiplications per entry at
 // two lanes a clock and SM, so every lane of a warp should hold an entry (4e6 rows of 8 entries:
-// 0.21 ms with 8 lanes per row, 0.84 ms with a warp per row).
+// 0.21 ms with 8 lanes per row, 0.84 ms with a warp per row).  Rows far longer than their lanes are set
+// aside for the whole CTA (sampling of 1e6 rows of 2 entries and 20 of 50,000 side by side: 0.58 ms, 4.5 ms
+// with two lanes to every row).
 // ---------------------------------------------------------------------------------------
+constexpr int RW_T = 256;
+__device__ __forceinline__ u128 group_sum_u128(u128 v, int lanes) {
+    for (int o = lanes >> 1; o > 0; o >>= 1) {
+        const unsigned long long lo = (unsigned long long)v, hi = (unsigned long long)(v >> 64);
+        const unsigned long long olo = __shfl_xor_sync(0xffffffffu, lo, o);
+        const unsigned long long ohi = __shfl_xor_sync(0xffffffffu, hi, o);
+        v += ((u128)ohi << 64) | olo;
+    }
+    return v;
+}
 template <int DT>
-__global__ void k_rowweight(lsq_matrix A, const double* inv_d2, u128* w, int uniform, int L) {
+__global__ void k_rowweight_dense(lsq_matrix A, const double* inv_d2, u128* w, int L) {
     const int lane = threadIdx.x & (L - 1);
     const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L;
     const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) / L;
     // the trip count is the same for every group of a warp (the shuffles need all 32 lanes)
     for (int64_t i0 = 0; i0 < A.m; i0 += ngrp) {
         const int64_t i = i0 + grp;
-        if (uniform) {   // the uniform density of the comparison in Sec. 3.1: w_i = 1
-            if (lane == 0 && i < A.m) w[i] = 1;
-            continue;
-        }
         u128 acc = 0;
-        if (i < A.m) {
-            if (A.dense) {
-                for (int64_t j = lane; j < A.n; j += L) {
-                    double a = Val<DT>::load(A.vals, i * A.ld + j);
-                    double u = __dmul_rn(__dmul_rn(a, a), inv_d2[j]);
-                    acc += floor_scaled(u, 51);
-                }
-            } else {
-                int64_t e0 = A.row_ptr[i], e1 = A.row_ptr[i + 1];
-                for (int64_t e = e0 + lane; e < e1; e += L) {
-                    double a = Val<DT>::load(A.vals, e);
-                    double u = __dmul_rn(__dmul_rn(a, a), inv_d2[A.col_idx[e]]);
-                    acc += floor_scaled(u, 51);
-                }
+        if (i < A.m)
+            for (int64_t j = lane; j < A.n; j += L) {
+                double a = Val<DT>::load(A.vals, i * A.ld + j);
+                double u = __dmul_rn(__dmul_rn(a, a), inv_d2[j]);
+                acc += floor_scaled(u, 51);
             }
-        }
-        for (int o = L >> 1; o > 0; o >>= 1) {
-            const unsigned long long lo = (unsigned long long)acc, hi = (unsigned long long)(acc >> 64);
-            const unsigned long long olo = __shfl_xor_sync(0xffffffffu, lo, o);
-            const unsigned long long ohi = __shfl_xor_sync(0xffffffffu, hi, o);
-            acc += ((u128)ohi << 64) | olo;
-        }
+        acc = group_sum_u128(acc, L);
         if (lane == 0 && i < A.m) w[i] = acc;
     }
 }
-// lanes per row of k_rowweight
-static int weight_lanes(const lsq_matrix* A) {
-    int L = 1;
-    while (L < 32 && (int64_t)L * A->m < (A->dense ? A->m * A->n : A->nnz)) L <<= 1;
-    return L;
+// The warps of a CTA take rows far from one another, so that long rows side by side go to several CTAs.
+// 32 registers, for as many warps as the SM takes (the pass waits on its gathers: 0.38 ms with 44).
+template <int DT>
+__global__ void __launch_bounds__(RW_T, 8) k_rowweight_csr(lsq_matrix A, const double* inv_d2, u128* w, int L) {
+    __shared__ LongRows s_long;
+    __shared__ u128 s_part[RW_T / 32];
+    const int lane = threadIdx.x & (L - 1), wid = threadIdx.x >> 5;
+    const int64_t grp = (((int64_t)wid * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31)) / L;
+    const int64_t ngrp = (int64_t)gridDim.x * RW_T / L;
+    const int64_t lng = 64 * L > LONG_ROW ? 64 * L : LONG_ROW;
+    s_long.init();
+    for (int64_t i0 = 0; i0 < A.m; i0 += ngrp) {
+        const int64_t i = i0 + grp;
+        int64_t e0 = i < A.m ? A.row_ptr[i] : 0, e1 = i < A.m ? A.row_ptr[i + 1] : 0;
+        const bool aside = s_long.put(lane == 0 && e1 - e0 > lng, i, L);
+        if (aside) e1 = e0;
+        u128 acc = 0;
+        for (int64_t e = e0 + lane; e < e1; e += L) {
+            double a = Val<DT>::load(A.vals, e);
+            double u = __dmul_rn(__dmul_rn(a, a), inv_d2[A.col_idx[e]]);
+            acc += floor_scaled(u, 51);
+        }
+        acc = group_sum_u128(acc, L);
+        if (lane == 0 && i < A.m && !aside) w[i] = acc;
+    }
+    s_long.each([&](int64_t i) {
+        const int64_t e1 = A.row_ptr[i + 1];
+        u128 acc = 0;
+        for (int64_t e = A.row_ptr[i] + threadIdx.x; e < e1; e += 4 * RW_T) {
+            double a[4], d[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = e + u * RW_T < e1;
+                a[u] = in ? load_f64<DT>(A.vals, e + u * RW_T) : 0.0;
+                d[u] = in ? inv_d2[A.col_idx[e + u * RW_T]] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc += floor_scaled(__dmul_rn(__dmul_rn(a[u], a[u]), d[u]), 51);
+        }
+        acc = group_sum_u128(acc, 32);
+        if ((threadIdx.x & 31) == 0) s_part[wid] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int v = 1; v < RW_T / 32; ++v) acc += s_part[v];
+            w[i] = acc;
+        }
+        __syncthreads();
+    });
+}
+// the uniform density of the comparison in Sec. 3.1: w_i = 1
+__global__ void k_rowweight_uniform(int64_t m, u128* w) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) w[i] = 1;
+}
+static int grid_for(int64_t work, int threads, int cap = 152 * 16) {
+    int64_t g = (work + threads - 1) / threads;
+    if (g < 1) g = 1;
+    if (g > cap) g = cap;
+    return (int)g;
+}
+template <int DT>
+static void launch_rowweight(const lsq_matrix& A, const double* inv_d2, u128* w, int uniform, cudaStream_t st) {
+    int L = 1;   // lanes per row
+    while (L < 32 && (int64_t)L * A.m < (A.dense ? A.m * A.n : A.nnz)) L <<= 1;
+    if (uniform) k_rowweight_uniform<<<grid_for(A.m, 256), 256, 0, st>>>(A.m, w);
+    else if (A.dense) k_rowweight_dense<DT><<<grid_for(A.m * L, 256), 256, 0, st>>>(A, inv_d2, w, L);
+    else k_rowweight_csr<DT><<<grid_for(A.m * L, RW_T), RW_T, 0, st>>>(A, inv_d2, w, L);
+    count_launch();
 }
 
 // ---------------------------------------------------------------------------------------
@@ -422,12 +477,6 @@ __global__ void k_draw_shard(const u128* P, int64_t m, int64_t row0, unsigned lo
     }
 }
 
-static int grid_for(int64_t work, int threads, int cap = 152 * 16) {
-    int64_t g = (work + threads - 1) / threads;
-    if (g < 1) g = 1;
-    if (g > cap) g = cap;
-    return (int)g;
-}
 
 // Scratch layout of one sampling call (256-byte aligned pieces; the first three are the
 // accumulating words that must start at zero).
@@ -489,13 +538,12 @@ static lsq_status sample_launch(const lsq_matrix* A, const lsq_opts* o, int64_t 
     if (A->dense) k_colsum_dense<DT><<<(int)((m + rpb - 1) / rpb), 256, 0, st>>>(Av, E1j, c, rpb);
     else k_colsum_csr<DT><<<grid_for(A->nnz, 256), 256, 0, st>>>(Av, E1j, c);
     k_colscale<<<grid_for(n, 256), 256, 0, st>>>(n, o->normalize ? 1 : 0, E1j, E1g, c, d2, inv, d);
-    const int wl = weight_lanes(A);
-    k_rowweight<DT><<<grid_for(m * wl, 256), 256, 0, st>>>(Av, inv, w, o->sampling == 1 ? 1 : 0, wl);
+    launch_rowweight<DT>(Av, inv, w, o->sampling == 1 ? 1 : 0, st);
     k_scan_tiles<<<(unsigned)ntiles, SCAN_THREADS, 0, st>>>(w, m, ts);
     k_scan_sums<<<1, 1024, 0, st>>>(ts, ntiles);
     k_scan_apply<<<(unsigned)ntiles, SCAN_THREADS, 0, st>>>(w, m, ts, P);
     k_draw<<<grid_for(s, 256), 256, 0, st>>>(P, m, s, (unsigned long long)o->seed, idx_out, p_out, err);
-    count_launch(9);
+    count_launch(8);
     LSQ_CUDA(cudaGetLastError());
     return read_dev_error(err, st);
 }
@@ -684,9 +732,7 @@ template <int DT> struct ColsumF {
 };
 template <int DT> struct WeightF {
     static lsq_status run(const lsq_matrix* A, const double* inv, u128* w, int uniform, cudaStream_t st) {
-        const int L = weight_lanes(A);
-        k_rowweight<DT><<<grid_for(A->m * L, 256), 256, 0, st>>>(*A, inv, w, uniform, L);
-        count_launch();
+        launch_rowweight<DT>(*A, inv, w, uniform, st);
         return LSQ_OK;
     }
 };

@@ -162,17 +162,28 @@ __global__ void k_col_len(const unsigned* ccnt, int64_t nc, int64_t* len, int* m
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(maxlen, mx);
 }
-// a group of L lanes per row (about the mean row length, a power of two)
+// a group of L lanes per row (about the mean row length, a power of two); rows far longer than that are
+// set aside for the whole CTA
 __global__ void k_col_place(const int64_t* rptr, const int32_t* col, int64_t nr, const int64_t* cptr,
                             const unsigned* slot, unsigned long long* word, int L) {
+    __shared__ LongRows s_long;
     const int sub = threadIdx.x & (L - 1);
     const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L;
     const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) / L;
-    for (int64_t r = grp; r < nr; r += ngrp) {
-        const int64_t e0 = rptr[r], e1 = rptr[r + 1];
+    s_long.init();
+    for (int64_t r0 = 0; r0 < nr; r0 += ngrp) {   // the same trip count for every group of a warp
+        const int64_t r = r0 + grp;
+        const int64_t e0 = r < nr ? rptr[r] : 0, e1 = r < nr ? rptr[r + 1] : 0;
+        if (s_long.put(sub == 0 && e1 - e0 > LONG_ROW && e1 - e0 > 64 * L, r, L)) continue;
         for (int64_t e = e0 + sub; e < e1; e += L)
             word[cptr[col[e]] + slot[e]] = ((unsigned long long)r << 32) | (unsigned long long)(e - e0);
     }
+    s_long.each([&](int64_t r) {
+        const int64_t e0 = rptr[r], e1 = rptr[r + 1];
+#pragma unroll 4
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x)
+            word[cptr[col[e]] + slot[e]] = ((unsigned long long)r << 32) | (unsigned long long)(e - e0);
+    });
 }
 constexpr int SPG_CAP = 8192;   // candidate products of one output row
 

@@ -24,7 +24,7 @@ __device__ __forceinline__ double widen(float f) {
     return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
 }
 
-template <int DT> struct Val;
+template <int DT> struct Val;   // load() widens by integer operations
 template <> struct Val<LSQ_F64> {
     typedef double T;
     static __device__ __forceinline__ double load(const void* p, int64_t e) {
@@ -49,5 +49,19 @@ template <> struct Val<LSQ_F32X2> {
         return __dadd_rn((double)f[2 * e], (double)f[2 * e + 1]);
     }
 };
+
+// an FP32 or BF16 value as FP32
+template <int DT>
+__device__ __forceinline__ float load_f32(const void* p, int64_t e) {
+    if constexpr (DT == LSQ_BF16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[e]);
+    else return reinterpret_cast<const float*>(p)[e];
+}
+// a value as FP64 by the hardware's conversion, for a pass that waits on memory and has FP64 slots
+// to spare (CSR, one column: 0.162 ms per column pass of 3.2e7 entries, 0.190 ms with integer widening)
+template <int DT>
+__device__ __forceinline__ double load_f64(const void* p, int64_t e) {
+    if constexpr (DT == LSQ_F32 || DT == LSQ_BF16) return (double)load_f32<DT>(p, e);
+    else return Val<DT>::load(p, e);
+}
 
 }  // namespace lsq

@@ -1,6 +1,6 @@
-"""CSR matrices of mostly short rows with a few long ones, which a warp takes together: lengths at the
-edges of what a row's own lanes take (32 entries a lane, 256 in the adjoint), several long rows in one
-warp, the last row long."""
+"""CSR matrices of mostly short rows with a few long ones, which a whole CTA takes together: lengths at
+the edge of what counts as long (1024 entries), several long rows in one warp, the last row long, and
+whole warps of long rows."""
 import numpy as np
 import pytest
 import torch
@@ -11,14 +11,16 @@ from helpers import to_device
 pytestmark = pytest.mark.gpu
 
 
-def _matrix(mean, seed):
+def _matrix(mean, seed, many=False):
     """4000 rows, most of 1 to 2 `mean` entries; the long ones small, so that few of them are drawn."""
     rng = np.random.default_rng(seed)
-    m, n = 4000, 700
+    m, n = 4000, 1500
     lens = rng.integers(1, 2 * mean + 1, m)
-    long = [1, 2, 3, 500, 501, 1500, 1501, 2600, 2601, m - 1]
-    lens[long] = [32 * mean, 32 * mean + 1, 63, 64, 65, 255, 256, 257, 699, 700]
-    lens = np.minimum(lens, n)
+    long = np.array([1, 2, 3, 500, 501, 1500, 1501, 2600, 2601, m - 1])
+    lens[long] = [1023, 1024, 1025, 1500, 65, 1026, 1027, 1500, 257, 1500]
+    if many:
+        lens[700:1000] = 1025
+        long = np.concatenate([long, np.arange(700, 1000)])
     rp = np.concatenate([[0], np.cumsum(lens)])
     ci = np.concatenate([np.sort(rng.choice(n, size=k, replace=False)) for k in lens])
     base = np.arange(n)                                # every column in a row of its own
@@ -26,7 +28,7 @@ def _matrix(mean, seed):
     ci = np.concatenate([ci, base]).astype(np.int32)
     va = rng.standard_normal(rp[-1])
     for i in long:
-        va[rp[i]:rp[i + 1]] *= 1e-2
+        va[rp[i]:rp[i + 1]] *= 1e-6 if many else 1e-3
     return {"kind": "csr", "m": m + n, "n": n, "row_ptr": rp.astype(np.int64), "col_idx": ci, "vals": va}
 
 
@@ -41,11 +43,11 @@ def test_sampling_with_long_rows(lsq, orc, mean, dtype):
 
 
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
-@pytest.mark.parametrize("k", [1, 3, 8, 17])
-def test_solve_and_adjoint_with_long_rows(lsq, k, dtype):
-    """Products and gradients against FP64 formulas on the returned X and Lambda: 700 terms a sum, so
+@pytest.mark.parametrize("k,many", [(1, False), (3, False), (8, False), (17, False), (2, True)])
+def test_solve_and_adjoint_with_long_rows(lsq, k, many, dtype):
+    """Products and gradients against FP64 formulas on the returned X and Lambda: 1500 terms a sum, so
     1e-12 of the largest entry; the solution against the normal equations (the transposed pattern)."""
-    mat = _matrix(2, 9)
+    mat = _matrix(2, 9, many)
     Mx, keep, seen = to_device(lsq, mat, dtype, with_f64=dtype == "f32")
     o = lsq.opts(seed=2, sample_factor=0.5)
     idx, p, d = lsq.lsq_sample_rows(Mx, o)
