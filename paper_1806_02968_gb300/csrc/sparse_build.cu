@@ -481,7 +481,8 @@ template <bool FILL>
 __global__ void __launch_bounds__(32) k_spgemm_long(SpgArgs a) {
     extern __shared__ __align__(16) unsigned char spg_smem[];
     const int lane = threadIdx.x;
-    const int words = (a.win + 31) >> 5, per = (words + 31) >> 5;
+    // words of the bitmap a lane walks: an odd number, so that the lanes' words lie in distinct banks
+    const int words = (a.win + 31) >> 5, per = ((words + 31) >> 5) | 1;
     double* acc = reinterpret_cast<double*>(spg_smem);                       // acap sums (pass 1)
     int32_t* ocol = reinterpret_cast<int32_t*>(acc + (FILL ? a.acap : 0));   // their columns
     unsigned* bits = reinterpret_cast<unsigned*>(ocol + (FILL ? a.acap : 0));
