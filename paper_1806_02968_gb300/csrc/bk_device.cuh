@@ -166,12 +166,15 @@ __device__ __forceinline__ void bk_rows_body(BkArgs a, int mode, int use_res, co
     if ((int)threadIdx.x < a.K) a.S->pw[threadIdx.x] = sh[threadIdx.x];
 }
 
-// out_j = (1/d_j) A^T_j q for every column (the transposed pattern; no atomics); entries are
-// loaded 8 at a time before their gathers, and 8 gathers are in flight.  Bound as the row pass.
-// 1e6 x 10,000, 16 columns, FP32 values: 0.30 ms, against 0.63 ms.
-template <int DT>
-__device__ __forceinline__ void bk_cols_body(BkArgs a, int use_res, double* out) {
-    const void* vals = use_res ? a.valsT_res : a.valsT;
+// out_j = (1/d_j) A^T_j q for every column (the transposed pattern; no atomics); U entries are loaded
+// before their gathers, and U gathers are in flight.  From 16 lanes a column on the pass is bound by FP64
+// operations, as the row pass, and takes eight entries with values widened by integer operations
+// (1e6 x 10,000, 16 columns, FP32 values: 0.30 ms, against 0.63 ms with four and hardware
+// conversions).  With fewer columns there are few lanes and the pass waits on memory: four entries and
+// the hardware's conversion are the faster form (1e6 x 10,000, 2 columns: 132 us against 221 us for FP32
+// values, 134 against 153 us for FP64; 4 columns: 132 against 182 and 117 against 135 us).
+template <int DT, int U, bool HW>
+__device__ __forceinline__ void bk_cols_walk(const BkArgs& a, const void* vals, double* out) {
     const int c = threadIdx.x & (a.GK - 1);
     const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / a.GK;
     const int64_t ngrp = ((int64_t)gridDim.x * blockDim.x) / a.GK;
@@ -180,21 +183,32 @@ __device__ __forceinline__ void bk_cols_body(BkArgs a, int use_res, double* out)
     for (int64_t j = grp; j < a.n; j += ngrp) {
         double t = 0.0;
         const int64_t eend = a.atptr[j + 1];
-        for (int64_t e = a.atptr[j]; e < eend; e += 8) {
-            int32_t row[8];
-            double v[8], qv[8];
+        for (int64_t e = a.atptr[j]; e < eend; e += U) {
+            int32_t row[U];
+            double v[U], qv[U];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) row[u] = e + u < eend ? a.atrow[e + u] : -1;
+            for (int u = 0; u < U; ++u) {
+                row[u] = -1;
+                v[u] = 0.0;
+                if (e + u < eend) {
+                    row[u] = a.atrow[e + u];
+                    v[u] = HW ? load_f64<DT>(vals, e + u) : Val<DT>::load(vals, e + u);
+                }
+            }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = e + u < eend ? Val<DT>::load(vals, e + u) : 0.0;
+            for (int u = 0; u < U; ++u) qv[u] = row[u] >= 0 ? a.q[(int64_t)row[u] * K + c] : 0.0;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) qv[u] = row[u] >= 0 ? a.q[(int64_t)row[u] * K + c] : 0.0;
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
+            for (int u = 0; u < U; ++u)
                 if (row[u] >= 0) t = fma(v[u], qv[u], t);
         }
         out[j * K + c] = t * a.inv_d[j];
     }
+}
+template <int DT>
+__device__ __forceinline__ void bk_cols_body(const BkArgs& a, int use_res, double* out) {
+    const void* vals = use_res ? a.valsT_res : a.valsT;
+    if (a.GK >= 16) bk_cols_walk<DT, 8, false>(a, vals, out);
+    else bk_cols_walk<DT, 4, true>(a, vals, out);
 }
 
 // alpha_c = rho_c / p_c^T w_c (0 for frozen columns), y += alpha p, g -= alpha w.  The last

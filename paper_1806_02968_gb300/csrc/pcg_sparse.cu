@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(SP_T) k_sp_rows(SpArgs a, int mode, int use_re
                     for (int u = 0; u < 4; ++u) {
                         const int64_t e = e0 + (int64_t)u * L;
                         const bool in = e < rp[4];
-                        av[u] = in ? (double)Val<DT>::load(vals, e) : 0.0;
+                        av[u] = in ? load_f64<DT>(vals, e) : 0.0;
                         cv[u] = in ? a.col_idx[e] : -1;
                     }
                     double xv[4];
