@@ -384,10 +384,11 @@ static lsq_status normal_matrix(const lsq_matrix* A, const int32_t* idx, const d
     const int64_t n = A->n;
     const int ntile = (int)((n + OZ_TILE - 1) / OZ_TILE), npad = ntile * OZ_TILE;
     const int tiles = ntile * (ntile + 1) / 2;
-    // draws per chunk: digits of at most 96 MB, which stay in L2 between the two kernels
+    // draws per chunk, the same number in each: digits of at most 112 MB, which stay in L2 between the kernels
     const int64_t srows = (s + OZ_FLUSH - 1) / OZ_FLUSH * OZ_FLUSH;
-    int64_t chunk = std::max<int64_t>(((int64_t)96 << 20) / (2 * OZ_PL * npad) / OZ_FLUSH * OZ_FLUSH, OZ_FLUSH);
-    chunk = std::min(chunk, srows);
+    const int64_t most = std::max<int64_t>(((int64_t)112 << 20) / (2 * OZ_PL * npad) / OZ_FLUSH, 1);
+    const int64_t chunks = (srows / OZ_FLUSH + most - 1) / most;
+    const int64_t chunk = (srows / OZ_FLUSH + chunks - 1) / chunks * OZ_FLUSH;
     // about one CTA per SM: each split takes at least 128 draws of a chunk
     int64_t splits = std::max<int64_t>(152 / tiles, 1);
     splits = std::min(splits, chunk / OZ_FLUSH);
