@@ -2,11 +2,13 @@
 // run to completion (including restarts from the true residual) inside ONE persistent
 // cooperative kernel.
 //
-// Several right-hand sides run side by side: the grid is cut into groups of G CTAs, each of
-// which solves one column at a time.  The columns are independent, so one group's barriers and
-// vector phases overlap the passes of the others, and groups that pass over the same rows
-// together share them in L2.  One column: one group of all CTAs.
-// Eight columns of 60,001 x 201 FP32 values (FP64 residuals): 3.2 ms, against 7.8 ms one column
+// Several right-hand sides of a matrix of about L2's size run side by side: the grid is cut into groups
+// of G CTAs, each of which solves one column at a time and takes the next one when it is done.  The
+// columns are independent, so one group's barriers and vector phases overlap the passes of the others, and
+// groups that pass over the same rows together share them in L2.  One column, or a larger matrix: one
+// group of all CTAs (launch_pcg_one has the rule).  A column's bits depend on G, so on the number of
+// columns in the call, not on which group takes it.
+// Eight columns of 60,001 x 201 FP32 values (FP64 residuals): 3.5 ms, against 7.8 ms one column
 // after the other.
 //
 // Work split (inside a group): CTA c owns the contiguous row block [c m/G, (c+1) m/G) of A for the fused
@@ -50,13 +52,15 @@ struct PcgArgs {
     int32_t* out_i;        // per column: iters, outer, converged, status
     double* out_d;         // per column: relres_rec, relres_true, relres_raw, unused
     unsigned max_polls = 1u << 26;   // bound of every grid-barrier wait
-    int G;                 // CTAs of a group: group q = CTAs [q G, (q + 1) G) solves columns q, q + NG, ...
-    int NG;                // groups
+    int G;                 // CTAs of a group: group q = CTAs [q G, (q + 1) G) starts with column q
+    int NG;                // groups; with more columns each takes the next one when it is done
     // set by the kernel for its own CTA
     int bid;               // CTA inside its group
     double *y, *g, *z;     // the group's n-vectors
 };
-constexpr int PCG_BAR_STRIDE = 16;   // 64-bit words: one 128-byte line per group's barrier
+// 64-bit words: one 128-byte line per group for its barrier (word 0), its next column (1) and, in the
+// first group's, the number of columns taken from the queue (2)
+constexpr int PCG_BAR_STRIDE = 16;
 
 __device__ __forceinline__ int64_t imin64(int64_t x, int64_t y) { return x < y ? x : y; }
 
@@ -1201,9 +1205,7 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(const PcgArgs args) {
         }                                               \
     } while (0)
 
-    for (int64_t col = grp; col < a.ncol; col += a.NG) {
-    // every CTA of the group has read the last column's vectors and partial sums
-    if (col != grp) LSQ_BARRIER();
+    for (int64_t col = grp; col < a.ncol;) {
     a.b = args.b ? args.b + col * a.ldb : nullptr;
     a.h_in = args.h_in ? args.h_in + col * a.ldb : nullptr;
     int iters = 0, outer_used = 0, converged = 0, status = LSQ_ERR_NOT_CONVERGED;
@@ -1377,13 +1379,15 @@ __global__ void __launch_bounds__(512, 1) k_pcg_dense(const PcgArgs args) {
             od[0] = rec; od[1] = tru; od[2] = (hn == 0.0) ? 0.0 : raw;
         }
     }
+    if (a.ncol <= a.NG) break;
+    // The next column; every CTA of the group has read this one's vectors and partial sums.  All groups are
+    // the same size, so a column's result does not depend on which of them takes it.
+    if (a.bid == 0 && threadIdx.x == 0) a.bar[1] = a.NG + atomicAdd(args.bar + 2, 1ull);
+    LSQ_BARRIER();
+    col = (int64_t)ld_acquire_u64(a.bar + 1);
     }
 #undef LSQ_BARRIER
     (void)lane;
 }
-
-// Host launcher (defined per dtype in pcg_f64.cu / pcg_f32.cu)
-lsq_status launch_pcg_dense(int dt, int dtr, int opt_dtype, int64_t nmax, PcgArgs& args,
-                            int grid_cap, cudaStream_t st, int* grid_used);
 
 }  // namespace lsq
