@@ -336,6 +336,7 @@ __global__ void __launch_bounds__(SB_T, 1) k_sweep_blocked(SbArgs a) {
         }
         __syncthreads();   // s_s and s_x are reused by the next block
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");   // the last block's left-over entries
 }
 
 // ---------------------------------------------------------------------------------------
