@@ -48,3 +48,20 @@ def test_groups_take_the_next_column(lsq, slow):
     kappa = np.linalg.cond(seen["A"] / d.cpu().numpy())
     assert_solution(X[slow[0]].cpu().numpy(), np.linalg.lstsq(seen["A"], B[slow[0]].cpu().numpy(), rcond=None)[0], kappa,
                     "column %d" % slow[0])
+
+
+def test_barriers_of_the_groups_run_out_then_recover(lsq):
+    """With two polls a wait the barriers of several groups give up, the call reports the timeout, and the
+    next one gives the same bits as before."""
+    Mx, keep, seen, o, d, P = _handle(lsq, W.gaussian_dense(5000, 130, 7))
+    B = torch.randn(8, 5000, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    X, info = lsq.lsq_pcg_solve(Mx, P, B, o)
+    lsq.set_wait_limit(2)
+    try:
+        with pytest.raises(lsq.L.LsqError) as e:
+            lsq.lsq_pcg_solve(Mx, P, B, o)
+        assert e.value.code == 6
+    finally:
+        lsq.set_wait_limit(0)
+    X1, info = lsq.lsq_pcg_solve(Mx, P, B, o)
+    assert torch.equal(X1, X) and all(info.converged == 1)

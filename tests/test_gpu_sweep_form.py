@@ -125,3 +125,32 @@ def test_no_memory_for_the_inverses_leaves_the_row_forms(lsq):
     del fill
     assert not by_blocks(lambda: P.apply(r))
     assert float((P.apply(r) - E).norm() / E.norm()) <= 1e-10
+
+
+def test_blocked_waits_run_out_then_recover(lsq):
+    """With two polls a wait the blocked level chain and the blocked sweeps (one column, several) give
+    up, report the timeout and leave the handle usable."""
+    def limited(f):
+        lsq.set_wait_limit(2)
+        try:
+            with pytest.raises(lsq.L.LsqError) as e:
+                f()
+            assert e.value.code == 6
+        finally:
+            lsq.set_wait_limit(0)
+
+    kw = dict(layers=500, width=16, reach=2, coupling=0.1)     # 8000 rows, 32 dependencies: blocks for both
+    A, P = layered(lsq, **kw)
+    r = torch.randn(A.n, dtype=torch.float64, device="cuda")
+    B = torch.randn(4, A.m, dtype=torch.float64, device="cuda")
+    o = lsq.opts()
+    apply, solve = lambda: P.apply(r), lambda: lsq.lsq_pcg_solve(A, P, B, o)
+    assert by_blocks(apply) and by_blocks(solve)
+    assert any("k_levels_blocked" in x for x in kernels(lambda: layered(lsq, **kw)))
+    E, (X, info) = apply(), solve()
+    limited(lambda: layered(lsq, **kw))
+    limited(apply)
+    limited(solve)
+    assert torch.equal(apply(), E)
+    X1, info = solve()
+    assert torch.equal(X1, X) and all(info.converged == 1)
