@@ -212,16 +212,16 @@ __device__ __forceinline__ void bt_q_products(const float* At, int pitch, const 
         }
 }
 
-// Rows [r_lo, r_hi) of problem P, KC columns, arithmetic type T (float: inner iteration):
+// Rows [r_lo, r_hi) of problem P, KC columns, in FP32 (inner iteration):
 //   Q = A X
 //   Wp = A^T Q over these rows, qq_out[c] = sum of Q_ic^2 over these rows (c < k)
 // X (npad x KC, rows j >= n zero) is in shared memory.  Tiles of BR rows are streamed with
 // cp.async; the next tiles (BtRing) are in flight while the current one is used.
 // W step: a thread owns 4 consecutive j and CQ columns (RS threads split the rows
 // when there are fewer such units than threads) and accumulates over all tiles in registers.
-template <int KC, typename T>
+template <int KC>
 __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int k,
-                            float* As, const T* Xs, T* Qs, T* Wp, double* qq_out, double* red) {
+                            float* As, const float* Xs, float* Qs, float* Wp, double* qq_out, double* red) {
     constexpr int CQ = KC < 4 ? KC : 4;
     constexpr int CG = KC / CQ;
     const int tid = threadIdx.x;
@@ -233,11 +233,11 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
     const bool wact = tid < units * RS;
     const int unit = tid % units, rs = tid / units;
     const int jg = unit / CG, cgw = unit % CG;
-    T acc[4][CQ];
+    float acc[4][CQ];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int c = 0; c < CQ; ++c) acc[u][c] = T(0);
+        for (int c = 0; c < CQ; ++c) acc[u][c] = 0.f;
     // ||Q||^2 in double-float on the FP32 units (the FP64 pipe runs at 1/64 of their rate)
     f2 qq{0.f, 0.f};   // of this thread's tile row and column
     int spot[NPMAX / 4 * BR / BT];
@@ -255,13 +255,13 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
         const float* At = As + buf * BR * ring.pitch;
         buf = ring.next(buf);
         fill = ring.next(fill);
-        bt_q_products<KC, T>(At, ring.pitch, Xs, n, nch, reinterpret_cast<T*>(red));
+        bt_q_products<KC, float>(At, ring.pitch, Xs, n, nch, reinterpret_cast<float*>(red));
         __syncthreads();
         if (tid < BR * KC) {   // one tile row and column per thread
             const int64_t i = r_lo + (int64_t)t * BR + tid / KC;
-            T q = T(0);
+            float q = 0.f;
             if (i < r_hi && tid % KC < k) {
-                const T* part = reinterpret_cast<const T*>(red) + tid;
+                const float* part = reinterpret_cast<const float*>(red) + tid;
                 q = (part[0] + part[BR * KC]) + (part[2 * BR * KC] + part[3 * BR * KC]);
                 df_add_sq(qq, q);
             }
@@ -272,12 +272,12 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
             for (int r = rs; r < BR; r += RS) {
                 const float4 a4 = *reinterpret_cast<const float4*>(At + r * ring.pitch + 4 * jg);
                 const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-                T qv[CQ];
+                float qv[CQ];
                 bt_read(qv, Qs + r * KC + cgw * CQ);
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
-                    for (int c = 0; c < CQ; ++c) acc[u][c] = fma((T)av[u], qv[c], acc[u][c]);
+                    for (int c = 0; c < CQ; ++c) acc[u][c] = fmaf(av[u], qv[c], acc[u][c]);
             }
         }
     }
@@ -290,7 +290,7 @@ __device__ void bt_row_pass(const BatchProb& P, int64_t r_lo, int64_t r_hi, int 
 #pragma unroll
                 for (int c = 0; c < CQ; ++c) {
                     const int at = (4 * jg + u) * KC + cgw * CQ + c;
-                    Wp[at] = (gph == 0 ? T(0) : Wp[at]) + acc[u][c];
+                    Wp[at] = (gph == 0 ? 0.f : Wp[at]) + acc[u][c];
                 }
         }
         __syncthreads();
@@ -613,7 +613,7 @@ __device__ void bt_solve_problem(cg::cluster_group& cl, const BatchProb& P, int 
         next_p(true);
         while (true) {
             // q = Â p, w = Â^T q (this CTA's rows), p^T w = ||q||^2
-            bt_row_pass<KC, float>(P, r_lo, r_hi, k, As, Xf, Qf, Wf, S->qq, red);
+            bt_row_pass<KC>(P, r_lo, r_hi, k, As, Xf, Qf, Wf, S->qq, red);
             if (tid < KC) { S->slot[sl][0][tid] = S->qq[tid]; S->slot[sl][1][tid] = 0.0; }
             __syncthreads();
             cl.sync();
