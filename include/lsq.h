@@ -400,10 +400,11 @@ LSQ_API lsq_status lsq_set_wait_limit(int64_t max_polls);
 /* Form of the one-column sparse Gauss-Seidel sweeps (Alg. 3 on a CSR A_s^T A_s), a tuning and
  * test setting; forms 1 to 3 compute the same rows in the same level order with the same
  * per-row arithmetic:
- *   0  chosen from the level schedule's shape (the default): one CTA, the grid, or, where the
- *      schedule is deep and rows are long, blocks of consecutive rows with inverted diagonal
- *      blocks: the same sweep, rounded in another order.  Captured and persistent solves
- *      keep the row forms,
+ *   0  chosen by shape (the default): one CTA, the grid, or blocks of consecutive rows with
+ *      inverted diagonal blocks where those are expected to take less time (a schedule deep
+ *      against the number of blocks, few entries near the diagonal, not too many rows; decided
+ *      for each number of columns): the same sweep, rounded in another order.  Captured and
+ *      persistent solves keep the row forms,
  *   1  the grid: every row waits (bounded) for the values of its own dependencies,
  *   2  one CTA: levels meet at block barriers,
  *   3  one thread-block cluster of 8 CTAs: the sweep vector in the cluster's shared memory
