@@ -793,10 +793,8 @@ __device__ __forceinline__ bool row_pass_split(const PcgArgs& a, const void* val
 // rows, where pairs of rows with four chains each took 26), one chain per row.  The products of
 // four warps per scheduler hide the loads, so nothing is staged and no barrier stands inside the
 // pass.  Rows wider than 512 columns are split over two warps, which exchange their halves' dot
-// products.  R is what the registers hold beside the sums: 8 up to 64 columns, 4 up to 256, else 2.
-// (One step more spills and is slower: 90,000 x 300 170.3 us an iteration with 4 rows, 160.6 with 2;
-// 60,000 x 70 71.8 us with 8, 69.9 with 4, few iterations and their restart.)
-// 90,000 x 300: 130 us per PCG iteration, against 182 us by pairs of rows from the staging ring
+// products.  R is what the registers hold: 8 up to 128 columns, 4 up to 320, else 2.
+// 90,000 x 300: 137 us per PCG iteration, against 182 us by pairs of rows from the staging ring
 // (86 us of FMAs at the pipe's rate).
 template <int NCH, int R, int WPR>
 __device__ __noinline__ void row_pass_f64(int mode, const double* vals, int64_t ld, const double* b, int n, const double* s_v,
@@ -895,7 +893,7 @@ __device__ __noinline__ void row_pass_f64(int mode, const double* vals, int64_t 
         pw[j] = t0 + t1;
     }
 }
-// Rows a CTA needs for the register form: two rounds of all its groups or more; below, the ring's
+// Rows a CTA needs for the register form: two rounds of all its groups; below, the ring's
 // stages, which are fetched during the barriers before the pass, are the better start.
 __device__ __forceinline__ bool f64_direct(int n, int64_t rows) {
     if (n > 1024) return false;
@@ -911,11 +909,11 @@ __device__ __forceinline__ bool row_pass_direct(const PcgArgs& a, const void* va
     const int n = (int)a.n;
 #define LSQ_F64_PASS(NCH, R, WPR) row_pass_f64<NCH, R, WPR>(MODE, A, a.ld, a.b, n, s_v, red, s_scal, pw, r0, r1)
     if constexpr (NMAX == 128) {
-        if (n <= 64) LSQ_F64_PASS(1, 8, 1); else LSQ_F64_PASS(2, 4, 1);
+        if (n <= 64) LSQ_F64_PASS(1, 8, 1); else LSQ_F64_PASS(2, 8, 1);
     } else if constexpr (NMAX == 256) {
         if (n <= 192) LSQ_F64_PASS(3, 4, 1); else LSQ_F64_PASS(4, 4, 1);
     } else if constexpr (NMAX == 512) {
-        if (n <= 320) LSQ_F64_PASS(5, 2, 1);
+        if (n <= 320) LSQ_F64_PASS(5, 4, 1);
         else if (n <= 384) LSQ_F64_PASS(6, 2, 1);
         else if (n <= 448) LSQ_F64_PASS(7, 2, 1);
         else LSQ_F64_PASS(8, 2, 1);
