@@ -793,7 +793,10 @@ __device__ __forceinline__ bool row_pass_split(const PcgArgs& a, const void* val
 // rows, where pairs of rows with four chains each took 26), one chain per row.  The products of
 // four warps per scheduler hide the loads, so nothing is staged and no barrier stands inside the
 // pass.  Rows wider than 512 columns are split over two warps, which exchange their halves' dot
-// products.  R is what the registers hold: 8 up to 128 columns, 4 up to 320, else 2.
+// products.  R: 8 up to 128 columns, 4 up to 320, else 2.  That is one step more than the registers hold
+// at 65 to 128 and at 257 to 320 columns, where the pass spills 60 to 148 bytes; half as many rows are
+// faster there (90,000 x 300, a solve of 11 iterations and its restart: 170.3 us an iteration with 4
+// rows, 160.6 with 2; 60,000 x 70: 71.8 with 8, 69.9 with 4).
 // 90,000 x 300: 137 us per PCG iteration, against 182 us by pairs of rows from the staging ring
 // (86 us of FMAs at the pipe's rate).
 template <int NCH, int R, int WPR>
