@@ -15,8 +15,8 @@
 // stands out) would keep fewer bits than an FP64 product gives it, so every entry's error is
 // bounded beside the products, and the tiles with one that may pass 8 roundings of its terms are
 // summed in FP64 (k_wide_check, k_wide_tiles).
-// 12,777 draws of 512 columns: 0.37 ms, and 0.11 ms for the digits; s = 9,586, n = 400: 0.23 ms
-// and 0.07, against 2.1 ms.  Error of M against extended precision (Frobenius, relative; FP64
+// 12,777 draws of 512 columns: 0.40 ms (0.37 without the magnitudes), 0.12 ms for the digits and 0.02
+// for the bound; in FP64 4.0 ms.  Error of M against extended precision (Frobenius, relative; FP64
 // product in brackets): Gaussian 1.45e-16 (1.83e-16), 2 % heavy rows 1.44e-16 (1.88e-16), the same
 // under uniform draws 1.75e-16 (2.95e-16), UDV 1.49e-16 (1.93e-16), FP32 values 1.42e-16
 // (2.32e-16), semi-Gaussian 1.82e-16 (2.57e-16).

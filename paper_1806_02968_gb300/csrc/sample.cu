@@ -186,7 +186,7 @@ __global__ void k_colscale(int64_t n, int normalize, const int* E1j, const unsig
 // S2: w_i = sum_j floor(2^51 fl(fl(a_ij^2) inv_d2_j)), a group of L lanes per row (about the mean
 // row length, a power of two up to a warp), exact.  Bound: two FP64 multiplications per entry at
 // two lanes a clock and SM, so every lane of a warp should hold an entry (4e6 rows of 8 entries:
-// 0.21 ms with 8 lanes per row, 0.84 ms with a warp per row).  Rows far longer than their lanes are set
+// 0.23 ms with 8 lanes per row, 0.84 ms with a warp per row).  Rows far longer than their lanes are set
 // aside for the whole CTA (sampling of 1e6 rows of 2 entries and 20 of 50,000 side by side: 0.58 ms, 4.5 ms
 // with two lanes to every row).
 // ---------------------------------------------------------------------------------------
