@@ -2,7 +2,7 @@
 //
 // M = X^T X with x_tj = a_{i_t j} / d_j / sqrt(s p_t) is a contraction over the draws, and GB300
 // multiplies FP64 at two FMAs a clock and SM: 12,777 draws of 512 columns took 4.0 ms there. It
-// runs on the tensor cores instead, exactly, in the manner of Ozaki, Ogita, Oishi & Rump
+// runs on the tensor cores instead, in the manner of Ozaki, Ogita, Oishi & Rump
 // ("Error-free transformations of matrix multiplication by using fast routines of matrix
 // multiplication", Numer. Algorithms 59, 2012): every column is scaled by a power of two and
 // cut into seven signed 8-bit digits, x = 2^e sum_p q_p 2^(-7-8p), which BF16 holds exactly; the

@@ -609,14 +609,17 @@ static lsq_status resident_ctas(const void* kern, int threads, size_t smem, int*
 template <typename MT, typename AR, bool FWD>
 static const void* sb_kernel(int K, int* B, int* KC) {
     constexpr bool pair = std::is_same<AR, SbPair>::value;
-    if (K == 1) {
-        *KC = 1;
-        *B = pair ? 128 : 64;
-        if constexpr (pair) return (const void*)k_sweep_blocked<MT, AR, FWD, 128, 1>;
-        else return (const void*)k_sweep_blocked<MT, AR, FWD, 64, 1>;
+    // one column of FP32 M is always summed in double-float
+    if constexpr (pair || sizeof(MT) == 8) {
+        if (K == 1) {
+            *KC = 1;
+            *B = pair ? 128 : 64;
+            if constexpr (pair) return (const void*)k_sweep_blocked<MT, AR, FWD, 128, 1>;
+            else return (const void*)k_sweep_blocked<MT, AR, FWD, 64, 1>;
+        }
     }
     *B = 64;
-    if (K == 2) { *KC = 2; return (const void*)k_sweep_blocked<MT, AR, FWD, 64, 2>; }
+    if (K <= 2) { *KC = 2; return (const void*)k_sweep_blocked<MT, AR, FWD, 64, 2>; }
     *KC = 4;
     return (const void*)k_sweep_blocked<MT, AR, FWD, 64, 4>;
 }
